@@ -144,6 +144,10 @@ bool apply_box(Geom* g, const int b[3]) {
   if (tot * 128 >= (1LL << 31)) return false;
   g->nbmax_tot = (int32_t)tot;
   g->per_tile = g->nbmax_tot * 128;
+  for (int a = 0; a < 3; ++a) g->fb[a] = make_fastdiv((uint32_t)b[a]);
+  g->fnb = make_fastdiv((uint32_t)g->nbmax_tot);
+  g->fpairs = make_fastdiv((uint32_t)(g->nbmax_tot + 1) / 2);
+  g->fslots = make_fastdiv((uint32_t)g->per_tile);
   return true;
 }
 
@@ -194,6 +198,14 @@ bool make_geom(const gattn_desc* desc, Geom* g) {
   g->window = d.window;
   g->scale = d.scale > 0.f ? d.scale : 1.0f / sqrtf((float)d.d);
   g->scale_log2 = g->scale * 1.4426950408889634f;
+  for (int a = 0; a < 3; ++a) {
+    g->fc[a] = make_fastdiv((uint32_t)g->c[a]);
+    g->fG[a] = make_fastdiv((uint32_t)g->G[a]);
+  }
+  g->fN = make_fastdiv((uint32_t)N);
+  g->fn2 = make_fastdiv((uint32_t)g->n[2]);
+  g->fn12 = make_fastdiv((uint32_t)(g->n[1] * g->n[2]));
+  g->fntiles = make_fastdiv((uint32_t)g->ntiles);
   // a box shape whose per-tile slot count does not fit 32 bits is refused
   if (!choose_box(g)) return false;
   if (g->R < 1 || g->nbmax_tot < 1 || (int64_t)g->nbmax_tot * 128 >= (1LL << 31)) return false;

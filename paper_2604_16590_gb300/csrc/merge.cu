@@ -61,8 +61,9 @@ __global__ void __launch_bounds__(kThreads) merge_fwd_kernel(Geom g, const float
        idx += (int64_t)gridDim.x * kThreads) {
     const int f = (int)(idx % F4);
     const int64_t bi = idx / F4;
-    const int bh = (int)(bi / g.N);
-    const int64_t i = bi % g.N;
+    int bh;
+    int64_t i;
+    split_row(g, bi, bh, i);
     Cover c;
     if (!cover_of(g, i, c)) continue;  // single-cover: written by the tile kernel
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -116,7 +117,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     int n = 0;
     float wsum = 0.f;
     if (idx < total) {
-      n = token_covers(g, tbl, (int)(idx / g.N), idx % g.N, slot, w);
+      int bh;
+      int64_t i;
+      split_row(g, idx, bh, i);
+      n = token_covers(g, tbl, bh, i, slot, w);
       if (n > MAXC) {  // the host chose MAXC from the largest cover count
         set_status(kStatusBounds);
         n = 0;
@@ -208,7 +212,10 @@ __global__ void __launch_bounds__(kThreads, 2) merge_bwd_warp_kernel(Geom g, con
     float w[MAXC];
     int n = 0;
     if (idx < total) {
-      n = token_covers(g, tbl, (int)(idx / g.N), idx % g.N, slot, w);
+      int bh;
+      int64_t i;
+      split_row(g, idx, bh, i);
+      n = token_covers(g, tbl, bh, i, slot, w);
       if (n > MAXC) {  // the host chose MAXC from the largest cover count
         set_status(kStatusBounds);
         n = 0;
@@ -345,10 +352,11 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
   const WinTable tbl = build_win_table(g, win);
   const int64_t S = (int64_t)g.B * g.nh * g.ntiles * g.per_tile;
   for (int64_t slot = (int64_t)blockIdx.x * kThreads + threadIdx.x; slot < S; slot += (int64_t)gridDim.x * kThreads) {
-    const int64_t ut = slot / g.per_tile;
+    // ut = slot / per_tile < 65536^2 (batch*head, tile)
+    const int64_t ut = slot < (1LL << 31) ? fdiv((int)slot, g.fslots) : slot / g.per_tile;
     const int within = (int)(slot - ut * g.per_tile);
-    const int tile = (int)(ut % g.ntiles);
-    const int bh = (int)(ut / g.ntiles);
+    const int bh = ut < (1LL << 31) ? fdiv((int)ut, g.fntiles) : (int)(ut / g.ntiles);
+    const int tile = (int)(ut - (int64_t)bh * g.ntiles);
     TileBox tb;
     tile_box(g, tile, tb);
     int lr[3];
@@ -361,9 +369,8 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
       continue;
     }
     const int64_t tok = grid_token(g, tb, lr);
-    int p[3];
-    token_pos(g, tok, p);
-    const bool single = single_cover(g, p);
+    const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
+    const bool single = only_cover(g, tb, p);
     const InT* a = dout + ((int64_t)bh * g.N + tok) * g.d;
     float part = 0.f;
     if (single) {
@@ -390,11 +397,7 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
       // c = w_t / sum over covering tiles of w
       Cover c;
       cover_of(g, tok, c);
-      int kt[3];
-      kt[0] = tile / (g.n[1] * g.n[2]);
-      kt[1] = (tile / g.n[2]) % g.n[1];
-      kt[2] = tile % g.n[2];
-      float wt = table_weight(g, tbl, p, kt), ws = 0.f;
+      float wt = table_weight(g, tbl, p, tb.k), ws = 0.f;
       int k[3];
       for (k[0] = c.k0[0]; k[0] <= c.k1[0]; ++k[0])
         for (k[1] = c.k0[1]; k[1] <= c.k1[1]; ++k[1])
@@ -420,8 +423,9 @@ __global__ void __launch_bounds__(kThreads) merge_bwd_kernel(Geom g, const float
        idx += (int64_t)gridDim.x * kThreads) {
     const int f = (int)(idx % F4);
     const int64_t bi = idx / F4;
-    const int bh = (int)(bi / g.N);
-    const int64_t i = bi % g.N;
+    int bh;
+    int64_t i;
+    split_row(g, bi, bh, i);
     Cover c;
     if (!cover_of(g, i, c)) continue;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, e = a;

@@ -61,8 +61,9 @@ __global__ void __launch_bounds__(kThreads) serve_update_kernel(const ReqDesc* _
       set_status(kStatusBounds);
       continue;
     }
-    const int h = (int)(local / g.N);
-    const int64_t i = local % g.N;
+    int h;
+    int64_t i;
+    split_row(g, local, h, i);
     int p[3], k0[3], k1[3];
     token_pos(g, i, p);
     bool multi = false;
@@ -164,7 +165,10 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int a = 0; a < 3; ++a) same = same && g.c[a] == g0.c[a] && g.h[a] == g0.h[a] && g.tiled[a] == g0.tiled[a];
         WinTable t = tbl;
         t.direct = t.direct || !same;
-        n = token_covers(g, t, (int)(local / g.N), local % g.N, slot, w);
+        int h;
+        int64_t i;
+        split_row(g, local, h, i);
+        n = token_covers(g, t, h, i, slot, w);
         if (n > MAXC) {  // the host chose MAXC from the largest cover count
           set_status(kStatusBounds);
           r = -1;

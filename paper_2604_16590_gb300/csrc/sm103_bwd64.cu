@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kThreads64, 1)
       const bool kvalid = inside(tbk, kl);
       const int p[3] = {tbk.tb.lo[0] + kl[0], tbk.tb.lo[1] + kl[1], tbk.tb.lo[2] + kl[2]};
       const int64_t tok = kvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = kvalid && single_cover(g, p);
+      const bool single = kvalid && only_cover(g, tbk.tb, p);
       const int64_t slot = tile_slot0(g, bh, tile) + kb * 128 + row;
       const int c0 = c4 * 16;
       // both accumulators into registers, then they are released at once: the
@@ -516,10 +516,10 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
         }
       }
       if (!(ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0)) break;
-      for (int j = 0; j < tbk.NB; ++j, ++G) {
+      BlockWalk bw;
+      for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
         const uint32_t st = G % C::kStages, n = G / C::kStages;
-        int ko[3];
-        block_origin(g, tbk, j, ko);
+        const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
         // the stage (K, V and its bias row) is free once box G - kStages is done
         if (lane == 0) ok = WAIT(kv_empty + st, (n & 1) ^ 1);
         if (!(ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0)) break;
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
       const bool qvalid = inside(tbk, ql);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
       const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = qvalid && single_cover(g, p);
+      const bool single = qvalid && only_cover(g, tbk.tb, p);
       const int c0 = c4 * 16;
       uint32_t rq[16];
       tmem_ld16(tl + C::kColDQ + c0, rq);

@@ -24,10 +24,10 @@ struct BwdArgs {
 };
 
 __device__ __forceinline__ void decode_item(const Geom& g, int w, int& bh, int& tile, int& blk) {
-  blk = w % g.nbmax_tot;
-  const int r = w / g.nbmax_tot;
-  tile = r % g.ntiles;
-  bh = r / g.ntiles;
+  const int r = fdiv(w, g.fnb);
+  blk = w - r * g.nbmax_tot;
+  bh = fdiv(r, g.fntiles);
+  tile = r - bh * g.ntiles;
 }
 
 // byte offset of K-step ks (16 elements) in a 128-byte-swizzled K-major operand

@@ -27,18 +27,16 @@ struct TileBlocks {
 
 __device__ __forceinline__ void tile_blocks(const Geom& g, int tile, TileBlocks& t) {
   tile_box(g, tile, t.tb);
-  t.nb[0] = (t.tb.e[0] + g.bt - 1) / g.bt;
-  t.nb[1] = (t.tb.e[1] + g.by - 1) / g.by;
-  t.nb[2] = (t.tb.e[2] + g.bx - 1) / g.bx;
+  t.nb[0] = fdiv(t.tb.e[0] + g.bt - 1, g.fb[0]);
+  t.nb[1] = fdiv(t.tb.e[1] + g.by - 1, g.fb[1]);
+  t.nb[2] = fdiv(t.tb.e[2] + g.bx - 1, g.fb[2]);
   t.NB = t.nb[0] * t.nb[1] * t.nb[2];
 }
 
 // tile-local origin of block j
 __device__ __forceinline__ void block_origin(const Geom& g, const TileBlocks& t, int j, int o[3]) {
-  const int jx = j % t.nb[2];
-  const int jr = j / t.nb[2];
-  const int jy = jr % t.nb[1];
-  const int jt = jr / t.nb[1];
+  int jt, jy, jx;
+  box_index(j, t.nb[1], t.nb[2], jt, jy, jx);
   o[0] = jt * g.bt;
   o[1] = jy * g.by;
   o[2] = jx * g.bx;
@@ -62,7 +60,7 @@ __device__ __forceinline__ void block_row(const Geom& g, const int o[3], int rho
 
 // every block of the tile holds 128 rows of the tile (no padding anywhere)
 __device__ __forceinline__ bool tile_all_full(const Geom& g, const TileBlocks& t) {
-  return g.R == 128 && t.tb.e[0] % g.bt == 0 && t.tb.e[1] % g.by == 0 && t.tb.e[2] % g.bx == 0;
+  return g.R == 128 && t.nb[0] * g.bt == t.tb.e[0] && t.nb[1] * g.by == t.tb.e[1] && t.nb[2] * g.bx == t.tb.e[2];
 }
 
 // Walks the blocks of a tile in index order with counters instead of

@@ -130,10 +130,10 @@ __device__ __forceinline__ bool resolve(const FwdArgs& a, const CUtensorMap* tq,
     it.ot = a.ot;
   }
   const Geom& g = *it.g;
-  it.blk = w % g.nbmax_tot;
-  const int r = w / g.nbmax_tot;
-  it.tile = r % g.ntiles;
-  it.bh = r / g.ntiles;
+  const int r = fdiv(w, g.fnb);
+  it.blk = w - r * g.nbmax_tot;
+  it.bh = fdiv(r, g.fntiles);
+  it.tile = r - it.bh * g.ntiles;
   it.req = req;
   if (RAGGED && (it.bh >= g.B * g.nh || g.R != a.pad_R)) {
     set_status(kStatusBounds);
@@ -425,10 +425,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int h = 0; h < C::kHalves; ++h)
           tma_load_5d(smem + C::kQ + h * 16384, it.tq, q_full, 64 * h, tbk.tb.lo[2] + o[2], tbk.tb.lo[1] + o[1],
                       tbk.tb.lo[0] + o[0], bh);
-        for (int j = 0; j < tbk.NB; ++j, ++G) {
+        BlockWalk bw;
+        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
           const uint32_t st = G % C::kStages, n = G / C::kStages;
-          block_origin(g, tbk, j, o);
-          const int c1 = tbk.tb.lo[2] + o[2], c2 = tbk.tb.lo[1] + o[1], c3 = tbk.tb.lo[0] + o[0];
+          const int c1 = tbk.tb.lo[2] + bw.jx * g.bx, c2 = tbk.tb.lo[1] + bw.jy * g.by,
+                    c3 = tbk.tb.lo[0] + bw.jt * g.bt;
           if (!(ok = mbar_wait<set_status_fwd>(k_empty + st, (n & 1) ^ 1, abort_flag))) break;
           mbar_arrive_expect_tx(k_full + st, C::kHalves * g.R * 128);
           k_arm |= 1u << st;
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (qvalid && ch == 0 && it.lse2) it.lse2[slot] = rs.m + __log2f(l);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
       const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = qvalid && single_cover(g, p);
+      const bool single = qvalid && only_cover(g, tbk.tb, p);
       const int c0 = ch * (D / 2);
       OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * D + c0;
       float* dst_scr = it.ot + slot * D + c0;

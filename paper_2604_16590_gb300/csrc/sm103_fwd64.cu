@@ -116,7 +116,7 @@ struct Item {
   int req;  // request index (ragged mode), else -1
 };
 
-__host__ __device__ __forceinline__ int box_pairs(const Geom& g) { return (g.nbmax_tot + 1) / 2; }
+inline int box_pairs(const Geom& g) { return (int)g.fpairs.d; }
 
 // Returns false (after recording GATTN_ERR_DEVICE_BOUNDS) if a ragged work item
 // does not decode to a valid (request, head, tile, pair); every role decodes
@@ -156,11 +156,10 @@ __device__ __forceinline__ bool resolve(const Fwd64Args& a, const CUtensorMap* t
     it.ot = a.ot;
   }
   const Geom& g = *it.g;
-  const int np = box_pairs(g);
-  it.pair = w % np;
-  const int r = w / np;
-  it.tile = r % g.ntiles;
-  it.bh = r / g.ntiles;
+  const int r = fdiv(w, g.fpairs);
+  it.pair = w - r * (int)g.fpairs.d;
+  it.bh = fdiv(r, g.fntiles);
+  it.tile = r - it.bh * g.ntiles;
   it.req = req;
   if (RAGGED && (it.bh >= g.B * g.nh || g.d != kD || g.R != a.pad_R)) {
     set_status(kStatusBounds);
@@ -464,10 +463,10 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         TileBlocks tbk;
         tile_blocks(g, it.tile, tbk);
         if (2 * it.pair >= tbk.NB) continue;
-        for (int j = 0; j < tbk.NB; ++j, ++G) {
+        BlockWalk bw;
+        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
           const uint32_t st = G % kStages, n = G / kStages;
-          int ko[3];
-          block_origin(g, tbk, j, ko);
+          const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
           if (lane == 0) ok = WAIT(k_empty + st, (n & 1) ^ 1);
           ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
           if (!ok) break;
@@ -598,7 +597,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       if (qvalid && it.lse2) it.lse2[slot] = m + __log2f(l);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
       const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = qvalid && single_cover(g, p);
+      const bool single = qvalid && only_cover(g, tbk.tb, p);
       OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * kD;
       float* dst_scr = it.ot + slot * kD;
       // the whole O row into registers, then O_x is released at once: the next
