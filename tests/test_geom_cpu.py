@@ -87,18 +87,30 @@ static int covers(int G, int c, int h) {
       tile_box(g, k, tb);
       CHECK(only_cover(g, tb, pos) == (first == last), "only_cover G %d c %d h %d p %d\n", G, c, h, p);
     }
-    for (int64_t bh : {(int64_t)0, (int64_t)3, (int64_t)(1LL << 31) / G + 5}) {
-      int b;
-      int64_t i;
-      split_row(g, bh * G + p, b, i);
-      CHECK(b == bh && i == p, "split_row\n");
-    }
+  }
+  return 0;
+}
+
+static int rows() {  // batch*head and token of a row index, on both sides of 2^31
+  const int64_t Ns[] = {1, 7, 262144, 1000003, (1LL << 31) - 1};
+  for (int64_t N : Ns) {
+    Geom g;
+    memset(&g, 0, sizeof(g));
+    g.N = N;
+    g.fN = make_fastdiv((uint32_t)N);
+    for (int64_t bh : {0, 1, 3, 2147, 2148, 65534})
+      for (int64_t i : {(int64_t)0, N / 2, N - 1}) {
+        int b;
+        int64_t k;
+        split_row(g, bh * N + i, b, k);
+        CHECK(b == bh && k == i, "split_row N %lld bh %lld\n", (long long)N, (long long)bh);
+      }
   }
   return 0;
 }
 
 int main() {
-  if (fastdiv() || quotients()) return 1;
+  if (fastdiv() || quotients() || rows()) return 1;
   for (int G = 1; G <= 40; ++G)
     for (int c = 1; c <= 12; ++c)
       for (int h = 0; h <= 14; ++h)
