@@ -69,19 +69,6 @@ __device__ __forceinline__ uint4 phi_chunk(uint4 u, bool valid, float (&f)[8]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// 5-D tiled store shared -> global (bulk group); rows past the tensor's end are
-// not written.
-__device__ __forceinline__ void tma_store_5d(const CUtensorMap* m, const void* src, int c0, int c1, int c2, int c3,
-                                             int c4) {
-  asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(m)),
-               "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // byte offset of 16-byte chunk c of row r in a 128-byte-swizzled tile
 __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
 
@@ -407,7 +394,7 @@ __global__ void __launch_bounds__(kThreadsQ, 3) la_query_kernel(const __grid_con
       for (int t = t0, G = 0; t < t1; ++t, ++G) {
         if (!(ok = LWAIT(staged, G & 1))) break;
         fence_proxy_async_smem();
-        tma_store_5d(&to, ost, 0, t * kTile, 0, 0, bh);
+        tma_store_5d(&to, smem_u32(ost), 0, t * kTile, 0, 0, bh);
         bulk_commit();
         bulk_wait_read();  // the staging tile may be rewritten once the store has read it
         mbar_arrive(sfree);

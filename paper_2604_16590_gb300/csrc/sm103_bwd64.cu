@@ -78,13 +78,14 @@ constexpr int kThreadsQ64 = kThreadsB + 32;
 
 // =============================================================== dK / dV
 struct Kv64 {
-  static constexpr int kStages = 4;  // (Q, dOut, statistics rows) ring
+  static constexpr int kStages = 3;  // (Q, dOut, statistics rows) ring
   // two (K, V) buffers, items alternate: buffer b holds K at kK + 2 b kBox, V after it
   static constexpr int kK = 0;
   static constexpr int kQ = 4 * kBox;  // stage s: Q at kQ + s*2*kBox, dOut after it
   // Extension operands, K-major without swizzle: 128 rows x 16 B (K-columns
   // 0..7) followed by 2 KB of zeros (K-columns 8..15, lbo = 2048).
-  static constexpr int kOnes = kQ + kStages * 2 * kBox;  // A: ones in K 0..2 at kOnes, ones in K 3..5 at kOnes+4096
+  static constexpr int kOut = kQ + kStages * 2 * kBox;  // staged dV slots, 4 KB per warp of column groups 2, 3
+  static constexpr int kOnes = kOut + 2 * kBox;  // A: ones in K 0..2 at kOnes, ones in K 3..5 at kOnes+4096
   static constexpr int kExt = kOnes + 2 * 4096;            // B, stage s at kExt + s*4096: the 128 statistics rows
   static constexpr int kBar = kExt + kStages * 4096;
   // kv_full[2], kv_empty[2], qd_full[S], qd_empty[S], s_full[2], s_empty[2], p_full[2], p_empty[2],
@@ -100,6 +101,7 @@ template <typename OutT>
 __global__ void __launch_bounds__(kThreads64, 1)
     dkdv64_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
                   const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tdo,
+                  const __grid_constant__ CUtensorMap tdk, const __grid_constant__ CUtensorMap tdv,
                   const BwdArgs a) {
   using C = Kv64;
   extern __shared__ uint8_t smem_raw[];
@@ -141,7 +143,7 @@ __global__ void __launch_bounds__(kThreads64, 1)
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(kv_full + b, 1);
-      mbar_init(kv_empty + b, 1);
+      mbar_init(kv_empty + b, 1 + kMath64 / 2);  // the last score product; the warps that staged dK there
     }
     for (int s = 0; s < C::kStages; ++s) {
       mbar_init(qd_full + s, 1);
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(kThreads64, 1)
     prefetch_tmap(&tk);
     prefetch_tmap(&tv);
     prefetch_tmap(&tdo);
+    prefetch_tmap(&tdk);
+    prefetch_tmap(&tdv);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, 512);
@@ -326,6 +330,19 @@ __global__ void __launch_bounds__(kThreads64, 1)
     const uint64_t s2 = f2pack(g.scale_log2, g.scale_log2);
     uint32_t G = 0, W = 0;
     bool ok = true;
+    // Epilogue: column groups 0, 1 write dK columns [32 c4, 32 c4 + 32), staged
+    // over the item's own K (c4 = 0) and V (c4 = 1) blocks, which the score
+    // products are done with; groups 2, 3 write dV columns [32 (c4 - 2), ...)
+    // through blocks of their own.
+    const bool has_dk = c4 < 2;
+    // the stores of item W - 1 have read this warp's staging block: its K, V
+    // buffer may be refilled
+    auto release_staged = [&]() {
+      if (W > 0 && lane == 0) {
+        bulk_wait_read();
+        if (has_dk) mbar_arrive(kv_empty + ((W - 1) & 1));
+      }
+    };
     for (int w = blockIdx.x; w < a.items && ok; w += gridDim.x) {
       int bh, tile, kb;
       decode_item(g, w, bh, tile, kb);
@@ -359,11 +376,21 @@ __global__ void __launch_bounds__(kThreads64, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(p_full + (c4 >> 1));
+        if (i == 0) release_staged();
       }
       if (!ok) break;
-      // ---- epilogue: this thread's key row of dK, dV (columns [16 c4, 16 c4 + 16))
+      // ---- epilogue: this thread's key row, 32 columns of dK or of dV
       if (!(ok = WAIT(acc_full, W & 1))) break;
       tc_fence_after();
+      // the accumulator columns into registers, then they are released at once:
+      // the next item's first gradient products may overwrite them during the stores
+      uint32_t r[32];
+      const int c0 = (c4 & 1) * 32;
+      tmem_ld32(tl + (has_dk ? C::kColDK : C::kColDV) + c0, r);
+      tmem_wait_ld(r);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty);
       int ko[3], kl[3];
       block_origin(g, tbk, kb, ko);
       block_row(g, ko, row, kl);
@@ -371,24 +398,16 @@ __global__ void __launch_bounds__(kThreads64, 1)
       const int p[3] = {tbk.tb.lo[0] + kl[0], tbk.tb.lo[1] + kl[1], tbk.tb.lo[2] + kl[2]};
       const int64_t tok = kvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const bool single = kvalid && only_cover(g, tbk.tb, p);
-      const int64_t slot = tile_slot0(g, bh, tile) + kb * 128 + row;
-      const int c0 = c4 * 16;
-      // both accumulators into registers, then they are released at once: the
-      // next item's first gradient products may overwrite them during the stores
-      uint32_t rk[16], rv[16];
-      tmem_ld16(tl + C::kColDK + c0, rk);
-      tmem_ld16(tl + C::kColDV + c0, rv);
-      tmem_wait_ld(rk);
-      tmem_wait_ld(rv);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty);
-      row_store<16, OutT>(rk, g.scale, kvalid, single, static_cast<OutT*>(a.dk) + ((int64_t)bh * g.N + tok) * kD + c0,
-                        a.dk_s + slot * kD + c0);
-      row_store<16, OutT>(rv, 1.f, kvalid, single, static_cast<OutT*>(a.dv) + ((int64_t)bh * g.N + tok) * kD + c0,
-                        a.dv_s + slot * kD + c0);
+      const int srow = (int)(tile_slot0(g, bh, tile) + kb * 128 + quad * 32);
+      row_out<32, OutT>(r, has_dk ? g.scale : 1.f, kvalid, single, row < g.R,
+                        static_cast<OutT*>(has_dk ? a.dk : a.dv) + ((int64_t)bh * g.N + tok) * kD + c0,
+                        has_dk ? &tdk : &tdv,
+                        smem_u32(smem + (has_dk ? C::kK + (W & 1) * 2 * kBox : C::kOut)) + (c4 & 1) * kBox + quad * 4096,
+                        lane, c0, srow);
       ++W;
     }
+    release_staged();
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -407,7 +426,8 @@ struct Q64 {
   // Key-mask extension operands (as in the forward): A = 1 in K-column 0 of
   // 128 rows, and per stage the key block's bias row (0, or -1e30 for a
   // padding key or a key outside the tile), each followed by 2 KB of zeros.
-  static constexpr int kOnes = kK + kStages * 2 * kBox;
+  static constexpr int kOut = kK + kStages * 2 * kBox;  // staged dQ slots, 32 rows x 64 bytes per math warp
+  static constexpr int kOnes = kOut + 2 * kBox;
   static constexpr int kBias = kOnes + 4096;
   static constexpr int kBar = kBias + kStages * 4096;
   // qd_full, qd_empty, qt_full, kv_full[S], kv_empty[S], s_full[2], s_empty[2], p_full[2], p_empty[2],
@@ -423,7 +443,8 @@ struct Q64 {
 template <typename OutT>
 __global__ void __launch_bounds__(kThreadsQ64, 1)
     dq64_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
-                const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tdo, const BwdArgs a) {
+                const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap tdo,
+                const __grid_constant__ CUtensorMap tdq, const BwdArgs a) {
   using C = Q64;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -478,6 +499,7 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
     prefetch_tmap(&tk);
     prefetch_tmap(&tv);
     prefetch_tmap(&tdo);
+    prefetch_tmap(&tdq);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, 512);
@@ -723,6 +745,17 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
       if (!ok) break;
       if (!(ok = WAIT(acc_full, W & 1))) break;
       tc_fence_after();
+      const int c0 = c4 * 16;
+      uint32_t rq[16];
+      tmem_ld16(tl + C::kColDQ + c0, rq);
+      tmem_wait_ld(rq);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(acc_empty);  // released before the stores
+        bulk_wait_read();        // the previous item's store has read this warp's staging block
+      }
+      __syncwarp();
       int qo[3], ql[3];
       block_origin(g, tbk, qb, qo);
       block_row(g, qo, row, ql);
@@ -730,17 +763,11 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
       const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const bool single = qvalid && only_cover(g, tbk.tb, p);
-      const int c0 = c4 * 16;
-      uint32_t rq[16];
-      tmem_ld16(tl + C::kColDQ + c0, rq);
-      tmem_wait_ld(rq);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty);  // released before the stores
-      row_store<16, OutT>(rq, g.scale, qvalid, single, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
-                        a.dq_s + qslot * kD + c0);
+      row_out<16, OutT>(rq, g.scale, qvalid, single, true, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
+                        &tdq, smem_u32(smem + C::kOut) + (warp - kMath0) * 2048, lane, c0, (int)(qslot - lane));
       ++W;
     }
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -770,25 +797,28 @@ cudaError_t run_bwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16
   if (items >= (1LL << 31)) return cudaErrorNotSupported;
   a.items = (int)items;
   const int BH = g.B * g.nh;
-  CUtensorMap mq, mk, mv, mdo;
+  const int64_t slots = (int64_t)BH * g.ntiles * g.per_tile;
+  CUtensorMap mq, mk, mv, mdo, mdq, mdk, mdv;
   if (!make_tmap_5d(&mq, q, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
       !make_tmap_5d(&mk, k, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
       !make_tmap_5d(&mv, v, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
-      !make_tmap_5d(&mdo, dout, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt))
+      !make_tmap_5d(&mdo, dout, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
+      !make_tmap_slots(&mdq, dq_s, kD, slots, 16) || !make_tmap_slots(&mdk, dk_s, kD, slots, 32) ||
+      !make_tmap_slots(&mdv, dv_s, kD, slots, 32))
     return cudaErrorInvalidValue;
   const int grid = (int)(a.items < num_sms() ? a.items : num_sms());
   auto k1 = dkdv64_kernel<OutT>;
   cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, Kv64::kSmem);
   if (e != cudaSuccess) return e;
   prof_begin(kKBwdDkdv, st);
-  k1<<<grid, kThreads64, Kv64::kSmem, st>>>(mq, mk, mv, mdo, a);
+  k1<<<grid, kThreads64, Kv64::kSmem, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
   prof_end(kKBwdDkdv, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   auto k2 = dq64_kernel<OutT>;
   e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, Q64::kSmem);
   if (e != cudaSuccess) return e;
   prof_begin(kKBwdDq, st);
-  k2<<<grid, kThreadsQ64, Q64::kSmem, st>>>(mq, mk, mv, mdo, a);
+  k2<<<grid, kThreadsQ64, Q64::kSmem, st>>>(mq, mk, mv, mdo, mdq, a);
   prof_end(kKBwdDq, st);
   return cudaGetLastError();
 }

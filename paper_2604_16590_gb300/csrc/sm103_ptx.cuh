@@ -125,6 +125,29 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
+// 2-D tiled store shared -> global (bulk group): a box of a row-major matrix at
+// column c0 (x element size a multiple of 16 bytes) and row c1.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, uint32_t src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(m)),
+               "r"(src), "r"(c0), "r"(c1)
+               : "memory");
+}
+// 5-D tiled store shared -> global (bulk group); rows past the tensor's end are
+// not written.
+__device__ __forceinline__ void tma_store_5d(const CUtensorMap* m, uint32_t src, int c0, int c1, int c2, int c3,
+                                             int c4) {
+  asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(m)),
+               "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+               : "memory");
+}
+// Close this thread's bulk group; wait until its groups have read their shared
+// memory; wait until their writes are complete.  (A wait ends with the copies.)
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ------------------------------------------------------------------ tcgen05
@@ -361,5 +384,10 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
 // Host: 5-D tiled tensor map over a [BH, T, Y, X, d] BF16 tensor (d innermost),
 // box (64, bx, by, bt, 1), 128-byte swizzle, zero fill out of range.
 bool make_tmap_5d(CUtensorMap* map, const void* base, int d, int X, int Y, int T, int BH, int bx, int by, int bt);
+
+// Host: 2-D tiled tensor map over `rows` FP32 rows of d columns (the per-tile
+// slots), box of 32 rows x `cols` columns: 32 (128-byte swizzle) or 16 (64-byte
+// swizzle).
+bool make_tmap_slots(CUtensorMap* map, const float* base, int d, int64_t rows, int cols);
 
 }  // namespace gattn
