@@ -4,386 +4,571 @@
 // the FP32 baseline the BF16 tensor-core form is measured against, and the
 // path used when the inputs are FP32.
 //
-// Work decomposition: one CTA of 128 threads per (row block, tile, batch*head);
-// each row of the extended tile is owned by TPR = D/DPT consecutive lanes,
-// each lane holding DPT = 16 of the D head dimensions in registers; partial
-// dot products are combined with warp shuffles.  Keys (or queries, for dK/dV)
-// stream through shared memory in chunks of KC rows; every chunk is reduced
+// Work decomposition: one CTA per (row block, tile, batch*head); a warp owns
+// 8 RG rows of the extended tile, keys (or queries, for dK/dV) stream through
+// shared memory 64 at a time.  Both kinds of products are register-tiled, 8
+// rows per thread, and issue packed FP32 pairs (fma.rn.f32x2), so that the FMA
+// pipe is the limit and not the issue slots or the shared-memory reads:
+//   scores   8 rows x KT keys a thread, contraction over d in pairs of
+//            neighbouring elements (both operands are d-contiguous, so pairs
+//            load as they lie; the two partial sums are added at the end);
+//            12 16-byte loads per 64 pair instructions at d = 64
+//   P V, ... 8 rows x CT columns a thread, one key at a time; the warp's P is
+//            kept key-major with every value doubled ((p, p) pairs), so its
+//            operand needs no moves; 5 loads per 16 pair instructions
+// Rows never leave their warp: P goes through a warp-private buffer, so CTA
+// barriers only order the streamed blocks.  Every 64-row block is reduced
 // locally before it is folded into the running sums (two-level summation,
-// which keeps the FP32 error of L-long sums near eps * (sqrt(KC) + sqrt(L/KC))).
+// which keeps the FP32 error of L-long sums near eps * (sqrt(64) + sqrt(L/64))).
+// Bound: the FP32 pipe (128 lanes a clock and SM).  4 heads of a 4 x 64 x 128
+// clip in 16 tiles of up to 4608 tokens, d = 64: forward 14.6 -> 7.4 ms, dQ
+// 17.0 -> 9.3, dK/dV 19.4 -> 12.4 (before: a thread group per row, one FMA per
+// shared-memory word).
 #include "internal.cuh"
+#include "sm103_common.cuh"
 
 GATTN_DEFINE_STATUS(simt)
 
 namespace gattn {
 namespace {
+using sm103::f2pack;
+using sm103::f2unpack;
+using sm103::fadd2;
+using sm103::ffma2;
+using sm103::fmul2;
 
-constexpr int kThreads = 128;
-constexpr int kDPT = 16;  // head dims per lane
-constexpr int kKC = 32;   // rows per shared-memory chunk
+constexpr int kBN = 64;  // streamed rows per block
 
-// Physical float4 slot of lane group `grp`'s f-th float4 in a staged row:
-// spreads the groups of one quarter-warp over distinct shared-memory banks.
-__device__ __forceinline__ int swz(int grp, int f) { return 4 * grp + (f ^ ((grp >> 1) & 3)); }
+// Shape of the kernels at head size D with W warps per CTA.
+template <int D_, int W_>
+struct Shape {
+  static constexpr int D = D_, W = W_;
+  static constexpr int RG = D == 128 ? 1 : 2;   // row groups of a warp, 8 rows each
+  static constexpr int LG = 32 / RG;            // lanes of a row group
+  static constexpr int KT = kBN / LG;           // score columns per thread: keys lg + LG * jj
+  static constexpr int CT = D / LG;             // output columns per thread: CT * lg ...
+  static constexpr int WR = 8 * RG;             // rows per warp
+  static constexpr int BM = W * WR;             // rows per CTA
+  static constexpr int T = 32 * W;
+  static constexpr int LD = D + 4;              // padded row of a staged matrix (floats): conflict-free column walks
+  static constexpr int HK = 2 * LG;             // keys of P exchanged at a time (two score columns per thread)
+  static constexpr int NH = kBN / HK;
+  static constexpr int PB = 2 * WR + 4;         // floats per key of the doubled P buffer, padded
+  static constexpr int PW = HK * PB;            // floats of a warp's P buffer
+};
 
-// Stage rows [j0, j0+KC) of the tile from two [N, D] tensors into shared memory.
-template <int D>
-__device__ __forceinline__ void stage_rows(const Geom& g, const TileBox& tb, int j0, const float* __restrict__ A,
-                                           const float* __restrict__ Bm, float* As, float* Bs) {
-  constexpr int F4 = D / 4;
-  for (int idx = threadIdx.x; idx < kKC * F4; idx += kThreads) {
-    int jj = idx / F4, F = idx % F4;
-    int j = j0 + jj;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (j < tb.L) {
-      int64_t tok = tile_token(g, tb, j);
-      a = __ldg(reinterpret_cast<const float4*>(A + tok * D) + F);
-      b = __ldg(reinterpret_cast<const float4*>(Bm + tok * D) + F);
+// Tile-row tokens: row r of the extended tile by FP32 quotients (box_index).
+__device__ __forceinline__ int64_t row_token(const Geom& g, const TileBox& tb, int r, int l[3]) {
+  box_index(r, tb.e[1], tb.e[2], l[0], l[1], l[2]);
+  return grid_token(g, tb, l);
+}
+
+__device__ __forceinline__ void cp16(float* dst, const float* src, bool ok) {
+  const int n = ok ? 16 : 0;  // 0: the 16 bytes are zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm103::smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Rows [j0, j0 + ROWS) of the tile of a [N, D] tensor into padded rows (zeros past the tile).
+template <class S, int ROWS>
+__device__ __forceinline__ void stage(const Geom& g, const TileBox& tb, int j0, const float* __restrict__ A, float* As) {
+  constexpr int F4 = S::D / 4;
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < ROWS * F4; idx += S::T) {
+    const int jj = idx / F4, f = idx % F4;
+    const bool ok = j0 + jj < tb.L;
+    int l[3];
+    const int64_t tok = row_token(g, tb, ok ? j0 + jj : 0, l);
+    cp16(As + jj * S::LD + 4 * f, A + tok * S::D + 4 * f, ok);
+  }
+}
+
+// acc[i][jj] = rows[i] . cols[lg + LG jj]: 8 rows from `rows` (this thread's row
+// group), KT columns.
+template <class S>
+__device__ __forceinline__ void dots(const float* __restrict__ rows, const float* __restrict__ cols, int lg,
+                                     float (&s)[8][S::KT]) {
+  uint64_t acc[8][S::KT];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) acc[i][j] = 0;
+  const float* cp = cols + lg * S::LD;
+#pragma unroll 2
+  for (int k = 0; k < S::D; k += 4) {
+    ulonglong2 b[S::KT];
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(cp + j * S::LG * S::LD + k);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(rows + i * S::LD + k);
+#pragma unroll
+      for (int j = 0; j < S::KT; ++j) {
+        acc[i][j] = ffma2(a.x, b[j].x, acc[i][j]);
+        acc[i][j] = ffma2(a.y, b[j].y, acc[i][j]);
+      }
     }
-    int p = swz(F / 4, F % 4);
-    reinterpret_cast<float4*>(As + jj * D)[p] = a;
-    reinterpret_cast<float4*>(Bs + jj * D)[p] = b;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) {
+      float x, y;
+      f2unpack(acc[i][j], x, y);
+      s[i][j] = x + y;
+    }
+}
+
+// out[i][c] += sum over the block's 64 keys of p[i][key] * M[key][CT lg + c],
+// p being this thread's score columns (exchanged within the warp through pb).
+template <class S>
+__device__ __forceinline__ void axpys(const float (&p)[8][S::KT], const float* __restrict__ M, float* pb, int rg, int lg,
+                                      uint64_t (&out)[8][S::CT / 2]) {
+  uint64_t acc[8][S::CT / 2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < S::CT / 2; ++c) acc[i][c] = 0;
+#pragma unroll
+  for (int h = 0; h < S::NH; ++h) {
+    __syncwarp();  // the previous half (or product) has been read
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj) {
+      float4* d = reinterpret_cast<float4*>(pb + (lg + S::LG * jj) * S::PB + 16 * rg);
+#pragma unroll
+      for (int i = 0; i < 8; i += 2)
+        d[i / 2] = make_float4(p[i][2 * h + jj], p[i][2 * h + jj], p[i + 1][2 * h + jj], p[i + 1][2 * h + jj]);
+    }
+    __syncwarp();
+    const float* m = M + h * S::HK * S::LD + S::CT * lg;
+    const float* pp = pb + 16 * rg;
+#pragma unroll 4
+    for (int key = 0; key < S::HK; ++key) {
+      uint64_t v[S::CT / 2];
+      if constexpr (S::CT == 4) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(m + key * S::LD);
+        v[0] = t.x;
+        v[1] = t.y;
+      } else {
+        v[0] = *reinterpret_cast<const uint64_t*>(m + key * S::LD);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i += 2) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pp + key * S::PB + 2 * i);
+#pragma unroll
+        for (int c = 0; c < S::CT / 2; ++c) {
+          acc[i][c] = ffma2(a.x, v[c], acc[i][c]);
+          acc[i + 1][c] = ffma2(a.y, v[c], acc[i + 1][c]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < S::CT / 2; ++c) out[i][c] = fadd2(out[i][c], acc[i][c]);
+}
+
+// CT accumulated columns of one row, times mul, to the output row or the slot row
+template <int CT, typename T>
+__device__ __forceinline__ void store_cols(T* dst, const uint64_t (&a)[CT / 2], float mul) {
+  float x[CT];
+#pragma unroll
+  for (int c = 0; c < CT / 2; ++c) f2unpack(a[c], x[2 * c], x[2 * c + 1]);
+  if constexpr (CT == 4) {
+    store4<T>(dst, make_float4(x[0] * mul, x[1] * mul, x[2] * mul, x[3] * mul));
+  } else if constexpr (sizeof(T) == 2) {
+    *reinterpret_cast<__nv_bfloat162*>(dst) = __floats2bfloat162_rn(x[0] * mul, x[1] * mul);
+  } else {
+    *reinterpret_cast<float2*>(dst) = make_float2(x[0] * mul, x[1] * mul);
   }
 }
 
-template <int D>
-__device__ __forceinline__ float dot_group(const float (&x)[kDPT], const float* row, int grp) {
-  float s = 0.f;
+template <int LG>
+__device__ __forceinline__ float group_max(float v) {
 #pragma unroll
-  for (int f = 0; f < kDPT / 4; ++f) {
-    float4 k4 = reinterpret_cast<const float4*>(row)[swz(grp, f)];
-    s = fmaf(x[4 * f + 0], k4.x, s);
-    s = fmaf(x[4 * f + 1], k4.y, s);
-    s = fmaf(x[4 * f + 2], k4.z, s);
-    s = fmaf(x[4 * f + 3], k4.w, s);
-  }
-  return s;
+  for (int o = 1; o < LG; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
 }
-
-template <int TPR>
-__device__ __forceinline__ float group_sum(float s) {
+template <int LG>
+__device__ __forceinline__ float group_sum(float v) {
 #pragma unroll
-  for (int o = 1; o < TPR; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
-template <int D>
-__device__ __forceinline__ void axpy_group(float (&acc)[kDPT], float a, const float* row, int grp) {
-#pragma unroll
-  for (int f = 0; f < kDPT / 4; ++f) {
-    float4 v4 = reinterpret_cast<const float4*>(row)[swz(grp, f)];
-    acc[4 * f + 0] = fmaf(a, v4.x, acc[4 * f + 0]);
-    acc[4 * f + 1] = fmaf(a, v4.y, acc[4 * f + 1]);
-    acc[4 * f + 2] = fmaf(a, v4.z, acc[4 * f + 2]);
-    acc[4 * f + 3] = fmaf(a, v4.w, acc[4 * f + 3]);
-  }
-}
-
-__device__ __forceinline__ void load_group(float (&x)[kDPT], const float* __restrict__ src) {
-#pragma unroll
-  for (int f = 0; f < kDPT / 4; ++f) {
-    float4 t = __ldg(reinterpret_cast<const float4*>(src) + f);
-    x[4 * f + 0] = t.x;
-    x[4 * f + 1] = t.y;
-    x[4 * f + 2] = t.z;
-    x[4 * f + 3] = t.w;
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void store_group(T* dst, const float (&x)[kDPT], float mul) {
-#pragma unroll
-  for (int f = 0; f < kDPT / 4; ++f)
-    store4<T>(dst + 4 * f, make_float4(x[4 * f] * mul, x[4 * f + 1] * mul, x[4 * f + 2] * mul, x[4 * f + 3] * mul));
+  for (int o = 1; o < LG; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // ---------------------------------------------------------------- forward
-template <int D, typename OutT>
-__global__ void __launch_bounds__(kThreads) simt_fwd_kernel(Geom g, const float* __restrict__ Q,
-                                                            const float* __restrict__ K,
-                                                            const float* __restrict__ V, OutT* __restrict__ out,
-                                                            float* __restrict__ lse2, float* __restrict__ ot) {
-  constexpr int TPR = D / kDPT, RPC = kThreads / TPR;
-  __shared__ __align__(16) float Ks[kKC * D];
-  __shared__ __align__(16) float Vs[kKC * D];
+template <class S>
+struct FwdSmem {
+  float q[S::BM * S::LD];
+  float k[2][kBN * S::LD];
+  float v[2][kBN * S::LD];
+  float p[S::W][S::PW];
+};
+
+template <class S, typename OutT>
+__global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const float* __restrict__ Q,
+                                                        const float* __restrict__ K, const float* __restrict__ V,
+                                                        OutT* __restrict__ out, float* __restrict__ lse2,
+                                                        float* __restrict__ ot) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  auto& sm = *reinterpret_cast<FwdSmem<S>*>(smem_raw);
   const int tile = blockIdx.y, bh = blockIdx.z;
   TileBox tb;
   tile_box(g, tile, tb);
-  const int row0 = blockIdx.x * RPC;
+  const int row0 = blockIdx.x * S::BM;
   if (row0 >= tb.L) return;  // uniform over the CTA
-  const int grp = threadIdx.x % TPR;
-  const int r = row0 + threadIdx.x / TPR;
-  const bool active = r < tb.L;
-  const int64_t base = (int64_t)bh * g.N * D;
-  const float* Qb = Q + base;
-  const float* Kb = K + base;
-  const float* Vb = V + base;
-  int64_t tok = active ? tile_token(g, tb, r) : 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rg = lane / S::LG, lg = lane % S::LG;
+  const int64_t base = (int64_t)bh * g.N * S::D;
+  stage<S, S::BM>(g, tb, row0, Q + base, sm.q);
+  stage<S, kBN>(g, tb, 0, K + base, sm.k[0]);
+  stage<S, kBN>(g, tb, 0, V + base, sm.v[0]);
+  cp_commit();
+  const int r0 = warp * S::WR + rg * 8;  // first of this thread's 8 rows within the CTA
+  float* pb = sm.p[warp];
 
-  float q[kDPT], o[kDPT], oc[kDPT];
-  if (active) load_group(q, Qb + tok * D + grp * kDPT);
-  else
+  uint64_t o[8][S::CT / 2];
+  float m[8], l[8];
 #pragma unroll
-    for (int e = 0; e < kDPT; ++e) q[e] = 0.f;
+  for (int i = 0; i < 8; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.f;
 #pragma unroll
-  for (int e = 0; e < kDPT; ++e) o[e] = 0.f;
-  float m = -INFINITY, l = 0.f;
-
-  for (int j0 = 0; j0 < tb.L; j0 += kKC) {
-    __syncthreads();
-    stage_rows<D>(g, tb, j0, Kb, Vb, Ks, Vs);
-    __syncthreads();
-    float s[kKC];
-    float cmax = -INFINITY;
-#pragma unroll
-    for (int jj = 0; jj < kKC; ++jj) {
-      float d = group_sum<TPR>(dot_group<D>(q, Ks + jj * D, grp));
-      s[jj] = (j0 + jj < tb.L) ? d * g.scale_log2 : -INFINITY;
-      cmax = fmaxf(cmax, s[jj]);
-    }
-    const float mnew = fmaxf(m, cmax);
-    const float alpha = exp2f(m - mnew);  // 0 on the first chunk (m = -inf)
-    float lc = 0.f;
-#pragma unroll
-    for (int e = 0; e < kDPT; ++e) oc[e] = 0.f;
-#pragma unroll
-    for (int jj = 0; jj < kKC; ++jj) {
-      float p = exp2f(s[jj] - mnew);
-      lc += p;
-      axpy_group<D>(oc, p, Vs + jj * D, grp);
-    }
-    l = l * alpha + lc;
-#pragma unroll
-    for (int e = 0; e < kDPT; ++e) o[e] = o[e] * alpha + oc[e];
-    m = mnew;
+    for (int c = 0; c < S::CT / 2; ++c) o[i][c] = 0;
   }
-  if (!active) return;
-  const float inv = 1.f / l;
-  int lr[3];
-  tile_local(tb, r, lr);
-  const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
-  if (grp == 0) lse2[slot] = m + log2f(l);
-  int p[3];
-  token_pos(g, tok, p);
-  if (single_cover(g, p)) {
-    store_group<OutT>(out + base + tok * D + grp * kDPT, o, inv);
-  } else {
-    store_group<float>(ot + slot * D + grp * kDPT, o, inv);
+  for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
+    cp_wait<0>();
+    __syncthreads();  // block j0 is staged, block j0 - 64 has been read by every warp
+    if (j0 + kBN < tb.L) {
+      stage<S, kBN>(g, tb, j0 + kBN, K + base, sm.k[b ^ 1]);
+      stage<S, kBN>(g, tb, j0 + kBN, V + base, sm.v[b ^ 1]);
+      cp_commit();
+    }
+    float s[8][S::KT];
+    dots<S>(sm.q + r0 * S::LD, sm.k[b], lg, s);
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) {
+      const bool in = j0 + lg + S::LG * j < tb.L;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i][j] = in ? s[i][j] * g.scale_log2 : -INFINITY;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float mx = s[i][0];
+#pragma unroll
+      for (int j = 1; j < S::KT; ++j) mx = fmaxf(mx, s[i][j]);
+      mx = fmaxf(m[i], group_max<S::LG>(mx));
+      const float alpha = exp2f(m[i] - mx);  // 0 on the first block (m = -inf)
+      m[i] = mx;
+      float lc = 0.f;
+#pragma unroll
+      for (int j = 0; j < S::KT; ++j) {
+        s[i][j] = exp2f(s[i][j] - mx);
+        lc += s[i][j];
+      }
+      l[i] = l[i] * alpha + lc;  // this thread's keys; the group's sums are added at the end
+      const uint64_t a2 = f2pack(alpha, alpha);
+#pragma unroll
+      for (int c = 0; c < S::CT / 2; ++c) o[i][c] = fmul2(o[i][c], a2);
+    }
+    axpys<S>(s, sm.v[b], pb, rg, lg, o);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float ls = group_sum<S::LG>(l[i]);
+    const int r = row0 + r0 + i;
+    if (r >= tb.L) continue;
+    int lr[3];
+    const int64_t tok = row_token(g, tb, r, lr);
+    const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
+    const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
+    if (lg == 0) lse2[slot] = m[i] + log2f(ls);
+    const float inv = 1.f / ls;
+    if (only_cover(g, tb, p)) store_cols<S::CT>(out + base + tok * S::D + S::CT * lg, o[i], inv);
+    else store_cols<S::CT>(ot + slot * S::D + S::CT * lg, o[i], inv);
   }
 }
 
 // ---------------------------------------------------------------- backward: dQ
 // P = exp2(s q.k log2e - lse') already carries the merge weight w_t / sum w,
 // so dS = P (dOut.v - D) and dQ_t = s sum_j dS k_j (the workspace holds -lse'
-// and -D).
-template <int D, typename OutT>
-__global__ void __launch_bounds__(kThreads) simt_dq_kernel(Geom g, const float* __restrict__ Q,
-                                                           const float* __restrict__ K,
-                                                           const float* __restrict__ V,
-                                                           const float* __restrict__ dO,
-                                                           const float* __restrict__ lse2c,
-                                                           const float* __restrict__ dd, OutT* __restrict__ dq,
-                                                           float* __restrict__ dq_s) {
-  constexpr int TPR = D / kDPT, RPC = kThreads / TPR;
-  __shared__ __align__(16) float Ks[kKC * D];
-  __shared__ __align__(16) float Vs[kKC * D];
+// and -D).  V of the next block is loaded while this block's dQ product runs,
+// K one block ahead.
+template <class S>
+struct DqSmem {
+  float q[S::BM * S::LD];
+  float go[S::BM * S::LD];
+  float k[2][kBN * S::LD];
+  float v[kBN * S::LD];
+  float p[S::W][S::PW];
+};
+
+template <class S, typename OutT>
+__global__ void __launch_bounds__(S::T) simt_dq_kernel(const Geom g, const float* __restrict__ Q,
+                                                       const float* __restrict__ K, const float* __restrict__ V,
+                                                       const float* __restrict__ dO, const float* __restrict__ lse2c,
+                                                       const float* __restrict__ dd, OutT* __restrict__ dq,
+                                                       float* __restrict__ dq_s) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  auto& sm = *reinterpret_cast<DqSmem<S>*>(smem_raw);
   const int tile = blockIdx.y, bh = blockIdx.z;
   TileBox tb;
   tile_box(g, tile, tb);
-  const int row0 = blockIdx.x * RPC;
+  const int row0 = blockIdx.x * S::BM;
   if (row0 >= tb.L) return;
-  const int grp = threadIdx.x % TPR;
-  const int r = row0 + threadIdx.x / TPR;
-  const bool active = r < tb.L;
-  const int64_t base = (int64_t)bh * g.N * D;
-  int64_t tok = active ? tile_token(g, tb, r) : 0;
-  int lr[3];
-  tile_local(tb, active ? r : 0, lr);
-  const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
-
-  float q[kDPT], go[kDPT], acc[kDPT], accc[kDPT];
-  if (active) {
-    load_group(q, Q + base + tok * D + grp * kDPT);
-    load_group(go, dO + base + tok * D + grp * kDPT);
-  } else {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rg = lane / S::LG, lg = lane % S::LG;
+  const int64_t base = (int64_t)bh * g.N * S::D;
+  stage<S, S::BM>(g, tb, row0, Q + base, sm.q);
+  stage<S, S::BM>(g, tb, row0, dO + base, sm.go);
+  stage<S, kBN>(g, tb, 0, K + base, sm.k[0]);
+  stage<S, kBN>(g, tb, 0, V + base, sm.v);
+  cp_commit();
+  const int r0 = warp * S::WR + rg * 8;
+  float nL[8], nD[8];  // -lse' and -D (negated in the workspace)
 #pragma unroll
-    for (int e = 0; e < kDPT; ++e) q[e] = go[e] = 0.f;
+  for (int i = 0; i < 8; ++i) {
+    const int r = row0 + r0 + i;
+    nL[i] = -INFINITY;
+    nD[i] = 0.f;
+    if (r < tb.L) {
+      int lr[3];
+      row_token(g, tb, r, lr);
+      const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
+      nL[i] = lse2c[slot];
+      nD[i] = dd[slot];
+    }
   }
-  const float nL = active ? lse2c[slot] : -INFINITY;  // -lse' (negated in the workspace)
-  const float nD = active ? dd[slot] : 0.f;           // -D
+  uint64_t acc[8][S::CT / 2];
 #pragma unroll
-  for (int e = 0; e < kDPT; ++e) acc[e] = 0.f;
-
-  for (int j0 = 0; j0 < tb.L; j0 += kKC) {
-    __syncthreads();
-    stage_rows<D>(g, tb, j0, K + base, V + base, Ks, Vs);
-    __syncthreads();
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int e = 0; e < kDPT; ++e) accc[e] = 0.f;
-#pragma unroll 8
-    for (int jj = 0; jj < kKC; ++jj) {
-      float sk = dot_group<D>(q, Ks + jj * D, grp);
-      float dp = dot_group<D>(go, Vs + jj * D, grp);
-      sk = group_sum<TPR>(sk);
-      dp = group_sum<TPR>(dp);
-      float p = (j0 + jj < tb.L) ? exp2f(fmaf(sk, g.scale_log2, nL)) : 0.f;
-      float ds = p * (dp + nD);
-      axpy_group<D>(accc, ds, Ks + jj * D, grp);
+    for (int c = 0; c < S::CT / 2; ++c) acc[i][c] = 0;
+  for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
+    const bool more = j0 + kBN < tb.L;
+    cp_wait<0>();
+    __syncthreads();  // block j0 is staged, the other K buffer has been read
+    if (more) stage<S, kBN>(g, tb, j0 + kBN, K + base, sm.k[b ^ 1]);
+    float s[8][S::KT], dp[8][S::KT];
+    dots<S>(sm.q + r0 * S::LD, sm.k[b], lg, s);
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) {
+      const bool in = j0 + lg + S::LG * j < tb.L;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i][j] = in ? exp2f(fmaf(s[i][j], g.scale_log2, nL[i])) : 0.f;
+    }
+    dots<S>(sm.go + r0 * S::LD, sm.v, lg, dp);
+    __syncthreads();  // V has been read
+    if (more) {
+      stage<S, kBN>(g, tb, j0 + kBN, V + base, sm.v);
+      cp_commit();
     }
 #pragma unroll
-    for (int e = 0; e < kDPT; ++e) acc[e] += accc[e];
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < S::KT; ++j) s[i][j] *= dp[i][j] + nD[i];
+    axpys<S>(s, sm.k[b], sm.p[warp], rg, lg, acc);
   }
-  if (!active) return;
-  int p[3];
-  token_pos(g, tok, p);
-  if (single_cover(g, p)) store_group<OutT>(dq + base + tok * D + grp * kDPT, acc, g.scale);
-  else store_group<float>(dq_s + slot * D + grp * kDPT, acc, g.scale);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = row0 + r0 + i;
+    if (r >= tb.L) continue;
+    int lr[3];
+    const int64_t tok = row_token(g, tb, r, lr);
+    const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
+    if (only_cover(g, tb, p)) store_cols<S::CT>(dq + base + tok * S::D + S::CT * lg, acc[i], g.scale);
+    else store_cols<S::CT>(dq_s + slot_of(g, bh, tile, tb.e, lr) * S::D + S::CT * lg, acc[i], g.scale);
+  }
 }
 
 // ---------------------------------------------------------------- backward: dK, dV
-// One row per key j: dV_t(j) = sum_i P_ij dOut_i, dK_t(j) = s sum_i dS_ij q_i.
-template <int D, typename OutT>
-__global__ void __launch_bounds__(kThreads) simt_dkdv_kernel(Geom g, const float* __restrict__ Q,
-                                                             const float* __restrict__ K,
-                                                             const float* __restrict__ V,
-                                                             const float* __restrict__ dO,
-                                                             const float* __restrict__ lse2c,
-                                                             const float* __restrict__ dd, OutT* __restrict__ dk,
-                                                             OutT* __restrict__ dv, float* __restrict__ dk_s,
-                                                             float* __restrict__ dv_s) {
-  constexpr int TPR = D / kDPT, RPC = kThreads / TPR;
-  __shared__ __align__(16) float Qs[kKC * D];
-  __shared__ __align__(16) float Os[kKC * D];
-  __shared__ float Ls[kKC];
-  __shared__ float Ds[kKC];
+// Rows are keys: dV_t(j) = sum_i P_ij dOut_i, dK_t(j) = s sum_i dS_ij q_i.
+// dOut of the next block is loaded while this block's dK product runs, Q one
+// block ahead.
+template <class S>
+struct DkvSmem {
+  float k[S::BM * S::LD];
+  float v[S::BM * S::LD];
+  float q[2][kBN * S::LD];
+  float go[kBN * S::LD];
+  float p[S::W][S::PW];
+  float nL[2][kBN], nD[2][kBN];
+};
+
+template <class S, typename OutT>
+__global__ void __launch_bounds__(S::T) simt_dkdv_kernel(const Geom g, const float* __restrict__ Q,
+                                                         const float* __restrict__ K, const float* __restrict__ V,
+                                                         const float* __restrict__ dO, const float* __restrict__ lse2c,
+                                                         const float* __restrict__ dd, OutT* __restrict__ dk,
+                                                         OutT* __restrict__ dv, float* __restrict__ dk_s,
+                                                         float* __restrict__ dv_s) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  auto& sm = *reinterpret_cast<DkvSmem<S>*>(smem_raw);
   const int tile = blockIdx.y, bh = blockIdx.z;
   TileBox tb;
   tile_box(g, tile, tb);
-  const int row0 = blockIdx.x * RPC;
+  const int row0 = blockIdx.x * S::BM;
   if (row0 >= tb.L) return;
-  const int grp = threadIdx.x % TPR;
-  const int r = row0 + threadIdx.x / TPR;
-  const bool active = r < tb.L;
-  const int64_t base = (int64_t)bh * g.N * D;
-  int64_t tok = active ? tile_token(g, tb, r) : 0;
-
-  float kr[kDPT], vr[kDPT], adk[kDPT], adv[kDPT], cdk[kDPT], cdv[kDPT];
-  if (active) {
-    load_group(kr, K + base + tok * D + grp * kDPT);
-    load_group(vr, V + base + tok * D + grp * kDPT);
-  } else {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rg = lane / S::LG, lg = lane % S::LG;
+  const int64_t base = (int64_t)bh * g.N * S::D;
+  // -lse' and -D of the block's queries; rows past the tile get P = 0
+  auto stats = [&](int i0, int b) {
+    for (int t = threadIdx.x; t < kBN; t += S::T) {
+      float a = -INFINITY, d = 0.f;
+      if (i0 + t < tb.L) {
+        int lr[3];
+        row_token(g, tb, i0 + t, lr);
+        const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
+        a = lse2c[slot];
+        d = dd[slot];
+      }
+      sm.nL[b][t] = a;
+      sm.nD[b][t] = d;
+    }
+  };
+  stage<S, S::BM>(g, tb, row0, K + base, sm.k);
+  stage<S, S::BM>(g, tb, row0, V + base, sm.v);
+  stage<S, kBN>(g, tb, 0, Q + base, sm.q[0]);
+  stage<S, kBN>(g, tb, 0, dO + base, sm.go);
+  cp_commit();
+  stats(0, 0);
+  const int r0 = warp * S::WR + rg * 8;
+  uint64_t adk[8][S::CT / 2], adv[8][S::CT / 2];
 #pragma unroll
-    for (int e = 0; e < kDPT; ++e) kr[e] = vr[e] = 0.f;
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < S::CT / 2; ++c) adk[i][c] = adv[i][c] = 0;
+  for (int i0 = 0, b = 0; i0 < tb.L; i0 += kBN, b ^= 1) {
+    const bool more = i0 + kBN < tb.L;
+    cp_wait<0>();
+    __syncthreads();  // block i0 is staged, the other Q buffer has been read
+    if (more) {
+      stage<S, kBN>(g, tb, i0 + kBN, Q + base, sm.q[b ^ 1]);
+      stats(i0 + kBN, b ^ 1);
+    }
+    float s[8][S::KT], dp[8][S::KT];
+    dots<S>(sm.k + r0 * S::LD, sm.q[b], lg, s);
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) {
+      const float nL = sm.nL[b][lg + S::LG * j];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i][j] = exp2f(fmaf(s[i][j], g.scale_log2, nL));
+    }
+    axpys<S>(s, sm.go, sm.p[warp], rg, lg, adv);
+    dots<S>(sm.v + r0 * S::LD, sm.go, lg, dp);
+    __syncthreads();  // dOut has been read
+    if (more) {
+      stage<S, kBN>(g, tb, i0 + kBN, dO + base, sm.go);
+      cp_commit();
+    }
+#pragma unroll
+    for (int j = 0; j < S::KT; ++j) {
+      const float nD = sm.nD[b][lg + S::LG * j];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i][j] *= dp[i][j] + nD;
+    }
+    axpys<S>(s, sm.q[b], sm.p[warp], rg, lg, adk);
   }
 #pragma unroll
-  for (int e = 0; e < kDPT; ++e) adk[e] = adv[e] = 0.f;
-
-  for (int i0 = 0; i0 < tb.L; i0 += kKC) {
-    __syncthreads();
-    stage_rows<D>(g, tb, i0, Q + base, dO + base, Qs, Os);
-    if (threadIdx.x < kKC) {
-      int i = i0 + threadIdx.x;
-      int li[3];
-      tile_local(tb, i < tb.L ? i : 0, li);
-      int64_t s = slot_of(g, bh, tile, tb.e, li);
-      Ls[threadIdx.x] = i < tb.L ? lse2c[s] : -INFINITY;  // -lse'
-      Ds[threadIdx.x] = i < tb.L ? dd[s] : 0.f;           // -D
+  for (int i = 0; i < 8; ++i) {
+    const int r = row0 + r0 + i;
+    if (r >= tb.L) continue;
+    int lr[3];
+    const int64_t tok = row_token(g, tb, r, lr);
+    const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
+    if (only_cover(g, tb, p)) {
+      store_cols<S::CT>(dk + base + tok * S::D + S::CT * lg, adk[i], g.scale);
+      store_cols<S::CT>(dv + base + tok * S::D + S::CT * lg, adv[i], 1.f);
+    } else {
+      const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
+      store_cols<S::CT>(dk_s + slot * S::D + S::CT * lg, adk[i], g.scale);
+      store_cols<S::CT>(dv_s + slot * S::D + S::CT * lg, adv[i], 1.f);
     }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < kDPT; ++e) cdk[e] = cdv[e] = 0.f;
-#pragma unroll 4
-    for (int ii = 0; ii < kKC; ++ii) {
-      float sk = dot_group<D>(kr, Qs + ii * D, grp);
-      float dp = dot_group<D>(vr, Os + ii * D, grp);
-      sk = group_sum<TPR>(sk);
-      dp = group_sum<TPR>(dp);
-      float p = exp2f(fmaf(sk, g.scale_log2, Ls[ii]));
-      float ds = p * (dp + Ds[ii]);
-      axpy_group<D>(cdv, p, Os + ii * D, grp);
-      axpy_group<D>(cdk, ds, Qs + ii * D, grp);
-    }
-#pragma unroll
-    for (int e = 0; e < kDPT; ++e) {
-      adk[e] += cdk[e];
-      adv[e] += cdv[e];
-    }
-  }
-  if (!active) return;
-  int lr[3];
-  tile_local(tb, r, lr);
-  const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
-  int p[3];
-  token_pos(g, tok, p);
-  if (single_cover(g, p)) {
-    store_group<OutT>(dk + base + tok * D + grp * kDPT, adk, g.scale);
-    store_group<OutT>(dv + base + tok * D + grp * kDPT, adv, 1.f);
-  } else {
-    store_group<float>(dk_s + slot * D + grp * kDPT, adk, g.scale);
-    store_group<float>(dv_s + slot * D + grp * kDPT, adv, 1.f);
   }
 }
 
-template <int D, typename OutT>
-cudaError_t simt_fwd_dispatch(const Geom& g, const float* q, const float* k, const float* v, void* out,
-                              float* lse2, float* ot, cudaStream_t st) {
-  constexpr int RPC = kThreads / (D / kDPT);
-  dim3 grid((g.Lmax + RPC - 1) / RPC, g.ntiles, g.B * g.nh);
-  simt_fwd_kernel<D, OutT><<<grid, kThreads, 0, st>>>(g, q, k, v, static_cast<OutT*>(out), lse2, ot);
+template <typename Kern>
+cudaError_t smem_limit(Kern k, size_t bytes) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <class S, typename OutT>
+cudaError_t fwd_run(const Geom& g, const float* q, const float* k, const float* v, void* out, float* lse2, float* ot,
+                    cudaStream_t st) {
+  const dim3 grid((g.Lmax + S::BM - 1) / S::BM, g.ntiles, g.B * g.nh);
+  auto kern = simt_fwd_kernel<S, OutT>;
+  cudaError_t e = smem_limit(kern, sizeof(FwdSmem<S>));
+  if (e != cudaSuccess) return e;
+  kern<<<grid, S::T, sizeof(FwdSmem<S>), st>>>(g, q, k, v, static_cast<OutT*>(out), lse2, ot);
   return cudaGetLastError();
 }
 
-template <int D, typename OutT>
-cudaError_t simt_bwd_dispatch(const Geom& g, const float* q, const float* k, const float* v, const float* dout,
-                              const float* lse2c, const float* dd, void* dq, void* dk, void* dv, float* dq_s,
-                              float* dk_s, float* dv_s, cudaStream_t st) {
-  constexpr int RPC = kThreads / (D / kDPT);
-  dim3 grid((g.Lmax + RPC - 1) / RPC, g.ntiles, g.B * g.nh);
-  prof_begin(kKBwdDq, st);
-  simt_dq_kernel<D, OutT><<<grid, kThreads, 0, st>>>(g, q, k, v, dout, lse2c, dd, static_cast<OutT*>(dq), dq_s);
-  prof_end(kKBwdDq, st);
-  cudaError_t e = cudaGetLastError();
+template <class S, typename OutT>
+cudaError_t bwd_run(const Geom& g, const float* q, const float* k, const float* v, const float* dout,
+                    const float* lse2c, const float* dd, void* dq, void* dk, void* dv, float* dq_s, float* dk_s,
+                    float* dv_s, cudaStream_t st) {
+  const dim3 grid((g.Lmax + S::BM - 1) / S::BM, g.ntiles, g.B * g.nh);
+  auto k1 = simt_dq_kernel<S, OutT>;
+  auto k2 = simt_dkdv_kernel<S, OutT>;
+  cudaError_t e = smem_limit(k1, sizeof(DqSmem<S>));
+  if (e == cudaSuccess) e = smem_limit(k2, sizeof(DkvSmem<S>));
   if (e != cudaSuccess) return e;
+  prof_begin(kKBwdDq, st);
+  k1<<<grid, S::T, sizeof(DqSmem<S>), st>>>(g, q, k, v, dout, lse2c, dd, static_cast<OutT*>(dq), dq_s);
+  prof_end(kKBwdDq, st);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   prof_begin(kKBwdDkdv, st);
-  simt_dkdv_kernel<D, OutT><<<grid, kThreads, 0, st>>>(g, q, k, v, dout, lse2c, dd, static_cast<OutT*>(dk),
-                                                       static_cast<OutT*>(dv), dk_s, dv_s);
+  k2<<<grid, S::T, sizeof(DkvSmem<S>), st>>>(g, q, k, v, dout, lse2c, dd, static_cast<OutT*>(dk),
+                                             static_cast<OutT*>(dv), dk_s, dv_s);
   prof_end(kKBwdDkdv, st);
   return cudaGetLastError();
+}
+
+// Runs f with the shape for this problem: BM = 64 rows a CTA (a staged block
+// serves twice the rows of BM = 32), or 32 where 64-row blocks would leave SMs
+// without a CTA.
+template <int D, typename F>
+cudaError_t with_shape(const Geom& g, F f) {
+  constexpr int W64 = D == 128 ? 8 : 4;
+  const int64_t blocks = (int64_t)((g.Lmax + 63) / 64) * g.ntiles * g.B * g.nh;
+  if (blocks > num_sms()) return f(Shape<D, W64>());
+  return f(Shape<D, W64 / 2>());
+}
+
+template <typename F>
+cudaError_t with_d(const Geom& g, F f) {
+  switch (g.d) {
+    case 32: return with_shape<32>(g, f);
+    case 64: return with_shape<64>(g, f);
+    case 128: return with_shape<128>(g, f);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
 cudaError_t launch_simt_fwd(const Geom& g, const float* q, const float* k, const float* v, void* out,
                             int out_dtype, float* lse2, float* ot, cudaStream_t st) {
-  const bool bf = out_dtype == GATTN_BF16;
-  switch (g.d) {
-    case 32:
-      return bf ? simt_fwd_dispatch<32, __nv_bfloat16>(g, q, k, v, out, lse2, ot, st)
-                : simt_fwd_dispatch<32, float>(g, q, k, v, out, lse2, ot, st);
-    case 64:
-      return bf ? simt_fwd_dispatch<64, __nv_bfloat16>(g, q, k, v, out, lse2, ot, st)
-                : simt_fwd_dispatch<64, float>(g, q, k, v, out, lse2, ot, st);
-    case 128:
-      return bf ? simt_fwd_dispatch<128, __nv_bfloat16>(g, q, k, v, out, lse2, ot, st)
-                : simt_fwd_dispatch<128, float>(g, q, k, v, out, lse2, ot, st);
-  }
-  return cudaErrorInvalidValue;
+  return with_d(g, [&](auto s) {
+    using S = decltype(s);
+    return out_dtype == GATTN_BF16 ? fwd_run<S, __nv_bfloat16>(g, q, k, v, out, lse2, ot, st)
+                                   : fwd_run<S, float>(g, q, k, v, out, lse2, ot, st);
+  });
 }
 
 cudaError_t launch_simt_bwd(const Geom& g, const float* q, const float* k, const float* v, const float* dout,
                             const float* lse2c, const float* dd, void* dq, void* dk, void* dv, int out_dtype,
                             float* dq_s, float* dk_s, float* dv_s, cudaStream_t st) {
-  const bool bf = out_dtype == GATTN_BF16;
-#define GATTN_SIMT_BWD(DD)                                                                                 \
-  return bf ? simt_bwd_dispatch<DD, __nv_bfloat16>(g, q, k, v, dout, lse2c, dd, dq, dk, dv, dq_s, dk_s, dv_s, st) \
-            : simt_bwd_dispatch<DD, float>(g, q, k, v, dout, lse2c, dd, dq, dk, dv, dq_s, dk_s, dv_s, st);
-  switch (g.d) {
-    case 32: GATTN_SIMT_BWD(32)
-    case 64: GATTN_SIMT_BWD(64)
-    case 128: GATTN_SIMT_BWD(128)
-  }
-#undef GATTN_SIMT_BWD
-  return cudaErrorInvalidValue;
+  return with_d(g, [&](auto s) {
+    using S = decltype(s);
+    return out_dtype == GATTN_BF16
+               ? bwd_run<S, __nv_bfloat16>(g, q, k, v, dout, lse2c, dd, dq, dk, dv, dq_s, dk_s, dv_s, st)
+               : bwd_run<S, float>(g, q, k, v, dout, lse2c, dd, dq, dk, dv, dq_s, dk_s, dv_s, st);
+  });
 }
 
 }  // namespace gattn
