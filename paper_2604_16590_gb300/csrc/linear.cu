@@ -92,16 +92,6 @@ __device__ __forceinline__ void split8(const float (&f)[8], uint4& hi, uint4& lo
   hi = make_uint4(h[0], h[1], h[2], h[3]);
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
-// hi + lo of eight BF16 pairs
-__device__ __forceinline__ void join8(uint4 hi, uint4 lo, float (&f)[8]) {
-  const uint32_t h[4] = {hi.x, hi.y, hi.z, hi.w}, l[4] = {lo.x, lo.y, lo.z, lo.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = __uint_as_float(h[i] << 16) + __uint_as_float(l[i] << 16);
-    f[2 * i + 1] = __uint_as_float(h[i] & 0xffff0000u) + __uint_as_float(l[i] & 0xffff0000u);
-  }
-}
-
 struct SumArgs {
   int N, BH, ntiles, chunk_tiles;
   float* ws_S;  // [chunks, BH, 64, 64]
@@ -471,7 +461,6 @@ __global__ void __launch_bounds__(kThreadsQ, 3) la_query_kernel(const __grid_con
       if (lane == 0) mbar_arrive(staged);
       den_cur = den_next;
     }
-    (void)ok;
   }
   tc_fence_before();
   __syncthreads();
@@ -497,15 +486,39 @@ __global__ void __launch_bounds__(kThreadsQ, 3) la_query_kernel(const __grid_con
 // core's BF16 operands stays below 2^-16; phi(k) and dS in the key pass are
 // split the same way.
 
-constexpr int kThreadsB = 320;               // producer, issuer, 8 math warps (two per TMEM lane quadrant)
-constexpr int kBQStage = 4 * kTileBytes;     // q -> phi hi, g -> g/den hi, phi lo, g/den lo
-constexpr int kBQStages = 2;
-constexpr int kBQBase = 16384 + 3072;        // S^T hi, lo (8 KB each), z, the row-sum exchange, padding
-constexpr int kBQSmem = kBQBase + kBQStages * kBQStage + 1024 + 256;
-constexpr int kBKStage = 3 * kTileBytes;     // k -> phi hi, v, phi lo
-constexpr int kBKStages = 2;
-constexpr int kBKBase = 32768 + 1024;        // dS hi, lo, dS^T hi, lo, then dz and padding
-constexpr int kBKSmem = kBKBase + kBKStages * kBKStage + 1024 + 256;
+// Both backward passes run two groups of eight math warps (two warps per TMEM
+// lane quadrant and group) on alternating tiles: a tile's work is a chain of
+// loads, exchanges and products whose latency one group cannot hide (with one
+// group the passes ran at a third of the HBM rate with 2 of 16 possible warps
+// per scheduler busy).
+constexpr int kThreadsB = 64 + 2 * 256;      // producer, issuer, 2 x 8 math warps
+constexpr int kBQStages = 3;                 // (q, g) ring; phi's and g / den's high parts replace them in place
+constexpr int kBQRaw = 16384 + 5120;         // S^T hi, lo (8 KB each), z, the row-sum exchanges, padding
+constexpr int kBQLo = kBQRaw + kBQStages * 2 * kTileBytes;  // per group: phi lo, g / den lo
+constexpr int kBQOut = kBQLo + 2 * 2 * kTileBytes;          // staged dq, 2 KB per math warp
+constexpr int kBQBar = kBQOut + 16 * 2048;
+constexpr int kBQSmem = kBQBar + 1024 + 256;
+constexpr int kBKStages = 4;                 // (k, v) ring; phi hi, then dk, replace k and dv replaces v in place
+constexpr int kBKRaw = 32768 + 1024;         // dS hi, lo, dS^T hi, lo, then dz and padding
+constexpr int kBKLo = kBKRaw + kBKStages * 2 * kTileBytes;  // per group: phi lo
+constexpr int kBKBar = kBKLo + 2 * kTileBytes;
+constexpr int kBKSmem = kBKBar + 1024 + 256;
+
+// phi of two BF16 values (one 32-bit word) as an FP32 pair: max(x, 0) + min(exp x, 1)
+__device__ __forceinline__ uint64_t phi_pair(uint32_t w) {
+  const float x0 = __uint_as_float(w << 16), x1 = __uint_as_float(w & 0xffff0000u);
+  float e0, e1;
+  f2unpack(fmul2(f2pack(x0, x1), f2pack(1.4426950408889634f, 1.4426950408889634f)), e0, e1);
+  return fadd2(f2pack(fmax_nan(x0, 0.f), fmax_nan(x1, 0.f)), f2pack(fmin_nan(ex2(e0), 1.f), fmin_nan(ex2(e1), 1.f)));
+}
+// BF16 high and low parts of an FP32 pair
+__device__ __forceinline__ void split_pair(uint64_t f, uint32_t& hi, uint32_t& lo) {
+  float a, b;
+  f2unpack(f, a, b);
+  hi = pack_bf16(a, b);
+  f2unpack(ffma2(u2pack(hi << 16, hi & 0xffff0000u), f2pack(-1.f, -1.f), f), a, b);
+  lo = pack_bf16(a, b);
+}
 
 // 64 x 64 BF16 matrices (rows of 128 bytes) from global memory into 128-byte-
 // swizzled shared memory, n of them; every math thread (tid 0..127) takes part
@@ -528,61 +541,68 @@ struct BQArgs {
 };
 
 // Query pass, grid (chunks, BH): every CTA streams a chunk of 128-token query
-// tiles (q and g by TMA through two stages).
-//   issuer: U = G S (A = g tile K-major, B = S^T parts MN-major), into one of
-//           two TMEM buffers; then dS += phi(Q)^T (G / den) over the tile's 128
-//           tokens (both operands MN-major; chains hi.hi, hi.lo, lo.hi)
-//   math:   per row, phi(q) and den in FP32, phi's parts over the q tile and a
-//           side buffer; with U: go, dq (stored), dz; g / den's parts over the
-//           g tile and a side buffer.  Two warps per TMEM lane quadrant, each
-//           taking 32 of a row's 64 columns (the work per row is long and
-//           latency-bound: one warp per sub-partition left it idle most of the
-//           time); the row's two sums (den, phi(q) . U) are exchanged through
-//           shared memory and added in a fixed order.
-// At the end the CTA writes its dS and dz partials.
+// tiles (q and g by TMA through three stages), tile t going to math group t & 1.
+//   issuer: U = G S (A = g tile K-major, B = S^T parts MN-major), into the
+//           group's TMEM buffer, two tiles ahead; dS += phi(Q)^T (G / den) over
+//           the tile's 128 tokens (both operands MN-major; chains hi.hi, hi.lo,
+//           lo.hi)
+//   math:   per row, phi(q) and den in FP32, phi's parts over the q tile and in
+//           the group's low tile; with U: go, dq (staged per warp, stored by
+//           TMA, which also drops rows past N), dz; g / den's parts over the g
+//           tile and in the low tile.  The two warps of a lane quadrant take 32
+//           of a row's 64 columns each and exchange the row's two sums (den,
+//           phi(q) . U) through shared memory, added in a fixed order.
+// At the end the CTA writes its dS and dz partials.  16 heads of 262144
+// tokens: 705 -> 481 us (one group of eight warps, plain stores of dq, before).
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid_constant__ CUtensorMap tq,
                                                                     const __grid_constant__ CUtensorMap tg,
+                                                                    const __grid_constant__ CUtensorMap tdq,
                                                                     const BQArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sHi = smem;
   uint8_t* sLo = smem + 8192;
   float* zs = reinterpret_cast<float*>(smem + 16384);
-  float* xden = reinterpret_cast<float*>(smem + 16384 + 256);  // [2 halves][128 rows]
-  float* xgo = xden + 256;                                     // [2 halves][128 rows]
-  auto stq = [&](int st) { return smem + kBQBase + st * kBQStage; };  // q, then phi hi
-  auto stg = [&](int st) { return stq(st) + kTileBytes; };              // g, then g/den hi
-  auto stpl = [&](int st) { return stq(st) + 2 * kTileBytes; };         // phi lo
-  auto stgl = [&](int st) { return stq(st) + 3 * kTileBytes; };         // g/den lo
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBQBase + kBQStages * kBQStage);
+  float* xsum = reinterpret_cast<float*>(smem + 16384 + 256);  // [group][den, go][half][128 rows]
+  auto stq = [&](int st) { return smem + kBQRaw + st * 2 * kTileBytes; };  // q, then phi hi
+  auto stg = [&](int st) { return stq(st) + kTileBytes; };                 // g, then g/den hi
+  auto lop = [&](int grp) { return smem + kBQLo + grp * 2 * kTileBytes; };  // phi lo
+  auto glo = [&](int grp) { return lop(grp) + kTileBytes; };                // g/den lo
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBQBar);
   uint64_t* empty = full + kBQStages;
-  uint64_t* ufull = empty + kBQStages;
-  uint64_t* ufree = ufull + kBQStages;
-  uint64_t* dsready = ufree + kBQStages;
-  uint64_t* sready = dsready + kBQStages;
+  uint64_t* ufull = empty + kBQStages;  // [group]
+  uint64_t* ufree = ufull + 2;          // [group]
+  uint64_t* dsready = ufree + 2;        // [group]
+  uint64_t* lofree = dsready + 2;       // [group]
+  uint64_t* sready = lofree + 2;
   uint64_t* done = sready + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int chunk = blockIdx.x, bh = blockIdx.y;
   const int t0 = chunk * a.chunk_tiles, t1 = min(a.ntiles, t0 + a.chunk_tiles);
+  const int count = t1 - t0;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kBQStages; ++i) {
       mbar_init(full + i, 1);
       mbar_init(empty + i, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(ufull + i, 1);
       mbar_init(ufree + i, 8);
       mbar_init(dsready + i, 8);
+      mbar_init(lofree + i, 1);
     }
-    mbar_init(sready, 8);
+    mbar_init(sready, 16);
     mbar_init(done, 1);
     *abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tq);
     prefetch_tmap(&tg);
+    prefetch_tmap(&tdq);
   }
   if (warp == 1) {
-    tmem_alloc(tslot, 256);  // U buffers at columns 0 and 64, dS (M = 64) at 128
+    tmem_alloc(tslot, 256);  // the groups' U buffers at columns 0 and 64, dS (M = 64) at 128
     tmem_relinquish();
   }
   tc_fence_before();
@@ -594,14 +614,14 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     if (lane == 0) {  // ------------------------------------------------ TMA producer
       uint32_t armed = 0, par = 0;
       bool ok = true;
-      for (int t = t0, G = 0; t < t1; ++t, ++G) {
+      for (int G = 0; G < count; ++G) {
         const int st = G % kBQStages, n = G / kBQStages;
         if (!(ok = LWAIT(empty + st, (n & 1) ^ 1))) break;
         mbar_arrive_expect_tx(full + st, 2 * kTileBytes);
         armed |= 1u << st;
         par = (par & ~(1u << st)) | ((n & 1) << st);
-        tma_load_5d(stq(st), &tq, full + st, 0, t * kTile, 0, 0, bh);
-        tma_load_5d(stg(st), &tg, full + st, 0, t * kTile, 0, 0, bh);
+        tma_load_5d(stq(st), &tq, full + st, 0, (t0 + G) * kTile, 0, 0, bh);
+        tma_load_5d(stg(st), &tg, full + st, 0, (t0 + G) * kTile, 0, 0, bh);
       }
       if (!ok)
         for (int s2 = 0; s2 < kBQStages; ++s2)
@@ -613,10 +633,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
       constexpr uint32_t idDS = idesc_bf16(64, 64, 1) | (1u << 15);    // A and B MN-major
       const uint64_t dSh = sw128_desc(smem_u32(sHi), 16384, 1024), dSl = sw128_desc(smem_u32(sLo), 16384, 1024);
       bool ok = LWAIT(sready, 0);
-      for (int t = t0, G = 0; t < t1 && ok; ++t, ++G) {
-        const int st = G % kBQStages, n = G / kBQStages, b = G & 1;
-        if (!(ok = LWAIT(full + st, n & 1))) break;
-        if (G >= 2 && !(ok = LWAIT(ufree + b, ((G >> 1) - 1) & 1))) break;
+      // U of tile G into its group's buffer
+      auto issue_u = [&](int G) -> bool {
+        const int st = G % kBQStages, b = G & 1;
+        if (!LWAIT(full + st, (G / kBQStages) & 1)) return false;
+        if (G >= 2 && !LWAIT(ufree + b, ((G >> 1) - 1) & 1)) return false;
         tc_fence_after();
         const uint32_t tU = tmem + 64 * b;
         const uint64_t dG = sw128_desc(smem_u32(stg(st)), 16, 1024);
@@ -625,11 +646,16 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) umma_bf16(tU, dmove(dG, ks * 32), dmove(dSl, ks * 2048), idU, 1u);
         umma_commit(ufull + b);
+        return true;
+      };
+      for (int G = 0; G < 2 && G < count && ok; ++G) ok = issue_u(G);
+      for (int G = 0; G < count && ok; ++G) {
+        const int st = G % kBQStages, b = G & 1;
         // dS += phi(Q)^T (G / den) once the math warps wrote both operands' parts
-        if (!(ok = LWAIT(dsready + st, n & 1))) break;
+        if (!(ok = LWAIT(dsready + b, (G >> 1) & 1))) break;
         tc_fence_after();
-        const uint64_t pH = sw128_desc(smem_u32(stq(st)), 16384, 1024), pL = sw128_desc(smem_u32(stpl(st)), 16384, 1024);
-        const uint64_t gH = sw128_desc(smem_u32(stg(st)), 16384, 1024), gL = sw128_desc(smem_u32(stgl(st)), 16384, 1024);
+        const uint64_t pH = sw128_desc(smem_u32(stq(st)), 16384, 1024), pL = sw128_desc(smem_u32(lop(b)), 16384, 1024);
+        const uint64_t gH = sw128_desc(smem_u32(stg(st)), 16384, 1024), gL = sw128_desc(smem_u32(glo(b)), 16384, 1024);
 #pragma unroll
         for (int ks = 0; ks < kTile / 16; ++ks)
           umma_bf16(tmem + 128, dmove(pH, ks * 2048), dmove(gH, ks * 2048), idDS, (G > 0 || ks > 0) ? 1u : 0u);
@@ -638,145 +664,192 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
 #pragma unroll
         for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tmem + 128, dmove(pL, ks * 2048), dmove(gH, ks * 2048), idDS, 1u);
         umma_commit(empty + st);
+        umma_commit(lofree + b);
+        if (G + 2 < count) ok = issue_u(G + 2);
       }
       umma_commit(done);
       if (!ok) *abort_flag = 1;
+      mbar_wait<set_status_l>(done, 0, abort_flag, false);  // before tensor memory is released
     }
   } else {
     // ------------------------------------------------------------------ math warps
     const int quad = warp & 3;
-    const int h = (warp - 2) >> 2;   // columns [32 h, 32 h + 32) of the row: chunks 4 h .. 4 h + 3
-    const int r = quad * 32 + lane;  // tile row = TMEM lane
+    const int grp = (warp - 2) >> 3;
+    const int h = ((warp - 2) >> 2) & 1;  // columns [32 h, 32 h + 32) of the row: chunks 4 h .. 4 h + 3
+    const int r = quad * 32 + lane;       // tile row = TMEM lane
     const int tid = threadIdx.x - 64;
-    const int pair_bar = 2 + quad;   // named barrier of the two warps of this lane quadrant
+    const int pair_bar = 2 + grp * 4 + quad;  // named barrier of the two warps of this group and lane quadrant
     {
       const __nv_bfloat16* src[2] = {a.sth + (size_t)bh * kD * kD, a.stl + (size_t)bh * kD * kD};
       uint8_t* dst[2] = {sHi, sLo};
-      load_mats(tid, 256, 2, src, dst);
+      load_mats(tid, 512, 2, src, dst);
       if (tid < kD) zs[tid] = a.zt[(size_t)bh * kD + tid];
       fence_proxy_async_smem();
-      asm volatile("bar.sync 1, 256;" ::: "memory");  // z visible to all eight math warps
+      asm volatile("bar.sync 1, 512;" ::: "memory");  // z visible to all math warps
       __syncwarp();
       if (lane == 0) mbar_arrive(sready);
     }
-    float dz[kD / 2];
+    const uint32_t zaddr = smem_u32(zs) + h * 128;
+    float* xden = xsum + grp * 512;
+    float* xgo = xden + 256;
+    const uint32_t out = smem_u32(smem + kBQOut) + (warp - 2) * 2048;  // 32 rows x 64 bytes, 64-byte swizzle
+    const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + 64 * grp + 32 * h;
+    uint64_t dz[kD / 4];
 #pragma unroll
-    for (int i = 0; i < kD / 2; ++i) dz[i] = 0.f;
+    for (int i = 0; i < kD / 4; ++i) dz[i] = 0;
     bool ok = true;
-    for (int t = t0, G = 0; t < t1; ++t, ++G) {
-      const int st = G % kBQStages, n = G / kBQStages, b = G & 1;
-      const bool valid = (int64_t)t * kTile + r < a.N;
-      if (!(ok = LWAIT(full + st, n & 1))) break;
-      // phi(q) in FP32, this half's part of den, and phi's parts (hi over q, lo in its own tile)
-      float dpart = 0.f;
+    for (int G = grp, n = 0; G < count; G += 2, ++n) {
+      const int st = G % kBQStages;
+      const bool valid = (int64_t)(t0 + G) * kTile + r < a.N;
+      if (!(ok = LWAIT(full + st, (G / kBQStages) & 1))) break;
+      // the group's low tiles are free once its previous tile's dS product is done
+      if (n > 0 && !(ok = LWAIT(lofree + grp, (n - 1) & 1))) break;
+      // phi(q) in FP32, this half's part of den, and phi's parts (hi over q, lo in the low tile)
+      const uint32_t aq = smem_u32(stq(st)), ap = smem_u32(lop(grp));
+      uint64_t dp2 = 0;
 #pragma unroll
-      for (int c = 4 * h; c < 4 * h + 4; ++c) {
-        uint4* pq = reinterpret_cast<uint4*>(stq(st) + swz(r, c));
-        float f[8];
-        phi8(*pq, valid, f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dpart = fmaf(f[e], zs[c * 8 + e], dpart);
-        uint4 hi, lo;
-        split8(f, hi, lo);
-        *pq = hi;
-        *reinterpret_cast<uint4*>(stpl(st) + swz(r, c)) = lo;
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t off = swz(r, 4 * h + c);
+        const uint4 u = ld_shared_v4(aq + off), za = ld_shared_v4(zaddr + c * 32), zb = ld_shared_v4(zaddr + c * 32 + 16);
+        const uint64_t f0 = phi_pair(u.x), f1 = phi_pair(u.y), f2 = phi_pair(u.z), f3 = phi_pair(u.w);
+        dp2 = ffma2(f0, u2pack(za.x, za.y), dp2);
+        dp2 = ffma2(f1, u2pack(za.z, za.w), dp2);
+        dp2 = ffma2(f2, u2pack(zb.x, zb.y), dp2);
+        dp2 = ffma2(f3, u2pack(zb.z, zb.w), dp2);
+        uint32_t hi[4], lo[4];
+        split_pair(f0, hi[0], lo[0]);
+        split_pair(f1, hi[1], lo[1]);
+        split_pair(f2, hi[2], lo[2]);
+        split_pair(f3, hi[3], lo[3]);
+        st_shared_v4(aq + off, hi[0], hi[1], hi[2], hi[3]);
+        st_shared_v4(ap + off, lo[0], lo[1], lo[2], lo[3]);
       }
-      xden[h * 128 + r] = dpart;
+      float d0, d1;
+      f2unpack(dp2, d0, d1);
+      xden[h * 128 + r] = d0 + d1;
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
       const float den = xden[r] + xden[128 + r];
       const float inv = valid ? 1.f / den : 0.f;
       // this half of the U row (the U product is done: the g tile may be overwritten below)
-      if (!(ok = LWAIT(ufull + b, n & 1))) break;
+      if (!(ok = LWAIT(ufull + grp, n & 1))) break;
       tc_fence_after();
-      uint32_t u[32];
-      const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + 64 * b + 32 * h;
-      tmem_ld32(tl, u);
-      tmem_wait_ld(u);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(ufree + b);
-      float gpart = 0.f;
+      // phi(q) again from its parts, eight columns of a chunk at a time
+      auto phi_parts = [&](int c, uint64_t (&f)[4]) {
+        const uint32_t off = swz(r, 4 * h + c);
+        const uint4 hi = ld_shared_v4(aq + off), lo = ld_shared_v4(ap + off);
+        f[0] = fadd2(u2pack(hi.x << 16, hi.x & 0xffff0000u), u2pack(lo.x << 16, lo.x & 0xffff0000u));
+        f[1] = fadd2(u2pack(hi.y << 16, hi.y & 0xffff0000u), u2pack(lo.y << 16, lo.y & 0xffff0000u));
+        f[2] = fadd2(u2pack(hi.z << 16, hi.z & 0xffff0000u), u2pack(lo.z << 16, lo.z & 0xffff0000u));
+        f[3] = fadd2(u2pack(hi.w << 16, hi.w & 0xffff0000u), u2pack(lo.w << 16, lo.w & 0xffff0000u));
+      };
+      uint64_t gp2 = 0;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float f[8];
-        join8(*reinterpret_cast<const uint4*>(stq(st) + swz(r, 4 * h + c)),
-              *reinterpret_cast<const uint4*>(stpl(st) + swz(r, 4 * h + c)), f);
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t u[16];
+        tmem_ld16(tl + 16 * hh, u);
+        tmem_wait_ld(u);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) gpart = fmaf(f[e], __uint_as_float(u[8 * c + e]), gpart);
+        for (int c = 0; c < 2; ++c) {
+          uint64_t f[4];
+          phi_parts(2 * hh + c, f);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) gp2 = ffma2(f[e], u2pack(u[8 * c + 2 * e], u[8 * c + 2 * e + 1]), gp2);
+        }
       }
-      xgo[h * 128 + r] = gpart;
+      f2unpack(gp2, d0, d1);
+      xgo[h * 128 + r] = d0 + d1;
+      if (lane == 0) bulk_wait_read();  // the previous dq store has read this warp's staging block
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
       const float go = (xgo[r] + xgo[128 + r]) * inv;
       // dq = (U - z go) / den * phi'(q); dz -= phi(q) go / den
-      __nv_bfloat16* dst = a.dq + ((size_t)bh * a.N + (size_t)t * kTile + r) * kD;
+      const uint64_t ngo2 = f2pack(-go, -go), inv2 = f2pack(inv, inv), ngi2 = f2pack(-(go * inv), -(go * inv));
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t u[16];
+        tmem_ld16(tl + 16 * hh, u);
+        tmem_wait_ld(u);
+        if (hh == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(ufree + grp);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int cc = 2 * hh + c;
+          uint64_t f[4];
+          phi_parts(cc, f);
+          const uint4 za = ld_shared_v4(zaddr + cc * 32), zb = ld_shared_v4(zaddr + cc * 32 + 16);
+          const uint64_t z[4] = {u2pack(za.x, za.y), u2pack(za.z, za.w), u2pack(zb.x, zb.y), u2pack(zb.z, zb.w)};
+          uint32_t pk[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float f0, f1;
+            f2unpack(f[e], f0, f1);
+            const uint64_t t = fmul2(ffma2(z[e], ngo2, u2pack(u[8 * c + 2 * e], u[8 * c + 2 * e + 1])), inv2);
+            f2unpack(fmul2(t, f2pack(fmin_nan(f0, 1.f), fmin_nan(f1, 1.f))), f0, f1);
+            pk[e] = pack_bf16(f0, f1);
+            dz[4 * cc + e] = ffma2(f[e], ngi2, dz[4 * cc + e]);
+          }
+          st_shared_v4(out + lane * 64 + ((cc ^ ((lane >> 1) & 3)) << 4), pk[0], pk[1], pk[2], pk[3]);
+        }
+      }
+      // g / den: hi over the g tile, lo in the low tile
+      const uint32_t ag = smem_u32(stg(st)), al = smem_u32(glo(grp));
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const int cc = 4 * h + c;
-        float f[8];
-        join8(*reinterpret_cast<const uint4*>(stq(st) + swz(r, cc)), *reinterpret_cast<const uint4*>(stpl(st) + swz(r, cc)),
-              f);
-        uint32_t pk[4];
+        const uint32_t off = swz(r, 4 * h + c);
+        const uint4 u = ld_shared_v4(ag + off);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+        uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-          const float d0 = (__uint_as_float(u[8 * c + e]) - zs[cc * 8 + e] * go) * inv * (f[e] > 1.f ? 1.f : f[e]);
-          const float d1 =
-              (__uint_as_float(u[8 * c + e + 1]) - zs[cc * 8 + e + 1] * go) * inv * (f[e + 1] > 1.f ? 1.f : f[e + 1]);
-          pk[e >> 1] = pack_bf16(d0, d1);
-          dz[c * 8 + e] = fmaf(-f[e], go * inv, dz[c * 8 + e]);
-          dz[c * 8 + e + 1] = fmaf(-f[e + 1], go * inv, dz[c * 8 + e + 1]);
-        }
-        if (valid) *reinterpret_cast<uint4*>(dst + cc * 8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        for (int e = 0; e < 4; ++e) split_pair(fmul2(u2pack(w[e] << 16, w[e] & 0xffff0000u), inv2), hi[e], lo[e]);
+        st_shared_v4(ag + off, hi[0], hi[1], hi[2], hi[3]);
+        st_shared_v4(al + off, lo[0], lo[1], lo[2], lo[3]);
       }
-      // g / den: hi over the g tile, lo in its own tile
-#pragma unroll
-      for (int c = 4 * h; c < 4 * h + 4; ++c) {
-        uint4* pg = reinterpret_cast<uint4*>(stg(st) + swz(r, c));
-        const uint4 uu = *pg;
-        const uint32_t w[4] = {uu.x, uu.y, uu.z, uu.w};
-        float f[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          f[2 * i] = __uint_as_float(w[i] << 16) * inv;
-          f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u) * inv;
-        }
-        uint4 hi, lo;
-        split8(f, hi, lo);
-        *pg = hi;
-        *reinterpret_cast<uint4*>(stgl(st) + swz(r, c)) = lo;
-      }
-      fence_proxy_async_smem();  // the tensor core reads what these threads wrote
+      fence_proxy_async_smem();  // the tensor core and the copy unit read what these threads wrote
       __syncwarp();
-      if (lane == 0) mbar_arrive(dsready + st);
+      if (lane == 0) {
+        mbar_arrive(dsready + grp);
+        tma_store_5d(&tdq, out, 32 * h, (t0 + G) * kTile + quad * 32, 0, 0, bh);
+        bulk_commit();
+      }
     }
     // epilogue: dS partial (M = 64: rows 16q .. 16q+15 in lanes 0..15 of lane
-    // quadrant q; this warp's 32 of the 64 columns) and dz reduced over the
-    // 128 rows in fixed order
+    // quadrant q; group 0's warps, 32 of the 64 columns each) and dz reduced
+    // over both groups' 128 rows in fixed order
     const bool got = ok && LWAIT(done, 0);
     tc_fence_after();
-    uint32_t s0[32];
-    const uint32_t tq4 = tmem + ((uint32_t)(quad * 32) << 16) + 128 + 32 * h;
-    tmem_ld32(tq4, s0);
-    tmem_wait_ld(s0);
     const size_t part = (size_t)chunk * a.BH + bh;
-    if (got && lane < 16) {
-      float* dst = a.part_dS + (part * kD + quad * 16 + lane) * kD + 32 * h;
+    if (grp == 0) {
+      uint32_t s0[32];
+      const uint32_t tq4 = tmem + ((uint32_t)(quad * 32) << 16) + 128 + 32 * h;
+      tmem_ld32(tq4, s0);
+      tmem_wait_ld(s0);
+      if (got && lane < 16) {
+        float* dst = a.part_dS + (part * kD + quad * 16 + lane) * kD + 32 * h;
 #pragma unroll
-      for (int j = 0; j < 32; j += 4)
-        *reinterpret_cast<float4*>(dst + j) = make_float4(__uint_as_float(s0[j]), __uint_as_float(s0[j + 1]),
-                                                          __uint_as_float(s0[j + 2]), __uint_as_float(s0[j + 3]));
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(dst + j) = make_float4(__uint_as_float(s0[j]), __uint_as_float(s0[j + 1]),
+                                                            __uint_as_float(s0[j + 2]), __uint_as_float(s0[j + 3]));
+      }
     }
-    // the stages are idle once `done` completed: reuse them for the dz rows
-    float* zbuf = reinterpret_cast<float*>(smem + kBQBase);
+    // the low tiles are idle once `done` completed: reuse them for the dz rows
+    float* zbuf = reinterpret_cast<float*>(smem + kBQLo);
     if (got) {
 #pragma unroll
-      for (int i = 0; i < kD / 2; ++i) zbuf[r * kD + 32 * h + i] = dz[i];
+      for (int i = 0; i < kD / 4; ++i) {
+        float x, y;
+        f2unpack(dz[i], x, y);
+        *reinterpret_cast<float2*>(zbuf + (grp * kTile + r) * kD + 32 * h + 2 * i) = make_float2(x, y);
+      }
     }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
+    asm volatile("bar.sync 1, 512;" ::: "memory");
     if (got && tid < kD) {
       float sum = 0.f;
-      for (int i = 0; i < kTile; ++i) sum += zbuf[i * kD + tid];
+      for (int i = 0; i < 2 * kTile; ++i) sum += zbuf[i * kD + tid];
       a.part_dz[part * kD + tid] = sum;
     }
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -834,18 +907,23 @@ struct BKArgs {
 };
 
 // Key pass, grid (ceil(ntiles / tiles_per_cta), BH): per 128-token key tile
-// (k and v by TMA through two stages)
-//   math:   phi(k)'s parts (hi over the k tile, lo in its own tile)
+// (k and v by TMA through four stages), tile t going to math group t & 1
+//   math:   phi(k)'s parts (hi over the k tile, lo in the group's low tile)
 //   issuer: P1 = V dS^T (A = v tile, B = dS rows; hi and lo) and P2 = phi(K) dS
 //           (A = phi parts, B = dS^T rows; chains hi.hi, hi.lo, lo.hi), into
-//           one of two TMEM buffer pairs
-//   math:   dk = (P1 + dz) * phi'(k), dv = P2, stored row by row
-// A stage is released by the issuer's commit and the eight math warps together
-// (phi' is recomputed from phi's parts in the epilogue).  Two math warps per
-// TMEM lane quadrant, each taking 32 of a row's 64 columns (nothing here sums
-// over a row).
+//           the group's TMEM buffers
+//   math:   dk = (P1 + dz) * phi'(k) over the k tile, dv = P2 over the v tile
+//           (the products have read both), 32 rows of each stored by TMA per
+//           lane quadrant (rows past N are dropped)
+// A stage is released by the four quadrants once their stores have read it.
+// Two math warps per group and TMEM lane quadrant, each taking 32 of a row's
+// 64 columns (nothing here sums over a row).  16 heads of 262144 tokens:
+// 713 -> 406 us (one group of eight warps, a thread storing its own 64
+// bytes of a row, before).
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_constant__ CUtensorMap tk,
                                                                   const __grid_constant__ CUtensorMap tv,
+                                                                  const __grid_constant__ CUtensorMap tdk,
+                                                                  const __grid_constant__ CUtensorMap tdv,
                                                                   const BKArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -854,36 +932,43 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
   uint8_t* mTh = smem + 16384;  // dS^T rows (v), hi
   uint8_t* mTl = smem + 24576;  // dS^T rows, lo
   float* dzs = reinterpret_cast<float*>(smem + 32768);
-  auto stk = [&](int st) { return smem + kBKBase + st * kBKStage; };  // k, then phi hi
-  auto stv = [&](int st) { return stk(st) + kTileBytes; };
-  auto stpl = [&](int st) { return stk(st) + 2 * kTileBytes; };        // phi lo
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBKBase + kBKStages * kBKStage);
+  auto stk = [&](int st) { return smem + kBKRaw + st * 2 * kTileBytes; };  // k, then phi hi, then dk
+  auto stv = [&](int st) { return stk(st) + kTileBytes; };                 // v, then dv
+  auto lop = [&](int grp) { return smem + kBKLo + grp * kTileBytes; };     // phi lo
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBKBar);
   uint64_t* empty = full + kBKStages;
-  uint64_t* kready = empty + kBKStages;
-  uint64_t* pfull = kready + kBKStages;
-  uint64_t* pfree = pfull + kBKStages;
-  uint64_t* sready = pfree + kBKStages;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sready + 1);
+  uint64_t* kready = empty + kBKStages;  // [group]
+  uint64_t* pfull = kready + 2;          // [group]
+  uint64_t* pfree = pfull + 2;           // [group]
+  uint64_t* sready = pfree + 2;
+  uint64_t* done = sready + 1;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.y;
   const int t0 = blockIdx.x * a.tiles_per_cta, t1 = min(a.ntiles, t0 + a.tiles_per_cta);
+  const int count = t1 - t0;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kBKStages; ++i) {
       mbar_init(full + i, 1);
-      mbar_init(empty + i, 9);  // the issuer's commit and the eight math warps
+      mbar_init(empty + i, 4);  // the lane quadrants of the tile's group
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(kready + i, 8);
       mbar_init(pfull + i, 1);
       mbar_init(pfree + i, 8);
     }
-    mbar_init(sready, 8);
+    mbar_init(sready, 16);
+    mbar_init(done, 1);
     *abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tk);
     prefetch_tmap(&tv);
+    prefetch_tmap(&tdk);
+    prefetch_tmap(&tdv);
   }
   if (warp == 1) {
-    tmem_alloc(tslot, 256);  // buffer b: P1 at 128 b, P2 at 128 b + 64
+    tmem_alloc(tslot, 256);  // group b: P1 at 128 b, P2 at 128 b + 64
     tmem_relinquish();
   }
   tc_fence_before();
@@ -895,14 +980,14 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
     if (lane == 0) {  // ------------------------------------------------ TMA producer
       uint32_t armed = 0, par = 0;
       bool ok = true;
-      for (int t = t0, G = 0; t < t1; ++t, ++G) {
+      for (int G = 0; G < count; ++G) {
         const int st = G % kBKStages, n = G / kBKStages;
         if (!(ok = LWAIT(empty + st, (n & 1) ^ 1))) break;
         mbar_arrive_expect_tx(full + st, 2 * kTileBytes);
         armed |= 1u << st;
         par = (par & ~(1u << st)) | ((n & 1) << st);
-        tma_load_5d(stk(st), &tk, full + st, 0, t * kTile, 0, 0, bh);
-        tma_load_5d(stv(st), &tv, full + st, 0, t * kTile, 0, 0, bh);
+        tma_load_5d(stk(st), &tk, full + st, 0, (t0 + G) * kTile, 0, 0, bh);
+        tma_load_5d(stv(st), &tv, full + st, 0, (t0 + G) * kTile, 0, 0, bh);
       }
       if (!ok)
         for (int s2 = 0; s2 < kBKStages; ++s2)
@@ -914,19 +999,21 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
       const uint64_t bDh = sw128_desc(smem_u32(mDh), 16, 1024), bDl = sw128_desc(smem_u32(mDl), 16, 1024);
       const uint64_t bTh = sw128_desc(smem_u32(mTh), 16, 1024), bTl = sw128_desc(smem_u32(mTl), 16, 1024);
       bool ok = LWAIT(sready, 0);
-      for (int t = t0, G = 0; t < t1 && ok; ++t, ++G) {
-        const int st = G % kBKStages, n = G / kBKStages, b = G & 1;
-        if (!(ok = LWAIT(full + st, n & 1))) break;
-        if (!(ok = LWAIT(kready + st, n & 1))) break;
+      for (int G = 0; G < count && ok; ++G) {
+        const int st = G % kBKStages, b = G & 1;
+        if (!(ok = LWAIT(full + st, (G / kBKStages) & 1))) break;
         if (G >= 2 && !(ok = LWAIT(pfree + b, ((G >> 1) - 1) & 1))) break;
         tc_fence_after();
         const uint32_t tP1 = tmem + 128 * b, tP2 = tP1 + 64;
         const uint64_t aV = sw128_desc(smem_u32(stv(st)), 16, 1024);
-        const uint64_t aH = sw128_desc(smem_u32(stk(st)), 16, 1024), aL = sw128_desc(smem_u32(stpl(st)), 16, 1024);
+        const uint64_t aH = sw128_desc(smem_u32(stk(st)), 16, 1024), aL = sw128_desc(smem_u32(lop(b)), 16, 1024);
+        // P1 needs only v: it runs while phi is formed
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) umma_bf16(tP1, dmove(aV, ks * 32), dmove(bDh, ks * 32), idP, ks > 0);
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) umma_bf16(tP1, dmove(aV, ks * 32), dmove(bDl, ks * 32), idP, 1u);
+        if (!(ok = LWAIT(kready + b, (G >> 1) & 1))) break;
+        tc_fence_after();
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) umma_bf16(tP2, dmove(aH, ks * 32), dmove(bTh, ks * 32), idP, ks > 0);
 #pragma unroll
@@ -934,80 +1021,103 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) umma_bf16(tP2, dmove(aL, ks * 32), dmove(bTh, ks * 32), idP, 1u);
         umma_commit(pfull + b);
-        umma_commit(empty + st);
       }
+      umma_commit(done);
       if (!ok) *abort_flag = 1;
+      mbar_wait<set_status_l>(done, 0, abort_flag, false);  // before tensor memory is released
     }
   } else {
     // ------------------------------------------------------------------ math warps
     const int quad = warp & 3;
-    const int h = (warp - 2) >> 2;  // columns [32 h, 32 h + 32) of the row: chunks 4 h .. 4 h + 3
+    const int grp = (warp - 2) >> 3;
+    const int h = ((warp - 2) >> 2) & 1;  // columns [32 h, 32 h + 32) of the row: chunks 4 h .. 4 h + 3
     const int r = quad * 32 + lane;
     const int tid = threadIdx.x - 64;
+    const int pair_bar = 2 + grp * 4 + quad;  // named barrier of the two warps of this group and lane quadrant
     {
       const size_t m = (size_t)bh * kD * kD;
       const __nv_bfloat16* src[4] = {a.dsh + m, a.dsl + m, a.dsth + m, a.dstl + m};
       uint8_t* dst[4] = {mDh, mDl, mTh, mTl};
-      load_mats(tid, 256, 4, src, dst);
+      load_mats(tid, 512, 4, src, dst);
       if (tid < kD) dzs[tid] = a.dz[(size_t)bh * kD + tid];
       fence_proxy_async_smem();
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      asm volatile("bar.sync 1, 512;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(sready);
     }
-    bool ok = true;
-    for (int t = t0, G = 0; t < t1; ++t, ++G) {
-      const int st = G % kBKStages, n = G / kBKStages, b = G & 1;
-      const bool valid = (int64_t)t * kTile + r < a.N;
-      if (!(ok = LWAIT(full + st, n & 1))) break;
+    const uint32_t zaddr = smem_u32(dzs) + h * 128;
+    const uint32_t al = smem_u32(lop(grp));
+    const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + 128 * grp + 32 * h;
+    const bool storer = h == 0 && lane == 0;  // stores its quadrant's rows
+    for (int G = grp, n = 0; G < count; G += 2, ++n) {
+      const int st = G % kBKStages;
+      if (n > 0 && storer) {  // the previous tile's stores have read their stage
+        bulk_wait_read();
+        mbar_arrive(empty + (G - 2) % kBKStages);
+      }
+      if (!LWAIT(full + st, (G / kBKStages) & 1)) break;
+      const uint32_t ak = smem_u32(stk(st)), av = smem_u32(stv(st));
+      uint64_t f[16];
 #pragma unroll
-      for (int c = 4 * h; c < 4 * h + 4; ++c) {
-        uint4* pk = reinterpret_cast<uint4*>(stk(st) + swz(r, c));
-        float f[8];
-        phi8(*pk, true, f);
-        uint4 hi, lo;
-        split8(f, hi, lo);
-        *pk = hi;
-        *reinterpret_cast<uint4*>(stpl(st) + swz(r, c)) = lo;
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t off = swz(r, 4 * h + c);
+        const uint4 u = ld_shared_v4(ak + off);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          f[4 * c + e] = phi_pair(w[e]);
+          split_pair(f[4 * c + e], hi[e], lo[e]);
+        }
+        st_shared_v4(ak + off, hi[0], hi[1], hi[2], hi[3]);
+        st_shared_v4(al + off, lo[0], lo[1], lo[2], lo[3]);
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(kready + st);
-      if (!(ok = LWAIT(pfull + b, n & 1))) break;
+      if (lane == 0) mbar_arrive(kready + grp);
+      if (!LWAIT(pfull + grp, n & 1)) break;
       tc_fence_after();
-      uint32_t p1[32], p2[32];
-      const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + 128 * b + 32 * h;
-      tmem_ld32(tl, p1);
-      tmem_ld32(tl + 64, p2);
-      tmem_wait_ld(p1);
-      tmem_wait_ld(p2);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(pfree + b);
-      const size_t row = ((size_t)bh * a.N + (size_t)t * kTile + r) * kD;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int cc = 4 * h + c;
-        float f[8];
-        join8(*reinterpret_cast<const uint4*>(stk(st) + swz(r, cc)), *reinterpret_cast<const uint4*>(stpl(st) + swz(r, cc)),
-              f);
-        uint32_t ok4[4], ov4[4];
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-          const float k0 = (__uint_as_float(p1[8 * c + e]) + dzs[cc * 8 + e]) * (f[e] > 1.f ? 1.f : f[e]);
-          const float k1 = (__uint_as_float(p1[8 * c + e + 1]) + dzs[cc * 8 + e + 1]) * (f[e + 1] > 1.f ? 1.f : f[e + 1]);
-          ok4[e >> 1] = pack_bf16(k0, k1);
-          ov4[e >> 1] = pack_bf16(__uint_as_float(p2[8 * c + e]), __uint_as_float(p2[8 * c + e + 1]));
+      for (int hh = 0; hh < 2; ++hh) {
+        uint32_t p1[16], p2[16];
+        tmem_ld16(tl + 16 * hh, p1);
+        tmem_ld16(tl + 64 + 16 * hh, p2);
+        tmem_wait_ld(p1);
+        tmem_wait_ld(p2);
+        if (hh == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(pfree + grp);
         }
-        if (valid) {
-          *reinterpret_cast<uint4*>(a.dk + row + cc * 8) = make_uint4(ok4[0], ok4[1], ok4[2], ok4[3]);
-          *reinterpret_cast<uint4*>(a.dv + row + cc * 8) = make_uint4(ov4[0], ov4[1], ov4[2], ov4[3]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int cc = 2 * hh + c;
+          const uint4 za = ld_shared_v4(zaddr + cc * 32), zb = ld_shared_v4(zaddr + cc * 32 + 16);
+          const uint64_t z[4] = {u2pack(za.x, za.y), u2pack(za.z, za.w), u2pack(zb.x, zb.y), u2pack(zb.z, zb.w)};
+          uint32_t ok4[4], ov4[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float f0, f1;
+            f2unpack(f[4 * cc + e], f0, f1);
+            const uint64_t t = fadd2(u2pack(p1[8 * c + 2 * e], p1[8 * c + 2 * e + 1]), z[e]);
+            f2unpack(fmul2(t, f2pack(fmin_nan(f0, 1.f), fmin_nan(f1, 1.f))), f0, f1);
+            ok4[e] = pack_bf16(f0, f1);
+            ov4[e] = pack_bf16(__uint_as_float(p2[8 * c + 2 * e]), __uint_as_float(p2[8 * c + 2 * e + 1]));
+          }
+          const uint32_t off = swz(r, 4 * h + cc);
+          st_shared_v4(ak + off, ok4[0], ok4[1], ok4[2], ok4[3]);
+          st_shared_v4(av + off, ov4[0], ov4[1], ov4[2], ov4[3]);
         }
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty + st);  // phi's parts read: the stage may be refilled
+      fence_proxy_async_smem();  // the copy unit reads what these threads wrote
+      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+      if (storer) {
+        tma_store_5d(&tdk, ak + quad * 4096, 0, (t0 + G) * kTile + quad * 32, 0, 0, bh);
+        tma_store_5d(&tdv, av + quad * 4096, 0, (t0 + G) * kTile + quad * 32, 0, 0, bh);
+        bulk_commit();
+      }
     }
-    (void)ok;
+    if (storer) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -1165,9 +1275,11 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   ka.dk = static_cast<__nv_bfloat16*>(dk);
   ka.dv = static_cast<__nv_bfloat16*>(dv);
 
-  CUtensorMap mq, mg, mk, mv;
+  CUtensorMap mq, mg, mk, mv, mdq, mdk, mdv;
   if (!make_tmap_5d(&mq, q, kD, (int)N, 1, 1, BH, kTile, 1, 1) || !make_tmap_5d(&mg, dout, kD, (int)N, 1, 1, BH, kTile, 1, 1) ||
-      !make_tmap_5d(&mk, k, kD, (int)N, 1, 1, BH, kTile, 1, 1) || !make_tmap_5d(&mv, v, kD, (int)N, 1, 1, BH, kTile, 1, 1))
+      !make_tmap_5d(&mk, k, kD, (int)N, 1, 1, BH, kTile, 1, 1) || !make_tmap_5d(&mv, v, kD, (int)N, 1, 1, BH, kTile, 1, 1) ||
+      !make_tmap_5d(&mdq, dq, kD, (int)N, 1, 1, BH, 32, 1, 1, 32) || !make_tmap_5d(&mdk, dk, kD, (int)N, 1, 1, BH, 32, 1, 1) ||
+      !make_tmap_5d(&mdv, dv, kD, (int)N, 1, 1, BH, 32, 1, 1))
     return cudaErrorInvalidValue;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(la_bwd_query_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBQSmem)) !=
@@ -1176,7 +1288,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
           cudaSuccess)
     return e;
   prof_begin(kKLinearBwdQuery, st);
-  la_bwd_query_kernel<<<dim3(p.chunks, BH), kThreadsB, kBQSmem, st>>>(mq, mg, qa);
+  la_bwd_query_kernel<<<dim3(p.chunks, BH), kThreadsB, kBQSmem, st>>>(mq, mg, mdq, qa);
   e = cudaGetLastError();
   prof_end(kKLinearBwdQuery, st);
   if (e != cudaSuccess) return e;
@@ -1187,7 +1299,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   if (e != cudaSuccess) return e;
   prof_begin(kKLinearBwdKey, st);
   la_bwd_key_kernel<<<dim3((p.ntiles + p.q_tiles_per_cta - 1) / p.q_tiles_per_cta, BH), kThreadsB, kBKSmem, st>>>(
-      mk, mv, ka);
+      mk, mv, mdk, mdv, ka);
   e = cudaGetLastError();
   prof_end(kKLinearBwdKey, st);
   return e;

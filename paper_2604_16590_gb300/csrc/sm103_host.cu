@@ -26,16 +26,18 @@ EncodeFn encode_fn() {
 }
 }  // namespace
 
-bool make_tmap_5d(CUtensorMap* map, const void* base, int d, int X, int Y, int T, int BH, int bx, int by, int bt) {
+bool make_tmap_5d(CUtensorMap* map, const void* base, int d, int X, int Y, int T, int BH, int bx, int by, int bt,
+                  int cols) {
   EncodeFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[5] = {(cuuint64_t)d, (cuuint64_t)X, (cuuint64_t)Y, (cuuint64_t)T, (cuuint64_t)BH};
   const cuuint64_t row = (cuuint64_t)d * 2;
   const cuuint64_t strides[4] = {row, row * X, row * X * Y, row * X * Y * T};
-  const cuuint32_t box[5] = {64u, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bt, 1u};
+  const cuuint32_t box[5] = {(cuuint32_t)cols, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bt, 1u};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }

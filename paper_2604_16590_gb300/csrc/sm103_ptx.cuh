@@ -369,6 +369,17 @@ __device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+// minimum and maximum that return NaN if either operand is NaN
+__device__ __forceinline__ float fmin_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
@@ -382,8 +393,10 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
 }  // namespace sm103
 
 // Host: 5-D tiled tensor map over a [BH, T, Y, X, d] BF16 tensor (d innermost),
-// box (64, bx, by, bt, 1), 128-byte swizzle, zero fill out of range.
-bool make_tmap_5d(CUtensorMap* map, const void* base, int d, int X, int Y, int T, int BH, int bx, int by, int bt);
+// box (cols, bx, by, bt, 1), 128-byte swizzle (cols = 64) or 64-byte swizzle
+// (cols = 32), zero fill out of range.
+bool make_tmap_5d(CUtensorMap* map, const void* base, int d, int X, int Y, int T, int BH, int bx, int by, int bt,
+                  int cols = 64);
 
 // Host: 2-D tiled tensor map over `rows` FP32 rows of d columns (the per-tile
 // slots), box of 32 rows x `cols` columns: 32 (128-byte swizzle) or 16 (64-byte
