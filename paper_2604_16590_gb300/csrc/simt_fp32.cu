@@ -21,7 +21,7 @@
 // locally before it is folded into the running sums (two-level summation,
 // which keeps the FP32 error of L-long sums near eps * (sqrt(64) + sqrt(L/64))).
 // Bound: the FP32 pipe (128 lanes a clock and SM).  4 heads of a 4 x 64 x 128
-// clip in 16 tiles of up to 4608 tokens, d = 64: forward 14.6 -> 7.4 ms, dQ
+// clip in 16 tiles of up to 4608 tokens, d = 64: forward 14.6 -> 7.1 ms, dQ
 // 17.0 -> 9.3, dK/dV 19.4 -> 12.4 (before: a thread group per row, one FMA per
 // shared-memory word).
 #include "internal.cuh"
@@ -101,14 +101,20 @@ __device__ __forceinline__ void dots(const float* __restrict__ rows, const float
     ulonglong2 b[S::KT];
 #pragma unroll
     for (int j = 0; j < S::KT; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(cp + j * S::LG * S::LD + k);
+    // four rows at a time: an accumulator's two updates are 4 KT instructions apart
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(rows + i * S::LD + k);
+    for (int i0 = 0; i0 < 8; i0 += 4) {
+      ulonglong2 a[4];
 #pragma unroll
-      for (int j = 0; j < S::KT; ++j) {
-        acc[i][j] = ffma2(a.x, b[j].x, acc[i][j]);
-        acc[i][j] = ffma2(a.y, b[j].y, acc[i][j]);
-      }
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(rows + (i0 + i) * S::LD + k);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < S::KT; ++j) acc[i0 + i][j] = ffma2(a[i].x, b[j].x, acc[i0 + i][j]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < S::KT; ++j) acc[i0 + i][j] = ffma2(a[i].y, b[j].y, acc[i0 + i][j]);
     }
   }
 #pragma unroll
