@@ -62,13 +62,14 @@ __device__ void set_status_f64(uint32_t c) { set_status(c); }
 
 constexpr int kD = 64;
 constexpr int kBox = 128 * kD * 2;  // one 128-token box of one operand, BF16, 16 KB
-constexpr int kStages = 4;          // K/V ring depth
 constexpr int kSoft0 = 4;           // first softmax warp
 constexpr int kThreadsF = 384;
 constexpr uint32_t kRegsLow = 72, kRegsHigh = 216;  // 128 x 72 + 256 x 216 = 384 x 168
 constexpr float kRescaleLog2 = 8.f;
 
+template <bool RAGGED>
 struct Cfg {
+  static constexpr int kStages = RAGGED ? 4 : 3;  // K/V ring depth: the staged outputs take a stage
   // two Q buffers (items alternate): buffer b holds Q_A at kQ + 2 b kBox, Q_B after it
   static constexpr int kQ = 0;
   static constexpr int kK = 4 * kBox;
@@ -77,14 +78,17 @@ struct Cfg {
   // then 2 KB of zeros for K-columns 8..15): the A operand has 1 in K-column 0
   // of every row; stage s of the B operand holds the key block's bias
   // (0 for a key of the tile, -1e30 for a padding row or a key outside it).
-  static constexpr int kOnes = kV + kStages * kBox;
+  static constexpr int kOut = kV + kStages * kBox;  // staged output columns 32..63, 4 KB per softmax warp
+  static constexpr int kOnes = kOut + (RAGGED ? 0 : 2 * kBox);
   static constexpr int kBias = kOnes + 4096;
   static constexpr int kBar = kBias + kStages * 4096;
   // q_full[2], q_empty[2], k_full[S], k_empty[S], v_full[S], v_empty[S],
   // per box: s_full, s_empty, p_full, p_empty, o_full, o_empty; drain[2], never
   static constexpr int kNumBars = 4 + 4 * kStages + 2 * 6 + 3;
   static constexpr int kMisc = kBar + kNumBars * 8;
-  static constexpr int kSmem = kMisc + 16 + 1024;
+  static constexpr int kGeom = kMisc + 16;  // ragged mode: one geometry per warp
+  static constexpr int kSmem = kGeom + (RAGGED ? (kThreadsF / 32) * (int)sizeof(Geom) : 0) + 1024;
+  static_assert(kGeom % 8 == 0, "the geometries are copied in 8-byte words");
 };
 __device__ __forceinline__ uint32_t col_s(int x) { return 128u * x; }
 __device__ __forceinline__ uint32_t col_p(int x) { return 256u + 64u * x; }
@@ -94,7 +98,6 @@ struct Fwd64Args {
   Geom g;
   void* out;
   float* lse2;
-  float* ot;
   int items;  // B*nh * ntiles * box pairs
   uint32_t flags;
   int pad_R;  // box rows of every geometry of the launch (rows pad_R..127 of each block are zeroed once)
@@ -111,41 +114,62 @@ struct Item {
   const CUtensorMap* tv;
   void* out;
   float* lse2;  // may be null (no backward)
-  float* ot;
+  float* ot;    // ragged mode (else the slots' tensor map serves)
   int bh, tile, pair;
   int req;  // request index (ragged mode), else -1
 };
 
 inline int box_pairs(const Geom& g) { return (int)g.fpairs.d; }
 
+// Ragged mode: the request that a warp's current item belongs to.  The search
+// runs, and the request's geometry is copied into the warp's own block of
+// shared memory, only when the item leaves the request's range: reading the
+// geometry field by field from the descriptor table put a chain of global
+// loads into every item of every role.
+struct ReqCache {
+  int req = -1, item0 = 0, item1 = 0;
+  Geom* g = nullptr;  // the warp's block
+};
+
 // Returns false (after recording GATTN_ERR_DEVICE_BOUNDS) if a ragged work item
 // does not decode to a valid (request, head, tile, pair); every role decodes
-// the same item identically, so all of them skip it together.
-template <bool RAGGED>
+// the same item identically, so all of them skip it together.  SOLO: called by
+// one lane of the warp, else by all of them together.
+template <bool RAGGED, bool SOLO>
 __device__ __forceinline__ bool resolve(const Fwd64Args& a, const CUtensorMap* tq, const CUtensorMap* tk,
-                                        const CUtensorMap* tv, int w, Item& it) {
-  int req = -1;
+                                        const CUtensorMap* tv, int w, ReqCache& rc, Item& it) {
   if constexpr (RAGGED) {
-    // requests are sorted by item0: binary search for the last item0 <= w
-    const int nreq = (int)a.counts[0];
-    int lo = 0, hi = nreq - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.reqs[mid].item0 <= w) lo = mid;
-      else hi = mid - 1;
+    if (w < rc.item0 || w >= rc.item1) {
+      // requests are sorted by item0: binary search for the last item0 <= w
+      const int nreq = (int)a.counts[0];
+      int lo = 0, hi = nreq - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (a.reqs[mid].item0 <= w) lo = mid;
+        else hi = mid - 1;
+      }
+      if (nreq < 1 || w < a.reqs[lo].item0 || w >= a.reqs[lo].item0 + a.reqs[lo].items) {
+        set_status(kStatusBounds);
+        return false;
+      }
+      rc.req = lo;
+      rc.item0 = a.reqs[lo].item0;
+      rc.item1 = rc.item0 + a.reqs[lo].items;
+      static_assert(sizeof(Geom) % 8 == 0, "copied in 8-byte words");
+      const uint64_t* src = reinterpret_cast<const uint64_t*>(&a.reqs[lo].g);
+      uint64_t* dst = reinterpret_cast<uint64_t*>(rc.g);
+      if constexpr (!SOLO) __syncwarp();
+      for (int i = SOLO ? 0 : (threadIdx.x & 31); i < (int)(sizeof(Geom) / 8); i += SOLO ? 1 : 32) dst[i] = src[i];
+      if constexpr (!SOLO) __syncwarp();
     }
-    if (nreq < 1 || w < a.reqs[lo].item0 || w >= a.reqs[lo].item0 + a.reqs[lo].items) {
-      set_status(kStatusBounds);
-      return false;
-    }
-    req = lo;
-    const ReqDesc& r = a.reqs[lo];
-    it.g = &r.g;
+    const ReqDesc& r = a.reqs[rc.req];
+    it.g = rc.g;
     it.tq = it.tk = it.tv = &r.tmap;
     it.out = r.out;
     it.lse2 = nullptr;
     it.ot = r.ot;
-    w -= r.item0;
+    it.req = rc.req;
+    w -= rc.item0;
   } else {
     it.g = &a.g;
     it.tq = tq;
@@ -153,14 +177,14 @@ __device__ __forceinline__ bool resolve(const Fwd64Args& a, const CUtensorMap* t
     it.tv = tv;
     it.out = a.out;
     it.lse2 = a.lse2;
-    it.ot = a.ot;
+    it.ot = nullptr;
+    it.req = -1;
   }
   const Geom& g = *it.g;
   const int r = fdiv(w, g.fpairs);
   it.pair = w - r * (int)g.fpairs.d;
   it.bh = fdiv(r, g.fntiles);
   it.tile = r - it.bh * g.ntiles;
-  it.req = req;
   if (RAGGED && (it.bh >= g.B * g.nh || g.d != kD || g.R != a.pad_R)) {
     set_status(kStatusBounds);
     return false;
@@ -208,11 +232,35 @@ __device__ __forceinline__ void rescale_o(uint32_t tO, float f) {
   tmem_wait_st();
 }
 
+// one output row of 64 FP32 values in registers, 16 bytes at a time
+__device__ __forceinline__ void store_row(float* dst, const uint32_t (&r0)[32], const uint32_t (&r1)[32]) {
+#pragma unroll
+  for (int e = 0; e < 32; e += 4) {
+    *reinterpret_cast<uint4*>(dst + e) = make_uint4(r0[e], r0[e + 1], r0[e + 2], r0[e + 3]);
+    *reinterpret_cast<uint4*>(dst + 32 + e) = make_uint4(r1[e], r1[e + 1], r1[e + 2], r1[e + 3]);
+  }
+}
+__device__ __forceinline__ void store_row(__nv_bfloat16* dst, const uint32_t (&r0)[32], const uint32_t (&r1)[32]) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const uint32_t* r = c == 0 ? r0 : r1;
+#pragma unroll
+    for (int e = 0; e < 32; e += 8)
+      *reinterpret_cast<uint4*>(dst + 32 * c + e) =
+          make_uint4(pack_bf16(__uint_as_float(r[e]), __uint_as_float(r[e + 1])),
+                     pack_bf16(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])),
+                     pack_bf16(__uint_as_float(r[e + 4]), __uint_as_float(r[e + 5])),
+                     pack_bf16(__uint_as_float(r[e + 6]), __uint_as_float(r[e + 7])));
+  }
+}
+
 template <typename OutT, bool RAGGED>
 __global__ void __launch_bounds__(kThreadsF, 1)
     fwd64_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
-                 const __grid_constant__ CUtensorMap tv, const Fwd64Args a) {
-  using C = Cfg;
+                 const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap to,
+                 const Fwd64Args a) {
+  using C = Cfg<RAGGED>;
+  constexpr int kStages = C::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBar);
@@ -247,7 +295,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(q_full + b, 1);
-      mbar_init(q_empty + b, 1);
+      mbar_init(q_empty + b, RAGGED ? 1 : 1 + 8);  // the last score product; the softmax warps (staged outputs read)
     }
     for (int s = 0; s < kStages; ++s) {
       mbar_init(k_full + s, 2);  // the K load (producer) and the stage's bias row (mask writer)
@@ -272,6 +320,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       prefetch_tmap(&tq);
       prefetch_tmap(&tk);
       prefetch_tmap(&tv);
+      prefetch_tmap(&to);
     }
   }
   if (warp == 1) {
@@ -283,6 +332,8 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int n_items = RAGGED ? (int)a.counts[1] : a.items;
+  ReqCache rc;
+  if constexpr (RAGGED) rc.g = reinterpret_cast<Geom*>(smem + C::kGeom) + warp;
 
   if (warp < kSoft0) {
     setmaxnreg_dec<kRegsLow>();
@@ -294,7 +345,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       bool ok = true;
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
-        if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+        if (!resolve<RAGGED, true>(a, &tq, &tk, &tv, w, rc, it)) continue;
         const Geom& g = *it.g;
         const int bh = it.bh;
         TileBlocks tbk;
@@ -365,7 +416,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         ok = mbar_wait<set_status_f64>(never, 0, abort_flag, true, 20000000ull);
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
-        if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+        if (!resolve<RAGGED, true>(a, &tq, &tk, &tv, w, rc, it)) continue;
         const Geom& g = *it.g;
         TileBlocks tbk;
         tile_blocks(g, it.tile, tbk);
@@ -414,7 +465,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       bool ok = true;
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
-        if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+        if (!resolve<RAGGED, true>(a, &tq, &tk, &tv, w, rc, it)) continue;
         TileBlocks tbk;
         tile_blocks(*it.g, it.tile, tbk);
         const int qa = 2 * it.pair;
@@ -458,7 +509,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       bool ok = true;
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
-        if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+        if (!resolve<RAGGED, false>(a, &tq, &tk, &tv, w, rc, it)) continue;
         const Geom& g = *it.g;
         TileBlocks tbk;
         tile_blocks(g, it.tile, tbk);
@@ -492,26 +543,56 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     const int row = quad * 32 + lane;  // TMEM lane = query row of the box
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t tS = tl + col_s(x), tP = tl + col_p(x), tO = tl + col_o(x);
-    uint32_t GX = 0, WX = 0;
+    // this warp's staging blocks: 32 rows x 128 bytes of the output row's columns 0..31
+    // (its rows of the item's own Q block, which the score products are done with) and 32..63
+    const uint32_t st_q = smem_u32(smem + C::kQ) + x * kBox + quad * 4096;
+    const uint32_t st_o = smem_u32(smem + C::kOut) + (warp - kSoft0) * 4096;
+    uint32_t GX = 0, WX = 0, W = 0;
+    int staged = -1;  // Q buffer whose staged output may still be read by this warp's stores
     bool ok = true;
+    // the stores have read the staged rows: the Q buffer may be refilled
+    auto release_staged = [&]() {
+      if (staged >= 0 && lane == 0) {
+        bulk_wait_read();
+        mbar_arrive(q_empty + staged);
+      }
+      staged = -1;
+    };
     for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
       Item it;
-      if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+      if (!resolve<RAGGED, false>(a, &tq, &tk, &tv, w, rc, it)) continue;
       const Geom& g = *it.g;
       const int bh = it.bh, tile = it.tile;
       const float sl2 = g.scale_log2;
       const uint64_t s2 = f2pack(sl2, sl2);
       TileBlocks tbk;
-      tile_blocks(g, tile, tbk);
+      tile_blocks(g, it.tile, tbk);
       const int qa = 2 * it.pair;
-      if (qa + x >= tbk.NB) continue;
+      if (qa >= tbk.NB) continue;
+      const uint32_t buf = W & 1;
+      if (qa + x >= tbk.NB) {  // an item of one box: this warp only passes its Q buffer on
+        if constexpr (!RAGGED) {
+          release_staged();
+          if (!(ok = WAIT(q_full + buf, (W >> 1) & 1))) break;
+          if (lane == 0) mbar_arrive(q_empty + buf);
+          ++W;
+        }
+        continue;
+      }
+      const int nb = tbk.NB;
+      // ragged mode resolves the row's place before its key blocks and keeps it,
+      // the other mode resolves it again after them (see the epilogue)
       const int qb = qa + x;
-      int qo[3], ql[3];
-      block_origin(g, tbk, qb, qo);
-      block_row(g, qo, row, ql);
-      const bool qvalid = inside(tbk, ql);
+      int ql[3] = {0, 0, 0};
+      bool qvalid = false;
+      if constexpr (RAGGED) {
+        int qo[3];
+        block_origin(g, tbk, qb, qo);
+        block_row(g, qo, row, ql);
+        qvalid = inside(tbk, ql);
+      }
       float m = -INFINITY, l = 0.f, lc = 0.f;  // lc: Kahan compensation of the row sum l
-      for (int j = 0; j < tbk.NB; ++j, ++GX) {
+      for (int j = 0; j < nb; ++j, ++GX) {
         if (!(ok = WAIT(s_full(x), GX & 1))) break;
         tc_fence_after();
         // the row's 128 scores into registers, then S_x is released
@@ -586,46 +667,115 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(p_full(x));
+        if (!RAGGED && j == 0) release_staged();  // the previous item's stores have had this block's time
       }
       if (!ok) break;
-      // ---- epilogue: wait for the last P V, O / l
-      if (!(ok = WAIT(o_full(x), WX & 1))) break;
-      tc_fence_after();
-      ++WX;
-      const float inv = 1.f / l;
-      const int64_t slot = tile_slot0(g, bh, tile) + qb * 128 + row;
-      if (qvalid && it.lse2) it.lse2[slot] = m + __log2f(l);
-      const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
-      const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = qvalid && only_cover(g, tbk.tb, p);
-      OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * kD;
-      float* dst_scr = it.ot + slot * kD;
-      // the whole O row into registers, then O_x is released at once: the next
-      // item's first P V may overwrite it while this row is scaled and stored
-      uint32_t r0[32], r1[32];
-      tmem_ld32(tO, r0);
-      tmem_ld32(tO + 32, r1);
-      tmem_wait_ld(r0);
-      tmem_wait_ld(r1);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(o_empty(x));
-      if (qvalid) {
+      // ---- epilogue: wait for the last P V, O / l.  Two forms, because ptxas's
+      // schedule of the softmax loop above hangs on what stays live across it
+      // (the same loop ran between 57 and 84 ms on the paper-regime tiles):
+      //   one problem: the row's place is resolved here, while the last P V runs,
+      //     and slots leave by TMA (small tiles 2.15 -> 2.01 ms)
+      //   ragged: resolved before the loop, plain stores (each request has its own
+      //     tensor map, which every storing warp would have to acquire; 3.21 ms per
+      //     iteration of six requests, 3.7 in the other form)
+      if constexpr (RAGGED) {
+        if (!(ok = WAIT(o_full(x), WX & 1))) break;
+        tc_fence_after();
+        ++WX;
+        const float inv = 1.f / l;
+        const int64_t slot = tile_slot0(g, bh, tile) + qb * 128 + row;
+        const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
+        const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
+        const bool single = qvalid && only_cover(g, tbk.tb, p);
+        OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * kD;
+        float* dst_scr = it.ot + slot * kD;
+        // the whole O row into registers, then O_x is released at once: the next
+        // item's first P V may overwrite it while this row is scaled and stored
+        uint32_t r0[32], r1[32];
+        tmem_ld32(tO, r0);
+        tmem_ld32(tO + 32, r1);
+        tmem_wait_ld(r0);
+        tmem_wait_ld(r1);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(o_empty(x));
+        if (qvalid) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint32_t* r = c == 0 ? r0 : r1;
+          for (int c = 0; c < 2; ++c) {
+            const uint32_t* r = c == 0 ? r0 : r1;
 #pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            const float4 v4 = make_float4(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv,
-                                          __uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
-            if (single)
-              store4<OutT>(dst_out + c * 32 + e, v4);
-            else
-              store4<float>(dst_scr + c * 32 + e, v4);
+            for (int e = 0; e < 32; e += 4) {
+              const float4 v4 = make_float4(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv,
+                                            __uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
+              if (single)
+                store4<OutT>(dst_out + c * 32 + e, v4);
+              else
+                store4<float>(dst_scr + c * 32 + e, v4);
+            }
           }
         }
+      } else {
+        Item it2;
+        TileBlocks tb2;
+        resolve<RAGGED, false>(a, &tq, &tk, &tv, w, rc, it2);
+        const Geom& g2 = *it2.g;
+        tile_blocks(g2, it2.tile, tb2);
+        const int qb2 = 2 * it2.pair + x;
+        int qo[3], l2[3];
+        block_origin(g2, tb2, qb2, qo);
+        block_row(g2, qo, row, l2);
+        const bool valid = inside(tb2, l2);
+        const float inv = 1.f / l;
+        const int64_t slot = tile_slot0(g2, it2.bh, it2.tile) + qb2 * 128 + row;
+        if (valid) it2.lse2[slot] = m + __log2f(l);
+        const int p[3] = {tb2.tb.lo[0] + l2[0], tb2.tb.lo[1] + l2[1], tb2.tb.lo[2] + l2[2]};
+        const int64_t tok = valid ? ((int64_t)p[0] * g2.G[1] + p[1]) * g2.G[2] + p[2] : 0;
+        const bool single = valid && only_cover(g2, tb2.tb, p);
+        if (!(ok = WAIT(o_full(x), WX & 1))) break;
+        tc_fence_after();
+        ++WX;
+        uint32_t r0[32], r1[32];
+        tmem_ld32(tO, r0);
+        tmem_ld32(tO + 32, r1);
+        tmem_wait_ld(r0);
+        tmem_wait_ld(r1);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(o_empty(x));
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          r0[e] = __float_as_uint(__uint_as_float(r0[e]) * inv);
+          r1[e] = __float_as_uint(__uint_as_float(r1[e]) * inv);
+        }
+        if (single) store_row(static_cast<OutT*>(it2.out) + ((int64_t)it2.bh * g2.N + tok) * kD, r0, r1);
+        if (__any_sync(0xffffffffu, valid && !single)) {
+          // FP32 slots of this warp's 32 rows, through shared memory (rows past R
+          // stay zero, they are padding of the Q block; slots of rows that are
+          // not multiply covered are never read)
+          const uint32_t sq = st_q + buf * 2 * kBox;
+          if (row < a.pad_R) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const uint32_t off = lane * 128 + ((c ^ (lane & 7)) << 4);
+              st_shared_v4(sq + off, r0[4 * c], r0[4 * c + 1], r0[4 * c + 2], r0[4 * c + 3]);
+              st_shared_v4(st_o + off, r1[4 * c], r1[4 * c + 1], r1[4 * c + 2], r1[4 * c + 3]);
+            }
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            const int srow = (int)(slot - lane);
+            tma_store_2d(&to, sq, 0, srow);
+            tma_store_2d(&to, st_o, 32, srow);
+            bulk_commit();
+          }
+        }
+        staged = (int)buf;
+        ++W;
       }
     }
+    release_staged();
+    if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -643,23 +793,23 @@ cudaError_t run_fwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16
   a.g = g;
   a.out = out;
   a.lse2 = lse2;
-  a.ot = ot;
   a.flags = flags;
   a.pad_R = g.R;
   const int64_t items = (int64_t)g.B * g.nh * g.ntiles * box_pairs(g);
   if (items >= (1LL << 31)) return cudaErrorNotSupported;
   a.items = (int)items;
   const int BH = g.B * g.nh;
-  CUtensorMap mq, mk, mv;
+  CUtensorMap mq, mk, mv, mo;
   if (!make_tmap_5d(&mq, q, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
       !make_tmap_5d(&mk, k, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
-      !make_tmap_5d(&mv, v, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt))
+      !make_tmap_5d(&mv, v, kD, g.G[2], g.G[1], g.G[0], BH, g.bx, g.by, g.bt) ||
+      !make_tmap_slots(&mo, ot, kD, (int64_t)BH * g.ntiles * g.per_tile, 32))
     return cudaErrorInvalidValue;
   auto kern = fwd64_kernel<OutT, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<false>::kSmem);
   if (e != cudaSuccess) return e;
   const int grid = (int)(a.items < num_sms() ? a.items : num_sms());
-  kern<<<grid, kThreadsF, Cfg::kSmem, st>>>(mq, mk, mv, a);
+  kern<<<grid, kThreadsF, Cfg<false>::kSmem, st>>>(mq, mk, mv, mo, a);
   return cudaGetLastError();
 }
 
@@ -683,9 +833,9 @@ cudaError_t launch_sm103_fwd64_ragged(const ReqDesc* reqs, const int64_t* counts
   CUtensorMap dummy;
   memset(&dummy, 0, sizeof(dummy));
   auto kern = fwd64_kernel<__nv_bfloat16, true>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<true>::kSmem);
   if (e != cudaSuccess) return e;
-  kern<<<num_sms(), kThreadsF, Cfg::kSmem, st>>>(dummy, dummy, dummy, a);
+  kern<<<num_sms(), kThreadsF, Cfg<true>::kSmem, st>>>(dummy, dummy, dummy, dummy, a);
   return cudaGetLastError();
 }
 
