@@ -320,32 +320,29 @@ __global__ void __launch_bounds__(kThreadsB, 1)
         if (lane == 0) mbar_arrive(p_full + 1);
       }
       if (!ok) break;
-      // ---- epilogue: this thread's key row of dK, dV (columns [32 c4, 32 c4 + 32))
-      if (!(ok = WAIT(acc_full, W & 1))) break;
-      tc_fence_after();
+      // ---- where this thread's key row goes, while the last gradient products run
       int ko[3], kl[3];
       block_origin(g, tbk, kb, ko);
       block_row(g, ko, row, kl);
       const bool kvalid = inside(tbk, kl);
       const int p[3] = {tbk.tb.lo[0] + kl[0], tbk.tb.lo[1] + kl[1], tbk.tb.lo[2] + kl[2]};
-      const int64_t tok = kvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const bool single = kvalid && only_cover(g, tbk.tb, p);
-      const int64_t slot = tile_slot0(g, bh, tile) + kb * 128 + row;
-      const int c0 = c4 * 32;
-      // both accumulators into registers, then they are released at once: the
-      // next item's first gradient products may overwrite them during the stores
-      uint32_t rk[32], rv[32];
-      tmem_ld32(tl + C::kColDK + c0, rk);
-      tmem_ld32(tl + C::kColDV + c0, rv);
-      tmem_wait_ld(rk);
-      tmem_wait_ld(rv);
+      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
+      const int64_t off = ((int64_t)bh * g.N + tok) * kD + c4 * 32;
+      const int64_t slots = (tile_slot0(g, bh, tile) + kb * 128 + quad * 32) * kD + c4 * 32;
+      // ---- epilogue: columns [32 c4, 32 c4 + 32) of dK, then of dV
+      if (!(ok = WAIT(acc_full, W & 1))) break;
+      tc_fence_after();
+      uint32_t r[32];
+      tmem_ld32(tl + C::kColDK + c4 * 32, r);
+      tmem_wait_ld(r);
+      row_slots<OutT>(r, g.scale, kvalid, single, static_cast<OutT*>(a.dk) + off, a.dk_s + slots, lane);
+      tmem_ld32(tl + C::kColDV + c4 * 32, r);
+      tmem_wait_ld(r);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);
-      row_store<32, OutT>(rk, g.scale, kvalid, single, static_cast<OutT*>(a.dk) + ((int64_t)bh * g.N + tok) * kD + c0,
-                          a.dk_s + slot * kD + c0);
-      row_store<32, OutT>(rv, 1.f, kvalid, single, static_cast<OutT*>(a.dv) + ((int64_t)bh * g.N + tok) * kD + c0,
-                          a.dv_s + slot * kD + c0);
+      row_slots<OutT>(r, 1.f, kvalid, single, static_cast<OutT*>(a.dv) + off, a.dv_s + slots, lane);
       ++W;
     }
   }
@@ -677,15 +674,16 @@ __global__ void __launch_bounds__(kThreadsB, 1)
         }
       }
       if (!ok) break;
-      if (!(ok = WAIT(acc_full, W & 1))) break;
-      tc_fence_after();
+      // where this item's rows go, while the last dQ product runs
       int qo[3], ql[3];
       block_origin(g, tbk, qb, qo);
       block_row(g, qo, row, ql);
       const bool qvalid = inside(tbk, ql);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
-      const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const bool single = qvalid && only_cover(g, tbk.tb, p);
+      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
+      if (!(ok = WAIT(acc_full, W & 1))) break;
+      tc_fence_after();
       const int c0 = c4 * 32;
       uint32_t rq[32];
       tmem_ld32(tl + C::kColDQ + c0, rq);
@@ -693,8 +691,8 @@ __global__ void __launch_bounds__(kThreadsB, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);  // released before the stores
-      row_store<32, OutT>(rq, g.scale, qvalid, single, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
-                          a.dq_s + qslot * kD + c0);
+      row_slots<OutT>(rq, g.scale, qvalid, single, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
+                      a.dq_s + (qslot - lane) * kD + c0, lane);
       ++W;
     }
   }

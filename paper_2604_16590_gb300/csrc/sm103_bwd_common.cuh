@@ -42,24 +42,6 @@ constexpr int kMath0 = 3;
 constexpr int kIssuerA = 2;
 constexpr int kThreadsB = 32 * (kMath0 + kMathW);
 
-// Stores N FP32 values of this thread's row (already in registers), scaled
-// by `mul`: to `out` (OutT) if the row is covered by one tile, else to the
-// FP32 slot `scr`, nothing if the row lies outside the tile.
-template <int N, typename OutT>
-__device__ __forceinline__ void row_store(const uint32_t (&r)[N], float mul, bool valid, bool single, OutT* out,
-                                          float* scr) {
-  if (!valid) return;
-#pragma unroll
-  for (int e = 0; e < N; e += 4) {
-    const float4 v = make_float4(__uint_as_float(r[e]) * mul, __uint_as_float(r[e + 1]) * mul,
-                                 __uint_as_float(r[e + 2]) * mul, __uint_as_float(r[e + 3]) * mul);
-    if (single)
-      store4<OutT>(out + e, v);
-    else
-      store4<float>(scr + e, v);
-  }
-}
-
 // N FP32 columns of this thread's row, already in registers and scaled, to the
 // output row (16 bytes at a time)
 template <int N>
@@ -111,6 +93,24 @@ __device__ __forceinline__ void row_out(uint32_t (&r)[N], float mul, bool valid,
     tma_store_2d(map, st, col, srow);
     bulk_commit();
   }
+}
+
+// Multiplies 32 accumulator columns by `mul` and writes them out, to `out` if
+// this thread's row is covered by one tile only, and (the warp's 32 rows
+// together, as soon as one of them is multiply covered) to the FP32 slots from
+// row 0 of the warp at `scr`; slots of other rows are never read.  The d = 128
+// kernels have no shared memory for staged stores (row_out above); the
+// transposed stores take a quarter of the LSU time of a thread writing its
+// own row.
+template <typename OutT>
+__device__ __forceinline__ void row_slots(uint32_t (&r)[32], float mul, bool valid, bool single, OutT* out, float* scr,
+                                          int lane) {
+#pragma unroll
+  for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * mul);
+  if (single) store_cols<32>(out, r);
+  if (!__any_sync(0xffffffffu, valid && !single)) return;
+  store_rows16(scr, 128, lane, r);
+  store_rows16(scr + 16, 128, lane, r + 16);
 }
 
 // dK/dV: P'^T of 32 columns of this thread's key row (S'^T already carries the

@@ -102,6 +102,35 @@ __device__ __forceinline__ void zero_pad_rows(uint8_t* base, int n, int R) {
   sm103::fence_proxy_async_smem();
 }
 
+// Writes a 32-row x 16-column FP32 piece of a warp, thread l holding row l, to
+// rows `base` (row 0) + l * ld: the four lanes of a quad transpose their 4 x 4
+// 16-byte units by shuffles, so that a store instruction writes eight 64-byte
+// segments instead of 16 bytes in each of 32 rows.
+__device__ __forceinline__ void store_rows16(float* base, int ld, int lane, const uint32_t* r) {
+  uint32_t v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = r[i];
+#pragma unroll
+  for (int s = 1; s < 4; s <<= 1) {
+    const bool up = lane & s;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (e & s) continue;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t lo = v[4 * e + i], hi = v[4 * (e | s) + i];
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, s);
+        v[4 * e + i] = up ? got : lo;
+        v[4 * (e | s) + i] = up ? hi : got;
+      }
+    }
+  }
+  float* dst = base + (int64_t)(lane & ~3) * ld + 4 * (lane & 3);
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    *reinterpret_cast<uint4*>(dst + (int64_t)e * ld) = make_uint4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+}
+
 // first slot of tile `tile` of batch*head bh (block j, row rho at + j*128 + rho)
 __device__ __forceinline__ int64_t tile_slot0(const Geom& g, int bh, int tile) {
   return ((int64_t)bh * g.ntiles + tile) * g.per_tile;

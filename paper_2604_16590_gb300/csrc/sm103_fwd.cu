@@ -626,26 +626,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int64_t slot = tile_slot0(g, bh, tile) + qb * 128 + row;
       if (qvalid && ch == 0 && it.lse2) it.lse2[slot] = rs.m + __log2f(l);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
-      const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const bool single = qvalid && only_cover(g, tbk.tb, p);
+      const bool slots = __any_sync(0xffffffffu, qvalid && !single);
+      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
       const int c0 = ch * (D / 2);
       OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * D + c0;
-      float* dst_scr = it.ot + slot * D + c0;
+      float* dst_scr = it.ot + (slot - lane) * D + c0;
       uint32_t r[32];
 #pragma unroll
       for (int c = 0; c < D / 64; ++c) {
         tmem_ld32(tO + c * 32, r);
         tmem_wait_ld(r);
-        if (qvalid) {
 #pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            const float4 v4 = make_float4(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv,
-                                          __uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
-            if (single)
-              store4<OutT>(dst_out + c * 32 + e, v4);
-            else
-              store4<float>(dst_scr + c * 32 + e, v4);
-          }
+        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
+        if (single) {
+#pragma unroll
+          for (int e = 0; e < 32; e += 4)
+            store4<OutT>(dst_out + c * 32 + e, make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
+                                                           __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])));
+        }
+        if (slots) {  // the warp's 32 rows together; slots of rows that are not multiply covered are never read
+          store_rows16(dst_scr + c * 32, D, lane, r);
+          store_rows16(dst_scr + c * 32 + 16, D, lane, r + 16);
         }
       }
       tc_fence_before();
