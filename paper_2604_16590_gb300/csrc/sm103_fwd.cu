@@ -17,7 +17,7 @@
 // and parks multiply-covered rows (FP32) for the deterministic Hann merge, and
 // stores the row log-sum-exp for the backward.
 //
-// Warp roles (320 threads, one CTA per SM, persistent over work items
+// Warp roles (384 threads, one CTA per SM, persistent over work items
 // (batch*head, tile, query block)):
 //   warp 0      TMA producer (Q once per item; K_j, V_j through a ring of stages)
 //   warp 1      TMEM allocator + issuer of the S = Q K^T products
@@ -25,6 +25,11 @@
 //               lane quadrant splitting each row's keys and output columns
 //               (two math warps per SM sub-partition hide TMEM/MUFU latency)
 //   warp 10     issuer of the P V products
+//   warp 11     key-mask writer: the bias row of a key block with padding rows or
+//               keys outside the tile, added to its scores by one more K = 16 MMA
+//               step, so the softmax has one branch-free form (a second, masked
+//               form of the loop, cost the ragged 7 x 45 x 77 crop of 12 heads 2.16 ms
+//               against 1.44 now, and unmasked tiles 1 %)
 // Two issuing threads, because a thread's shared-memory accesses (an mbarrier
 // wait included) are held until the tcgen05.mma it issued before them have
 // drained from the tensor pipe: with one issuer every wait between the S and
@@ -51,7 +56,12 @@ struct FwdCfg {
   static constexpr int kQ = 0;
   static constexpr int kK = kQ + kBlock;
   static constexpr int kV = kK + kStages * kBlock;
-  static constexpr int kBar = kV + kStages * kBlock;
+  // Key-mask extension operands (as in the d = 64 forward): A = 1 in K-column 0
+  // of 128 rows, and per stage the key block's bias row (0, or -1e30 for a
+  // padding key or a key outside the tile), each followed by 2 KB of zeros.
+  static constexpr int kOnes = kV + kStages * kBlock;
+  static constexpr int kBias = kOnes + 4096;
+  static constexpr int kBar = kBias + kStages * 4096;
   // q_full, q_empty, qt_full, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], s_empty[2],
   // p_full, pv_done[2], o_empty, drain[2], never (test hook: nothing arrives on it)
   static constexpr int kNumBars = 3 + 4 * kStages + 4 + 7;
@@ -154,8 +164,9 @@ __device__ void set_status_fwd(uint32_t c) { set_status(c); }
 // its 32 query rows, warp half `ch` owning keys [64 ch, 64 ch + 64) of every
 // block (one 64-key chunk of P) and output columns [ch D/2, (ch+1) D/2).
 constexpr int kMathWarps = 8;
-constexpr int kThreads = 64 + 32 * kMathWarps + 32;
+constexpr int kThreads = 64 + 32 * kMathWarps + 64;
 constexpr int kIssuerPV = 2 + kMathWarps;  // warp index of the P V issuer
+constexpr int kMaskWriter = kIssuerPV + 1;
 
 // Online-softmax state of one query row, as held by one of its two threads.
 // P = exp2(s S log2e - m) is formed against a reference max m that only moves
@@ -201,42 +212,27 @@ __device__ __forceinline__ float pair_exchange(float* red, int parity, int ch, i
 }
 
 // running max of 32 scores into 4 partial maxima (3-input max)
-template <bool MASK>
-__device__ __forceinline__ void chunk_max(const uint32_t (&r)[32], uint32_t mbits, float (&mx)[4]) {
+__device__ __forceinline__ void chunk_max(const uint32_t (&r)[32], float (&mx)[4]) {
 #pragma unroll
-  for (int i = 0; i < 32; i += 2) {
-    float x0 = __uint_as_float(r[i]), x1 = __uint_as_float(r[i + 1]);
-    if (MASK) {
-      x0 = (mbits >> i) & 1u ? x0 : -INFINITY;
-      x1 = (mbits >> (i + 1)) & 1u ? x1 : -INFINITY;
-    }
-    mx[(i >> 1) & 3] = sm103::fmax3(mx[(i >> 1) & 3], x0, x1);
-  }
+  for (int i = 0; i < 32; i += 2)
+    mx[(i >> 1) & 3] = sm103::fmax3(mx[(i >> 1) & 3], __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
 }
 
 // exp2 of 32 scores -> 16 BF16 pairs (for TMEM), with the exp2 argument and the
 // row sum formed by packed FP32 pair instructions
-template <bool MASK>
-__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[32], uint32_t mbits, uint64_t s2, uint64_t nm2,
-                                          uint64_t (&acc)[4], uint32_t* pk) {
+__device__ __forceinline__ void exp_chunk(const uint32_t (&r)[32], uint64_t s2, uint64_t nm2, uint64_t (&acc)[4],
+                                          uint32_t* pk) {
   using namespace sm103;
 #pragma unroll
   for (int i = 0; i < 32; i += 2) {
     float a0, a1;
     f2unpack(ffma2(u2pack(r[i], r[i + 1]), s2, nm2), a0, a1);
-    float p0 = ex2(a0), p1 = ex2(a1);
-    if (MASK) {
-      p0 = (mbits >> i) & 1u ? p0 : 0.f;
-      p1 = (mbits >> (i + 1)) & 1u ? p1 : 0.f;
-    }
+    const float p0 = ex2(a0), p1 = ex2(a1);
     acc[(i >> 1) & 3] = fadd2(acc[(i >> 1) & 3], f2pack(p0, p1));
     pk[i >> 1] = pack_bf16(p0, p1);
   }
 }
 
-// One 128-key block of the online softmax for this thread's half of a query
-// row: partial row max (exchanged with the partner), fold of the previous
-// block's P V into O, exp2 of its 64 scores into P (shared memory), row-sum.
 // Rescale this thread's half (D/2 columns) of the O accumulator in TMEM by
 // `f` (1 for rows that keep their reference max).  Warp-synchronous.
 template <int D>
@@ -264,9 +260,9 @@ __device__ __forceinline__ void rescale_o(uint32_t tO, float f) {
 // row: partial row max (exchanged with the partner thread), lazy rescale of
 // the reference max (and of O in TMEM, after the previous P V completed),
 // exp2 of the 64 scores into BF16 P in TMEM, row-sum update.
-template <int D, bool MASK>
+template <int D>
 __device__ __forceinline__ bool softmax_block(RowState& rs, uint32_t tS, uint32_t tO, uint32_t tP, int row, int ch,
-                                              int quad, float* red, int parity, const uint32_t (&kmask)[2], float sl2,
+                                              int quad, float* red, int parity, float sl2,
                                               bool first,
                                               uint64_t* pv_last, uint32_t pv_last_par, uint64_t* p_free,
                                               uint32_t p_free_par, volatile int* abort_flag) {
@@ -283,8 +279,9 @@ __device__ __forceinline__ bool softmax_block(RowState& rs, uint32_t tS, uint32_
   tmem_ld32(tS + 32, r1);
   tmem_wait_ld(r0);
   tmem_wait_ld(r1);
-  chunk_max<MASK>(r0, kmask[0], mx);
-  chunk_max<MASK>(r1, kmask[1], mx);
+  // masked keys carry -1e30 from the extension step: no mask here
+  chunk_max(r0, mx);
+  chunk_max(r1, mx);
   const float mine = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
   const float other = pair_exchange(red, parity, ch, row, quad, mine);
   const float mblk = fmaxf(mine, other) * sl2;
@@ -305,8 +302,8 @@ __device__ __forceinline__ bool softmax_block(RowState& rs, uint32_t tS, uint32_
   }
   const uint64_t s2 = f2pack(sl2, sl2), nm2 = f2pack(-rs.m, -rs.m);
   uint32_t pk0[16], pk1[16];
-  exp_chunk<MASK>(r0, kmask[0], s2, nm2, acc, pk0);
-  exp_chunk<MASK>(r1, kmask[1], s2, nm2, acc, pk1);
+  exp_chunk(r0, s2, nm2, acc, pk0);
+  exp_chunk(r1, s2, nm2, acc, pk1);
   // this P buffer is free once the P V product that last read it completed
   if (!mbar_wait<set_status_fwd>(p_free, p_free_par, abort_flag)) return false;
   tc_fence_after();
@@ -356,12 +353,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   zero_pad_rows(smem, (1 + 2 * C::kStages) * C::kHalves, a.pad_R);  // Q and the K and V rings
+  for (int r = threadIdx.x; r < (1 + C::kStages) * 256; r += kThreads) {
+    const int blk = r >> 8, rr = r & 255;
+    const uint4 v = (blk == 0 && rr < 128) ? make_uint4(0x00003F80u, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+    if (blk == 0 || rr >= 128) *reinterpret_cast<uint4*>(smem + C::kOnes + blk * 4096 + rr * 16) = v;
+  }
+  fence_proxy_async_smem();
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     mbar_init(q_empty, kMathWarps);
     mbar_init(qt_full, kMathWarps);
     for (int s = 0; s < C::kStages; ++s) {
-      mbar_init(k_full + s, 1);
+      mbar_init(k_full + s, 2);  // the K load (producer) and the stage's bias row (mask writer)
       mbar_init(k_empty + s, 1);
       mbar_init(v_full + s, 1);
       mbar_init(v_empty + s, 1);
@@ -459,6 +462,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       constexpr uint32_t idS = idesc_bf16(128, 128, 0);
       const uint64_t dK0 = sw128_desc(smem_u32(smem + C::kK), 16, 1024);
+      const uint64_t dOnes = noswz_desc(smem_u32(smem + C::kOnes), 2048, 128);
+      const uint64_t dBias0 = noswz_desc(smem_u32(smem + C::kBias), 2048, 128);
       uint32_t G = 0, W = 0;
       bool ok = true;
       if (a.flags & GATTN_FLAG_TEST_STALL)  // failure-detection hook: a wait that cannot complete
@@ -470,8 +475,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         tile_blocks(*it.g, it.tile, tbk);
         if (it.blk >= tbk.NB) continue;
         if (!(ok = mbar_wait<set_status_fwd>(qt_full, W & 1, abort_flag))) break;  // Q in TMEM
-        for (int j = 0; j < tbk.NB; ++j, ++G) {
+        const bool all_full = tile_all_full(*it.g, tbk);
+        BlockWalk bw;
+        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
           const uint32_t st = G % C::kStages, sb = G & 1;
+          // a masked block's bias row was filled by the mask writer
+          const bool masked = !all_full && !bw.full(*it.g, tbk);
           if (!(ok = mbar_wait<set_status_fwd>(k_full + st, (G / C::kStages) & 1, abort_flag))) break;
           if (!(ok = mbar_wait<set_status_fwd>(s_empty + sb, ((G >> 1) & 1) ^ 1, abort_flag))) break;
           tc_fence_after();
@@ -480,6 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int ks = 0; ks < D / 16; ++ks)
             umma_bf16_ts(tmem + sb * 128, tmem + C::kColQ + ks * 8, dmove(dk, (ks >> 2) * 16384 + (ks & 3) * 32),
                          idS, ks > 0);
+          if (masked) umma_bf16(tmem + sb * 128, dOnes, dmove(dBias0, st * 4096), idS, 1u);  // + bias of each key column
           umma_commit(s_full + sb);
           umma_commit(k_empty + st);
         }
@@ -521,6 +531,40 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       umma_commit(drain + 1);
       mbar_wait<set_status_fwd>(drain + 1, 0, abort_flag, false);
+    }
+  } else if (warp == kMaskWriter) {
+    // ------------------------------------------------------------ key-mask writer
+    // One arrival on k_full per stage use (the stage's second arrival), in the
+    // producer's order; it first waits until the stage is free again.
+    const uint32_t neg = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(-1e30f));
+    uint32_t G = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+      Item it;
+      if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+      const Geom& g = *it.g;
+      TileBlocks tbk;
+      tile_blocks(g, it.tile, tbk);
+      if (it.blk >= tbk.NB) continue;
+      BlockWalk bw;
+      for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
+        const uint32_t st = G % C::kStages, n = G / C::kStages;
+        const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
+        if (lane == 0) ok = mbar_wait<set_status_fwd>(k_empty + st, (n & 1) ^ 1, abort_flag);
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        if (!ok) break;
+        if (!block_full(g, tbk, ko)) {
+          for (int r = lane; r < 128; r += 32) {
+            int kl[3];
+            block_row(g, ko, r, kl);
+            *reinterpret_cast<uint4*>(smem + C::kBias + st * 4096 + r * 16) =
+                make_uint4(inside(tbk, kl) ? 0u : neg, 0u, 0u, 0u);
+          }
+          fence_proxy_async_smem();  // the tensor core reads what these lanes wrote
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(k_full + st);
+      }
     }
   } else {
     // ------------------------------------------------------------ softmax + epilogue
@@ -571,29 +615,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       rs.m = -INFINITY;
       rs.l = 0.f;
       rs.lc = 0.f;
-      // key-block coordinates stepped incrementally (no divisions in the loop)
-      int jt = 0, jy = 0, jx = 0;
       for (int j = 0; j < tbk.NB; ++j, ++G) {
         const uint32_t sb = G & 1, pb = G % C::kPBufs;
-        const int ko[3] = {jt * g.bt, jy * g.by, jx * g.bx};
-        if (++jx == tbk.nb[2]) {
-          jx = 0;
-          if (++jy == tbk.nb[1]) {
-            jy = 0;
-            ++jt;
-          }
-        }
-        // validity of this thread's 64 key columns, one ballot per 32
-        uint32_t kmask[2] = {~0u, ~0u};
-        const bool full = block_full(g, tbk, ko);
-        if (!full) {
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            int kl[3];
-            block_row(g, ko, ch * 64 + c * 32 + lane, kl);
-            kmask[c] = __ballot_sync(0xffffffffu, inside(tbk, kl));
-          }
-        }
         if (!(ok = mbar_wait<set_status_fwd>(s_full + sb, (G >> 1) & 1, abort_flag))) break;
         tc_fence_after();
         const uint32_t tS = tl + sb * 128 + ch * 64;
@@ -602,12 +625,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint64_t* pv_last = pv_done + (G - 1) % C::kPBufs;
         const uint32_t pv_last_par = ((G - 1) / C::kPBufs) & 1;
         const uint32_t p_free_par = ((G / C::kPBufs) & 1) ^ 1;
-        if (full)
-          ok = softmax_block<D, false>(rs, tS, tO, tP, row, ch, quad, red, sb, kmask, g.scale_log2, j == 0, pv_last,
-                                       pv_last_par, pv_done + pb, p_free_par, abort_flag);
-        else
-          ok = softmax_block<D, true>(rs, tS, tO, tP, row, ch, quad, red, sb, kmask, g.scale_log2, j == 0, pv_last,
-                                      pv_last_par, pv_done + pb, p_free_par, abort_flag);
+        ok = softmax_block<D>(rs, tS, tO, tP, row, ch, quad, red, sb, g.scale_log2, j == 0, pv_last, pv_last_par,
+                              pv_done + pb, p_free_par, abort_flag);
         if (!ok) break;
         tc_fence_before();
         __syncwarp();
