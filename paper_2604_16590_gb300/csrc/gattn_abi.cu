@@ -61,6 +61,8 @@ void prof_end(int kernel, cudaStream_t st) {
   p.open_start[kernel] = nullptr;
 }
 
+static_assert(sizeof(gattn_desc) == 68, "no padding: descriptors are compared as bytes");
+
 static bool dtype_ok(int32_t t) { return t == GATTN_BF16 || t == GATTN_FP32; }
 
 static int clipped_extent(const Geom& g, int a, int k) {
@@ -151,8 +153,7 @@ bool apply_box(Geom* g, const int b[3]) {
   return true;
 }
 
-bool make_geom(const gattn_desc* desc, Geom* g) {
-  if (!desc || !g) return false;
+static bool build_geom(const gattn_desc* desc, Geom* g) {
   memset(g, 0, sizeof(*g));
   const gattn_desc& d = *desc;
   if (d.B < 1 || d.nh < 1 || d.T < 1 || d.Y < 1 || d.X < 1) return false;
@@ -209,6 +210,32 @@ bool make_geom(const gattn_desc* desc, Geom* g) {
   // a box shape whose per-tile slot count does not fit 32 bits is refused
   if (!choose_box(g)) return false;
   if (g->R < 1 || g->nbmax_tot < 1 || (int64_t)g->nbmax_tot * 128 >= (1LL << 31)) return false;
+  return true;
+}
+
+// The geometry of a descriptor.  Building one takes 5-6 us (the box search),
+// and a forward or backward call and its two size queries need the same one, so
+// each thread keeps the last four it built, by the descriptor's value.
+bool make_geom(const gattn_desc* desc, Geom* g) {
+  struct Entry {
+    gattn_desc desc;
+    Geom g;
+    bool used;
+  };
+  static thread_local Entry memo[4];
+  static thread_local int next;
+  if (!desc || !g) return false;
+  for (const Entry& e : memo)
+    if (e.used && memcmp(&e.desc, desc, sizeof(gattn_desc)) == 0) {
+      *g = e.g;
+      return true;
+    }
+  if (!build_geom(desc, g)) return false;
+  Entry& e = memo[next];
+  next = (next + 1) & 3;
+  e.desc = *desc;
+  e.g = *g;
+  e.used = true;
   return true;
 }
 

@@ -13,6 +13,7 @@ arguments; tensors may be passed where the C side takes device pointers).
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 
@@ -204,16 +205,16 @@ def _ptr(x):
     if x is None:
         return None
     if isinstance(x, torch.Tensor):
-        return ctypes.c_void_p(x.data_ptr())
-    return ctypes.c_void_p(int(x))
+        return x.data_ptr()  # the prototypes convert to void *
+    return int(x)
 
 
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _nbytes(x, given):
@@ -612,6 +613,28 @@ def desc_for(q: torch.Tensor, tiling: Tiling, out_dtype=None, flags: int = 0):
     )
 
 
+@functools.lru_cache(maxsize=256)
+def _plan(shape, dtype, tiling, out_dtype):
+    """(desc, torch output dtype, saved bytes, workspace bytes) of a forward or
+    backward call; the descriptor is not handed out.  A call on one small frame
+    spends more host time on these than on its launches."""
+    B, nh, N, d = shape
+    if N != tiling.N:
+        raise ValueError(f"N={N} does not match grid {tiling.grid}")
+    desc = make_desc(B, nh, d, tiling.grid, tiling.core, tiling.halo, tiling.window, dtype, out_dtype, tiling.scale)
+    return desc, _TORCH_DTYPE[desc.out_dtype], gattn_saved_bytes(desc), gattn_bwd_workspace_bytes(desc)
+
+
+def _plan_for(q, tiling, out_dtype):
+    if q.dim() != 4:
+        raise ValueError("expected [B, heads, N, d]")
+    out_dtype = out_dtype if out_dtype is not None else q.dtype
+    try:
+        return _plan(q.shape, q.dtype, tiling, out_dtype)
+    except TypeError:  # a tiling given as lists cannot be looked up
+        return _plan.__wrapped__(q.shape, q.dtype, tiling, out_dtype)
+
+
 def _require_cuda(*ts):
     for t in ts:
         if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
@@ -621,24 +644,24 @@ def _require_cuda(*ts):
 def forward(q, k, v, tiling: Tiling, out_dtype=None, stream=None):
     """Out = GPA(q, k, v) and the saved state the backward needs."""
     _require_cuda(q, k, v)
-    desc = desc_for(q, tiling, out_dtype)
-    out = torch.empty(q.shape, dtype=_TORCH_DTYPE[desc.out_dtype], device=q.device)
-    saved = torch.empty(gattn_saved_bytes(desc), dtype=torch.uint8, device=q.device)
-    check(gattn_fwd(desc, q, k, v, out, saved, stream=stream), "gattn_fwd")
+    desc, dtype, nsaved, _ = _plan_for(q, tiling, out_dtype)
+    out = torch.empty(q.shape, dtype=dtype, device=q.device)
+    saved = torch.empty(nsaved, dtype=torch.uint8, device=q.device)
+    check(gattn_fwd(desc, q, k, v, out, saved, nsaved, stream), "gattn_fwd")
     return out, saved
 
 
 def backward(q, k, v, out, dout, saved, tiling: Tiling, stream=None):
     """(dq, dk, dv) of sum(out * dout)."""
     _require_cuda(q, k, v, out, dout, saved)
-    desc = desc_for(q, tiling, out.dtype)
+    desc, _, _, nws = _plan_for(q, tiling, out.dtype)
     if dout.dtype != q.dtype:
         raise ValueError("dout must have the input dtype")
     dq = torch.empty_like(out)
     dk = torch.empty_like(out)
     dv = torch.empty_like(out)
-    ws = torch.empty(gattn_bwd_workspace_bytes(desc), dtype=torch.uint8, device=q.device)
-    check(gattn_bwd(desc, q, k, v, out, dout, saved, dq, dk, dv, ws, stream=stream), "gattn_bwd")
+    ws = torch.empty(nws, dtype=torch.uint8, device=q.device)
+    check(gattn_bwd(desc, q, k, v, out, dout, saved, dq, dk, dv, ws, ws_bytes=nws, stream=stream), "gattn_bwd")
     return dq, dk, dv
 
 
