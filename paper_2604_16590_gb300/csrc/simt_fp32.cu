@@ -13,17 +13,20 @@
 //            neighbouring elements (both operands are d-contiguous, so pairs
 //            load as they lie; the two partial sums are added at the end);
 //            12 16-byte loads per 64 pair instructions at d = 64
-//   P V, ... 8 rows x CT columns a thread, one key at a time; the warp's P is
-//            kept key-major with every value doubled ((p, p) pairs), so its
-//            operand needs no moves; 5 loads per 16 pair instructions
+//   P V, ... 8 rows x CT columns a thread in pairs of rows, one key at a time;
+//            the warp's P is kept key-major, so a key's rows load as pairs, and
+//            the CT values of the other operand are doubled in registers; 3
+//            loads per 16 pair instructions (with P doubled in shared memory
+//            instead, 5: the loads, not the FMAs, then set the pace)
 // Rows never leave their warp: P goes through a warp-private buffer, so CTA
 // barriers only order the streamed blocks.  Every 64-row block is reduced
 // locally before it is folded into the running sums (two-level summation,
 // which keeps the FP32 error of L-long sums near eps * (sqrt(64) + sqrt(L/64))).
-// Bound: the FP32 pipe (128 lanes a clock and SM).  4 heads of a 4 x 64 x 128
-// clip in 16 tiles of up to 4608 tokens, d = 64: forward 14.6 -> 7.1 ms, dQ
-// 17.0 -> 9.3, dK/dV 19.4 -> 12.4 (before: a thread group per row, one FMA per
-// shared-memory word).
+// Bound: the FP32 pipe (128 lanes a clock and SM), 53-57 % active with two
+// warps per scheduler (registers), shared memory at half its rate.  4 heads of
+// a 4 x 64 x 128 clip in 16 tiles of up to 4608 tokens, d = 64: forward 14.6 ->
+// 6.2 ms, dQ 17.0 -> 8.8, dK/dV 19.4 -> 10.9 (before: a thread group per row,
+// one FMA per shared-memory word).
 #include "internal.cuh"
 #include "sm103_common.cuh"
 
@@ -39,11 +42,11 @@ using sm103::fmul2;
 
 constexpr int kBN = 64;  // streamed rows per block
 
-// Shape of the kernels at head size D with W warps per CTA.
-template <int D_, int W_>
+// Shape of the kernels at head size D with W warps per CTA and RG row groups
+// of 8 rows per warp.
+template <int D_, int W_, int RG_>
 struct Shape {
-  static constexpr int D = D_, W = W_;
-  static constexpr int RG = D == 128 ? 1 : 2;   // row groups of a warp, 8 rows each
+  static constexpr int D = D_, W = W_, RG = RG_;
   static constexpr int LG = 32 / RG;            // lanes of a row group
   static constexpr int KT = kBN / LG;           // score columns per thread: keys lg + LG * jj
   static constexpr int CT = D / LG;             // output columns per thread: CT * lg ...
@@ -51,9 +54,11 @@ struct Shape {
   static constexpr int BM = W * WR;             // rows per CTA
   static constexpr int T = 32 * W;
   static constexpr int LD = D + 4;              // padded row of a staged matrix (floats): conflict-free column walks
-  static constexpr int HK = 2 * LG;             // keys of P exchanged at a time (two score columns per thread)
+  static constexpr int HJ = RG == 1 && D == 64 ? 1 : 2;  // score columns per thread exchanged at a time
+  static constexpr int HK = HJ * LG;            // keys of P exchanged at a time
   static constexpr int NH = kBN / HK;
-  static constexpr int PB = 2 * WR + 4;         // floats per key of the doubled P buffer, padded
+  static constexpr int CTAS = D == 128 ? 1 : 2;  // resident CTAs per SM (shared memory)
+  static constexpr int PB = WR + 4;             // floats per key of the P buffer, padded
   static constexpr int PW = HK * PB;            // floats of a warp's P buffer
 };
 
@@ -127,63 +132,83 @@ __device__ __forceinline__ void dots(const float* __restrict__ rows, const float
     }
 }
 
-// out[i][c] += sum over the block's 64 keys of p[i][key] * M[key][CT lg + c],
+// Accumulators of 8 rows x CT columns: pairs of rows (2 i, 2 i + 1).
+template <class S>
+using Acc = uint64_t[4][S::CT];
+
+// out[i][c] += sum over the block's 64 keys of p[row][key] * M[key][CT lg + c],
 // p being this thread's score columns (exchanged within the warp through pb).
 template <class S>
 __device__ __forceinline__ void axpys(const float (&p)[8][S::KT], const float* __restrict__ M, float* pb, int rg, int lg,
-                                      uint64_t (&out)[8][S::CT / 2]) {
-  uint64_t acc[8][S::CT / 2];
+                                      Acc<S>& out) {
+  Acc<S> acc;
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int c = 0; c < S::CT / 2; ++c) acc[i][c] = 0;
+    for (int c = 0; c < S::CT; ++c) acc[i][c] = 0;
 #pragma unroll
   for (int h = 0; h < S::NH; ++h) {
     __syncwarp();  // the previous half (or product) has been read
 #pragma unroll
-    for (int jj = 0; jj < 2; ++jj) {
-      float4* d = reinterpret_cast<float4*>(pb + (lg + S::LG * jj) * S::PB + 16 * rg);
-#pragma unroll
-      for (int i = 0; i < 8; i += 2)
-        d[i / 2] = make_float4(p[i][2 * h + jj], p[i][2 * h + jj], p[i + 1][2 * h + jj], p[i + 1][2 * h + jj]);
+    for (int jj = 0; jj < S::HJ; ++jj) {
+      float4* d = reinterpret_cast<float4*>(pb + (lg + S::LG * jj) * S::PB + 8 * rg);
+      const int j = S::HJ * h + jj;
+      d[0] = make_float4(p[0][j], p[1][j], p[2][j], p[3][j]);
+      d[1] = make_float4(p[4][j], p[5][j], p[6][j], p[7][j]);
     }
     __syncwarp();
     const float* m = M + h * S::HK * S::LD + S::CT * lg;
-    const float* pp = pb + 16 * rg;
+    const float* pp = pb + 8 * rg;
 #pragma unroll 4
     for (int key = 0; key < S::HK; ++key) {
-      uint64_t v[S::CT / 2];
+      uint64_t v[S::CT];
       if constexpr (S::CT == 4) {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(m + key * S::LD);
-        v[0] = t.x;
-        v[1] = t.y;
+        const float4 t = *reinterpret_cast<const float4*>(m + key * S::LD);
+        v[0] = f2pack(t.x, t.x);
+        v[1] = f2pack(t.y, t.y);
+        v[2] = f2pack(t.z, t.z);
+        v[3] = f2pack(t.w, t.w);
       } else {
-        v[0] = *reinterpret_cast<const uint64_t*>(m + key * S::LD);
+        const float2 t = *reinterpret_cast<const float2*>(m + key * S::LD);
+        v[0] = f2pack(t.x, t.x);
+        v[1] = f2pack(t.y, t.y);
       }
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pp + key * S::PB);
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(pp + key * S::PB + 4);
 #pragma unroll
-      for (int i = 0; i < 8; i += 2) {
-        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pp + key * S::PB + 2 * i);
-#pragma unroll
-        for (int c = 0; c < S::CT / 2; ++c) {
-          acc[i][c] = ffma2(a.x, v[c], acc[i][c]);
-          acc[i + 1][c] = ffma2(a.y, v[c], acc[i + 1][c]);
-        }
+      for (int c = 0; c < S::CT; ++c) {
+        acc[0][c] = ffma2(a.x, v[c], acc[0][c]);
+        acc[1][c] = ffma2(a.y, v[c], acc[1][c]);
+        acc[2][c] = ffma2(b.x, v[c], acc[2][c]);
+        acc[3][c] = ffma2(b.y, v[c], acc[3][c]);
       }
     }
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int c = 0; c < S::CT / 2; ++c) out[i][c] = fadd2(out[i][c], acc[i][c]);
+    for (int c = 0; c < S::CT; ++c) out[i][c] = fadd2(out[i][c], acc[i][c]);
 }
 
-// CT accumulated columns of one row, times mul, to the output row or the slot row
-template <int CT, typename T>
-__device__ __forceinline__ void store_cols(T* dst, const uint64_t (&a)[CT / 2], float mul) {
-  float x[CT];
+template <class S>
+__device__ __forceinline__ void zero_acc(Acc<S>& a) {
 #pragma unroll
-  for (int c = 0; c < CT / 2; ++c) f2unpack(a[c], x[2 * c], x[2 * c + 1]);
-  if constexpr (CT == 4) {
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < S::CT; ++c) a[i][c] = 0;
+}
+
+// the CT accumulated columns of row i, times mul, to the output row or the slot row
+template <class S, typename T>
+__device__ __forceinline__ void store_cols(T* dst, const Acc<S>& a, int i, float mul) {
+  float x[S::CT];
+#pragma unroll
+  for (int c = 0; c < S::CT; ++c) {
+    float u, v;
+    f2unpack(a[i >> 1][c], u, v);
+    x[c] = i & 1 ? v : u;
+  }
+  if constexpr (S::CT == 4) {
     store4<T>(dst, make_float4(x[0] * mul, x[1] * mul, x[2] * mul, x[3] * mul));
   } else if constexpr (sizeof(T) == 2) {
     *reinterpret_cast<__nv_bfloat162*>(dst) = __floats2bfloat162_rn(x[0] * mul, x[1] * mul);
@@ -215,7 +240,7 @@ struct FwdSmem {
 };
 
 template <class S, typename OutT>
-__global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const float* __restrict__ Q,
+__global__ void __launch_bounds__(S::T, S::CTAS) simt_fwd_kernel(const Geom g, const float* __restrict__ Q,
                                                         const float* __restrict__ K, const float* __restrict__ V,
                                                         OutT* __restrict__ out, float* __restrict__ lse2,
                                                         float* __restrict__ ot) {
@@ -236,14 +261,13 @@ __global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const floa
   const int r0 = warp * S::WR + rg * 8;  // first of this thread's 8 rows within the CTA
   float* pb = sm.p[warp];
 
-  uint64_t o[8][S::CT / 2];
+  Acc<S> o;
+  zero_acc<S>(o);
   float m[8], l[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     m[i] = -INFINITY;
     l[i] = 0.f;
-#pragma unroll
-    for (int c = 0; c < S::CT / 2; ++c) o[i][c] = 0;
   }
   for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
     cp_wait<0>();
@@ -261,13 +285,14 @@ __global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const floa
 #pragma unroll
       for (int i = 0; i < 8; ++i) s[i][j] = in ? s[i][j] * g.scale_log2 : -INFINITY;
     }
+    float alpha[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       float mx = s[i][0];
 #pragma unroll
       for (int j = 1; j < S::KT; ++j) mx = fmaxf(mx, s[i][j]);
       mx = fmaxf(m[i], group_max<S::LG>(mx));
-      const float alpha = exp2f(m[i] - mx);  // 0 on the first block (m = -inf)
+      alpha[i] = exp2f(m[i] - mx);  // 0 on the first block (m = -inf)
       m[i] = mx;
       float lc = 0.f;
 #pragma unroll
@@ -275,11 +300,12 @@ __global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const floa
         s[i][j] = exp2f(s[i][j] - mx);
         lc += s[i][j];
       }
-      l[i] = l[i] * alpha + lc;  // this thread's keys; the group's sums are added at the end
-      const uint64_t a2 = f2pack(alpha, alpha);
-#pragma unroll
-      for (int c = 0; c < S::CT / 2; ++c) o[i][c] = fmul2(o[i][c], a2);
+      l[i] = l[i] * alpha[i] + lc;  // this thread's keys; the group's sums are added at the end
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < S::CT; ++c) o[i][c] = fmul2(o[i][c], f2pack(alpha[2 * i], alpha[2 * i + 1]));
     axpys<S>(s, sm.v[b], pb, rg, lg, o);
   }
 #pragma unroll
@@ -293,8 +319,8 @@ __global__ void __launch_bounds__(S::T) simt_fwd_kernel(const Geom g, const floa
     const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
     if (lg == 0) lse2[slot] = m[i] + log2f(ls);
     const float inv = 1.f / ls;
-    if (only_cover(g, tb, p)) store_cols<S::CT>(out + base + tok * S::D + S::CT * lg, o[i], inv);
-    else store_cols<S::CT>(ot + slot * S::D + S::CT * lg, o[i], inv);
+    if (only_cover(g, tb, p)) store_cols<S>(out + base + tok * S::D + S::CT * lg, o, i, inv);
+    else store_cols<S>(ot + slot * S::D + S::CT * lg, o, i, inv);
   }
 }
 
@@ -313,7 +339,7 @@ struct DqSmem {
 };
 
 template <class S, typename OutT>
-__global__ void __launch_bounds__(S::T) simt_dq_kernel(const Geom g, const float* __restrict__ Q,
+__global__ void __launch_bounds__(S::T, S::CTAS) simt_dq_kernel(const Geom g, const float* __restrict__ Q,
                                                        const float* __restrict__ K, const float* __restrict__ V,
                                                        const float* __restrict__ dO, const float* __restrict__ lse2c,
                                                        const float* __restrict__ dd, OutT* __restrict__ dq,
@@ -348,11 +374,8 @@ __global__ void __launch_bounds__(S::T) simt_dq_kernel(const Geom g, const float
       nD[i] = dd[slot];
     }
   }
-  uint64_t acc[8][S::CT / 2];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int c = 0; c < S::CT / 2; ++c) acc[i][c] = 0;
+  Acc<S> acc;
+  zero_acc<S>(acc);
   for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
     const bool more = j0 + kBN < tb.L;
     cp_wait<0>();
@@ -385,8 +408,8 @@ __global__ void __launch_bounds__(S::T) simt_dq_kernel(const Geom g, const float
     int lr[3];
     const int64_t tok = row_token(g, tb, r, lr);
     const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
-    if (only_cover(g, tb, p)) store_cols<S::CT>(dq + base + tok * S::D + S::CT * lg, acc[i], g.scale);
-    else store_cols<S::CT>(dq_s + slot_of(g, bh, tile, tb.e, lr) * S::D + S::CT * lg, acc[i], g.scale);
+    if (only_cover(g, tb, p)) store_cols<S>(dq + base + tok * S::D + S::CT * lg, acc, i, g.scale);
+    else store_cols<S>(dq_s + slot_of(g, bh, tile, tb.e, lr) * S::D + S::CT * lg, acc, i, g.scale);
   }
 }
 
@@ -405,7 +428,7 @@ struct DkvSmem {
 };
 
 template <class S, typename OutT>
-__global__ void __launch_bounds__(S::T) simt_dkdv_kernel(const Geom g, const float* __restrict__ Q,
+__global__ void __launch_bounds__(S::T, S::CTAS) simt_dkdv_kernel(const Geom g, const float* __restrict__ Q,
                                                          const float* __restrict__ K, const float* __restrict__ V,
                                                          const float* __restrict__ dO, const float* __restrict__ lse2c,
                                                          const float* __restrict__ dd, OutT* __restrict__ dk,
@@ -443,11 +466,9 @@ __global__ void __launch_bounds__(S::T) simt_dkdv_kernel(const Geom g, const flo
   cp_commit();
   stats(0, 0);
   const int r0 = warp * S::WR + rg * 8;
-  uint64_t adk[8][S::CT / 2], adv[8][S::CT / 2];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int c = 0; c < S::CT / 2; ++c) adk[i][c] = adv[i][c] = 0;
+  Acc<S> adk, adv;
+  zero_acc<S>(adk);
+  zero_acc<S>(adv);
   for (int i0 = 0, b = 0; i0 < tb.L; i0 += kBN, b ^= 1) {
     const bool more = i0 + kBN < tb.L;
     cp_wait<0>();
@@ -487,12 +508,12 @@ __global__ void __launch_bounds__(S::T) simt_dkdv_kernel(const Geom g, const flo
     const int64_t tok = row_token(g, tb, r, lr);
     const int p[3] = {tb.lo[0] + lr[0], tb.lo[1] + lr[1], tb.lo[2] + lr[2]};
     if (only_cover(g, tb, p)) {
-      store_cols<S::CT>(dk + base + tok * S::D + S::CT * lg, adk[i], g.scale);
-      store_cols<S::CT>(dv + base + tok * S::D + S::CT * lg, adv[i], 1.f);
+      store_cols<S>(dk + base + tok * S::D + S::CT * lg, adk, i, g.scale);
+      store_cols<S>(dv + base + tok * S::D + S::CT * lg, adv, i, 1.f);
     } else {
       const int64_t slot = slot_of(g, bh, tile, tb.e, lr);
-      store_cols<S::CT>(dk_s + slot * S::D + S::CT * lg, adk[i], g.scale);
-      store_cols<S::CT>(dv_s + slot * S::D + S::CT * lg, adv[i], 1.f);
+      store_cols<S>(dk_s + slot * S::D + S::CT * lg, adk, i, g.scale);
+      store_cols<S>(dv_s + slot * S::D + S::CT * lg, adv, i, 1.f);
     }
   }
 }
@@ -534,15 +555,17 @@ cudaError_t bwd_run(const Geom& g, const float* q, const float* k, const float* 
   return cudaGetLastError();
 }
 
-// Runs f with the shape for this problem: BM = 64 rows a CTA (a staged block
-// serves twice the rows of BM = 32), or 32 where 64-row blocks would leave SMs
-// without a CTA.
+// Runs f with the shape for this problem.  64-row CTAs of warps with 16 rows
+// (8 x 4 score tiles a thread: fewest shared-memory reads per FMA), or, where
+// those would leave SMs without a CTA, 32-row CTAs of warps with 8 rows (8 x 2
+// tiles, twice the warps: a training step on one head of a 64 x 64 frame 285
+// us, 16-row warps 311; the 8-row form costs large problems 15 %).
 template <int D, typename F>
 cudaError_t with_shape(const Geom& g, F f) {
-  constexpr int W64 = D == 128 ? 8 : 4;
   const int64_t blocks = (int64_t)((g.Lmax + 63) / 64) * g.ntiles * g.B * g.nh;
-  if (blocks > num_sms()) return f(Shape<D, W64>());
-  return f(Shape<D, W64 / 2>());
+  if constexpr (D == 128) return blocks > num_sms() ? f(Shape<D, 8, 1>()) : f(Shape<D, 4, 1>());
+  else if constexpr (D == 64) return blocks > num_sms() ? f(Shape<D, 4, 2>()) : f(Shape<D, 4, 1>());
+  else return blocks > num_sms() ? f(Shape<D, 4, 2>()) : f(Shape<D, 2, 2>());
 }
 
 template <typename F>
