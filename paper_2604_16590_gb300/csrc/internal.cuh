@@ -118,7 +118,10 @@ cudaError_t launch_merge_fwd(const Geom& g, const float* ot, void* out, int out_
 // factorised linear attention (linear.cu): split-N summary over chunks of
 // 128-token tiles, fixed-order combine, query pass; BF16, d = 64.
 struct LinearPlan {
-  int ntiles, chunk_tiles, chunks, q_tiles_per_cta;
+  int ntiles;
+  int chunk_tiles, chunks;      // summary
+  int q_tiles;                  // query pass, tiles per CTA
+  int b_chunk_tiles, b_chunks;  // both backward passes
 };
 LinearPlan linear_plan(int B, int nh, int64_t N);
 // Forward workspace: per-chunk FP32 partials of S and z, then the combined

@@ -92,6 +92,27 @@ __device__ __forceinline__ void split8(const float (&f)[8], uint4& hi, uint4& lo
   hi = make_uint4(h[0], h[1], h[2], h[3]);
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
+// Sums of the 64 columns of a ROWS x 64 matrix in shared memory by THREADS math
+// threads (named barrier 1), in a fixed order: thread t adds every
+// (THREADS / 64)-th row of column t % 64, then threads 0..63 add those.  The
+// result is in threads 0..63.  Rows 0.. of the matrix are overwritten.
+template <int THREADS, int ROWS>
+__device__ __forceinline__ float column_sum(float* m, int t) {
+  constexpr int P = THREADS / 64;
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");  // the rows are written
+  float s = 0.f;
+#pragma unroll 8
+  for (int i = t / 64; i < ROWS; i += P) s += m[i * 64 + (t & 63)];
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");  // the rows are read
+  m[t] = s;
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (t >= 64) return 0.f;
+  s = 0.f;
+#pragma unroll
+  for (int p = 0; p < P; ++p) s += m[p * 64 + t];
+  return s;
+}
+
 struct SumArgs {
   int N, BH, ntiles, chunk_tiles;
   float* ws_S;  // [chunks, BH, 64, 64]
@@ -229,19 +250,34 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
 #pragma unroll
       for (int i = 0; i < kD / 2; ++i) zbuf[r * kD + 32 * h + i] = zacc[i];
     }
-    asm volatile("bar.sync 1, 256;" ::: "memory");  // the eight math warps only
-    const int tid = threadIdx.x - 64;
-    if (got && tid < kD) {
-      float s = 0.f;
-      for (int i = 0; i < kTile; ++i) s += zbuf[i * kD + tid];
-      a.ws_z[part * kD + tid] = s;
-    }
+    const float zs = column_sum<256, kTile>(zbuf, threadIdx.x - 64);
+    if (got && threadIdx.x - 64 < kD) a.ws_z[part * kD + threadIdx.x - 64] = zs;
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 64);
+  }
+}
+
+// Kahan-compensated sum of n values a `stride` apart in ascending order, the
+// loads sixteen at a time: few heads make many chunks, and with one load in
+// flight the combine of one head took longer than a tenth of the call.
+__device__ __forceinline__ void kahan_chunks(const float* __restrict__ src, size_t stride, int n, float& sum,
+                                             float& comp) {
+  for (int c0 = 0; c0 < n; c0 += 16) {
+    float x[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = c0 + i < n ? __ldg(src + (size_t)(c0 + i) * stride) : 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (c0 + i >= n) break;
+      const float y = x[i] - comp;
+      const float t = sum + y;
+      comp = (t - sum) - y;
+      sum = t;
+    }
   }
 }
 
@@ -260,14 +296,8 @@ __global__ void __launch_bounds__(256) la_combine_kernel(const CombArgs a) {
   for (int e = blockIdx.y * 256 + threadIdx.x; e < kD * kD + kD; e += 256 * gridDim.y) {
     const bool is_z = e >= kD * kD;
     float sum = 0.f, comp = 0.f;  // Kahan
-    for (int c = 0; c < a.chunks; ++c) {
-      const size_t part = (size_t)c * a.BH + bh;
-      const float x = is_z ? a.ws_z[part * kD + (e - kD * kD)] : a.ws_S[part * kD * kD + e];
-      const float y = x - comp;
-      const float t = sum + y;
-      comp = (t - sum) - y;
-      sum = t;
-    }
+    const float* src = is_z ? a.ws_z + (size_t)bh * kD + (e - kD * kD) : a.ws_S + (size_t)bh * kD * kD + e;
+    kahan_chunks(src, (size_t)a.BH * (is_z ? kD : kD * kD), a.chunks, sum, comp);
     if (is_z) {
       a.zt[(size_t)bh * kD + (e - kD * kD)] = sum;
     } else {
@@ -843,12 +873,8 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
         *reinterpret_cast<float2*>(zbuf + (grp * kTile + r) * kD + 32 * h + 2 * i) = make_float2(x, y);
       }
     }
-    asm volatile("bar.sync 1, 512;" ::: "memory");
-    if (got && tid < kD) {
-      float sum = 0.f;
-      for (int i = 0; i < 2 * kTile; ++i) sum += zbuf[i * kD + tid];
-      a.part_dz[part * kD + tid] = sum;
-    }
+    const float sum = column_sum<512, 2 * kTile>(zbuf, tid);
+    if (got && tid < kD) a.part_dz[part * kD + tid] = sum;
     if (lane == 0) bulk_wait_all();
   }
   tc_fence_before();
@@ -875,14 +901,8 @@ __global__ void __launch_bounds__(256) la_bwd_combine_kernel(const BCombArgs a) 
   for (int e = blockIdx.y * 256 + threadIdx.x; e < kD * kD + kD; e += 256 * gridDim.y) {
     const bool is_z = e >= kD * kD;
     float sum = 0.f, comp = 0.f;
-    for (int c = 0; c < a.chunks; ++c) {
-      const size_t part = (size_t)c * a.BH + bh;
-      const float x = is_z ? a.part_dz[part * kD + (e - kD * kD)] : a.part_dS[part * kD * kD + e];
-      const float y = x - comp;
-      const float t = sum + y;
-      comp = (t - sum) - y;
-      sum = t;
-    }
+    const float* src = is_z ? a.part_dz + (size_t)bh * kD + (e - kD * kD) : a.part_dS + (size_t)bh * kD * kD + e;
+    kahan_chunks(src, (size_t)a.BH * (is_z ? kD : kD * kD), a.chunks, sum, comp);
     if (is_z) {
       a.dz[(size_t)bh * kD + (e - kD * kD)] = sum;
     } else {
@@ -1132,15 +1152,39 @@ constexpr int kQSmem = 16384 + (kQStages + 1) * kTileBytes + 1024 + 512;
 
 }  // namespace
 
+// Tiles per CTA for BH heads of `ntiles` tiles on `slots` resident CTAs: the
+// fewest waves (up to four) that leave at most 5 % of the slots empty, else the
+// fullest.  Every CTA pays for its tensor memory, its operand matrices and the
+// fill of its ring, and the split-N passes for a partial that the combine reads
+// (forward and backward, one head of 1.5 M tokens: 1087 -> 484 us with the
+// sixteen-load combine, half of it from the combines; 16 heads of 262144:
+// 1360 -> 1164; before, 1216 CTAs or 16 tiles each whatever the problem).
+static int tiles_per_cta(int ntiles, int BH, int slots) {
+  int best = 1;
+  double full = 0.0;
+  for (int w = 1; w <= 4; ++w) {
+    const int want = slots * w / BH;  // CTAs per head
+    const int per = want < 1 ? ntiles : (ntiles + want - 1) / want;
+    const int ctas = (ntiles + per - 1) / per * BH;
+    const double f = (double)ntiles * BH / ((double)per * slots * ((ctas + slots - 1) / slots));
+    if (f > full + 1e-9) {
+      full = f;
+      best = per;
+    }
+    if (full >= 0.95) break;
+  }
+  return best;
+}
+
 LinearPlan linear_plan(int B, int nh, int64_t N) {
   LinearPlan p;
+  const int BH = B * nh;
   p.ntiles = (int)((N + kTile - 1) / kTile);
-  const int64_t units = (int64_t)p.ntiles * B * nh;
-  int64_t ct = (units + 304 * 4 - 1) / (304 * 4);
-  if (ct < 1) ct = 1;
-  p.chunk_tiles = (int)ct;
-  p.chunks = (int)((p.ntiles + ct - 1) / ct);
-  p.q_tiles_per_cta = 16;
+  p.chunk_tiles = tiles_per_cta(p.ntiles, BH, 304);  // two CTAs per SM
+  p.chunks = (p.ntiles + p.chunk_tiles - 1) / p.chunk_tiles;
+  p.q_tiles = tiles_per_cta(p.ntiles, BH, 456);      // three
+  p.b_chunk_tiles = tiles_per_cta(p.ntiles, BH, 152);  // one, as the key pass
+  p.b_chunks = (p.ntiles + p.b_chunk_tiles - 1) / p.b_chunk_tiles;
   return p;
 }
 
@@ -1184,7 +1228,7 @@ cudaError_t launch_linear(const void* q, const void* k, const void* v, void* out
   qa.N = (int)N;
   qa.BH = BH;
   qa.ntiles = p.ntiles;
-  qa.tiles_per_cta = p.q_tiles_per_cta;
+  qa.tiles_per_cta = p.q_tiles;
   qa.sth = ca.sth;
   qa.stl = ca.stl;
   qa.zt = ca.zt;
@@ -1211,7 +1255,7 @@ cudaError_t launch_linear(const void* q, const void* k, const void* v, void* out
   prof_end(kKLinearCombine, st);
   if (e != cudaSuccess) return e;
   prof_begin(kKLinearQuery, st);
-  la_query_kernel<<<dim3((p.ntiles + p.q_tiles_per_cta - 1) / p.q_tiles_per_cta, BH), kThreadsQ, kQSmem, st>>>(mq, mo,
+  la_query_kernel<<<dim3((p.ntiles + p.q_tiles - 1) / p.q_tiles, BH), kThreadsQ, kQSmem, st>>>(mq, mo,
                                                                                                              qa);
   e = cudaGetLastError();
   prof_end(kKLinearQuery, st);
@@ -1223,8 +1267,8 @@ LinearBwdLayout linear_bwd_layout(int B, int nh, int64_t N) {
   const size_t BH = (size_t)B * nh;
   LinearBwdLayout l;
   l.part_dS = 0;
-  l.part_dz = l.part_dS + align_up((size_t)p.chunks * BH * kD * kD * 4);
-  l.dsh = l.part_dz + align_up((size_t)p.chunks * BH * kD * 4);
+  l.part_dz = l.part_dS + align_up((size_t)p.b_chunks * BH * kD * kD * 4);
+  l.dsh = l.part_dz + align_up((size_t)p.b_chunks * BH * kD * 4);
   l.dsl = l.dsh + align_up(BH * kD * kD * 2);
   l.dsth = l.dsl + align_up(BH * kD * kD * 2);
   l.dstl = l.dsth + align_up(BH * kD * kD * 2);
@@ -1245,7 +1289,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   qa.N = (int)N;
   qa.BH = BH;
   qa.ntiles = p.ntiles;
-  qa.chunk_tiles = p.chunk_tiles;
+  qa.chunk_tiles = p.b_chunk_tiles;
   qa.sth = reinterpret_cast<const __nv_bfloat16*>(sv + fl.sth);
   qa.stl = reinterpret_cast<const __nv_bfloat16*>(sv + fl.stl);
   qa.zt = reinterpret_cast<const float*>(sv + fl.z);
@@ -1254,7 +1298,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   qa.part_dz = reinterpret_cast<float*>(w + bl.part_dz);
   BCombArgs ca;
   ca.BH = BH;
-  ca.chunks = p.chunks;
+  ca.chunks = p.b_chunks;
   ca.part_dS = qa.part_dS;
   ca.part_dz = qa.part_dz;
   ca.dsh = reinterpret_cast<__nv_bfloat16*>(w + bl.dsh);
@@ -1266,7 +1310,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   ka.N = (int)N;
   ka.BH = BH;
   ka.ntiles = p.ntiles;
-  ka.tiles_per_cta = p.q_tiles_per_cta;
+  ka.tiles_per_cta = p.b_chunk_tiles;
   ka.dsh = ca.dsh;
   ka.dsl = ca.dsl;
   ka.dsth = ca.dsth;
@@ -1288,7 +1332,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
           cudaSuccess)
     return e;
   prof_begin(kKLinearBwdQuery, st);
-  la_bwd_query_kernel<<<dim3(p.chunks, BH), kThreadsB, kBQSmem, st>>>(mq, mg, mdq, qa);
+  la_bwd_query_kernel<<<dim3(p.b_chunks, BH), kThreadsB, kBQSmem, st>>>(mq, mg, mdq, qa);
   e = cudaGetLastError();
   prof_end(kKLinearBwdQuery, st);
   if (e != cudaSuccess) return e;
@@ -1298,7 +1342,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   prof_end(kKLinearBwdCombine, st);
   if (e != cudaSuccess) return e;
   prof_begin(kKLinearBwdKey, st);
-  la_bwd_key_kernel<<<dim3((p.ntiles + p.q_tiles_per_cta - 1) / p.q_tiles_per_cta, BH), kThreadsB, kBKSmem, st>>>(
+  la_bwd_key_kernel<<<dim3(p.b_chunks, BH), kThreadsB, kBKSmem, st>>>(
       mk, mv, mdk, mdv, ka);
   e = cudaGetLastError();
   prof_end(kKLinearBwdKey, st);
