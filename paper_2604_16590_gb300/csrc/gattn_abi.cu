@@ -352,11 +352,13 @@ gattn_status gattn_bwd(const gattn_desc* desc, const void* q, const void* k, con
   float* dd = reinterpret_cast<float*>(w + bl.dd_off);
   // the statistics rows are read only by the tensor-core dK/dV kernels
   void* ext = desc->in_dtype == GATTN_BF16 ? static_cast<void*>(w + bl.ext_off) : nullptr;
+  int32_t* dst = ext ? reinterpret_cast<int32_t*>(w + bl.dst_off) : nullptr;
+  int32_t* nbt = ext ? reinterpret_cast<int32_t*>(w + bl.nbt_off) : nullptr;
   float* dq_s = reinterpret_cast<float*>(w + bl.dq_off);
   float* dk_s = reinterpret_cast<float*>(w + bl.dk_off);
   float* dv_s = reinterpret_cast<float*>(w + bl.dv_off);
   prof_begin(kKBwdPrep, st);
-  cudaError_t e = launch_bwd_prep(g, out, desc->out_dtype, dout, desc->in_dtype, lse2, ot, lse2c, dd, ext, st);
+  cudaError_t e = launch_bwd_prep(g, out, desc->out_dtype, dout, desc->in_dtype, lse2, ot, lse2c, dd, ext, dst, nbt, st);
   prof_end(kKBwdPrep, st);
   if (e != cudaSuccess) return GATTN_ERR_CUDA;
   if (desc->in_dtype == GATTN_FP32)
@@ -364,7 +366,7 @@ gattn_status gattn_bwd(const gattn_desc* desc, const void* q, const void* k, con
                         dv, desc->out_dtype, dq_s, dk_s, dv_s, st);
   else
     e = launch_sm103_bwd(g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                         (const __nv_bfloat16*)dout, lse2c, dd, ext, dq, dk, dv, desc->out_dtype, dq_s, dk_s, dv_s,
+                         (const __nv_bfloat16*)dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, desc->out_dtype, dq_s, dk_s, dv_s,
                          desc->flags, st);
   if (e == cudaErrorNotSupported) return GATTN_ERR_UNSUPPORTED;
   if (e != cudaSuccess) return GATTN_ERR_CUDA;

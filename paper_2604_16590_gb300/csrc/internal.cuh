@@ -34,11 +34,14 @@ inline SavedLayout saved_layout(const Geom& g) {
 //   lse2c : float[S]      -(log2-domain LSE - log2(w_t / sum w)) (folds the dO_t scaling into P), negated
 //   dd    : float[S]      -D, D = dOut . O_t per slot, negated
 //   dq_s, dk_s, dv_s : float[S * d]  per-tile gradients of multiply-covered rows
+//   dst   : int32[S]      where a slot's output row goes: the token of a row covered by one tile, -2 for a
+//                          multiply-covered row (its slot), -1 for a slot outside the tile (tensor-core form only)
+//   nbt   : int32[ntiles] boxes of each tile
 //   ext   : 16 B[S]       BF16 row (x0, x1, x2, y0, y1, y2, 0, 0) per slot: x0 + x1 + x2 = -lse' / (scale
 //                          log2 e) and y0 + y1 + y2 = -D, each split into three BF16 terms; the BF16
 //                          dK/dV kernels add both to S^T and dP^T with one extra K = 16 MMA step each
 struct BwdLayout {
-  size_t S, lse_off, dd_off, ext_off, dq_off, dk_off, dv_off, bytes;
+  size_t S, lse_off, dd_off, dst_off, nbt_off, ext_off, dq_off, dk_off, dv_off, bytes;
 };
 inline BwdLayout bwd_layout(const Geom& g) {
   BwdLayout b;
@@ -47,8 +50,10 @@ inline BwdLayout bwd_layout(const Geom& g) {
   size_t mat = align_up(b.S * g.d * sizeof(float));
   b.lse_off = 0;
   b.dd_off = vec;
-  b.ext_off = 2 * vec;
-  b.dq_off = 2 * vec + align_up(b.S * 16);
+  b.dst_off = 2 * vec;
+  b.nbt_off = 3 * vec;
+  b.ext_off = b.nbt_off + align_up((size_t)g.ntiles * sizeof(int32_t));
+  b.dq_off = b.ext_off + align_up(b.S * 16);
   b.dk_off = b.dq_off + mat;
   b.dv_off = b.dk_off + mat;
   b.bytes = b.dv_off + mat;
@@ -154,7 +159,7 @@ cudaError_t launch_gated_mix(const Geom& g, void* out, const void* cross, const 
                              cudaStream_t st);
 cudaError_t launch_bwd_prep(const Geom& g, const void* out, int out_dtype, const void* dout,
                             int in_dtype, const float* lse2, const float* ot, float* lse2c, float* dd,
-                            void* ext, cudaStream_t st);
+                            void* ext, int32_t* dst, int32_t* nbt, cudaStream_t st);
 cudaError_t launch_merge_bwd(const Geom& g, const float* dq_s, const float* dk_s, const float* dv_s,
                              void* dq, void* dk, void* dv, int out_dtype, cudaStream_t st);
 cudaError_t launch_sm103_fwd(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
@@ -165,12 +170,14 @@ cudaError_t launch_sm103_fwd64(const Geom& g, const __nv_bfloat16* q, const __nv
                                uint32_t flags, cudaStream_t st);
 cudaError_t launch_sm103_bwd(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
                              const __nv_bfloat16* v, const __nv_bfloat16* dout, const float* lse2c,
-                             const float* dd, const void* ext, void* dq, void* dk, void* dv, int out_dtype,
-                             float* dq_s, float* dk_s, float* dv_s, uint32_t flags, cudaStream_t st);
+                             const float* dd, const void* ext, const int32_t* dst, const int32_t* nbt, void* dq,
+                             void* dk, void* dv, int out_dtype, float* dq_s, float* dk_s, float* dv_s, uint32_t flags,
+                             cudaStream_t st);
 cudaError_t launch_sm103_bwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k,
                                const __nv_bfloat16* v, const __nv_bfloat16* dout, const float* lse2c,
-                               const float* dd, const void* ext, void* dq, void* dk, void* dv, int out_dtype,
-                               float* dq_s, float* dk_s, float* dv_s, cudaStream_t st);
+                               const float* dd, const void* ext, const int32_t* dst, const int32_t* nbt, void* dq,
+                               void* dk, void* dv, int out_dtype, float* dq_s, float* dk_s, float* dv_s,
+                               cudaStream_t st);
 
 // ---- ragged (multi-request) forward, used by the serving engine.
 // One descriptor per active request, in device memory, sorted by item0: the

@@ -359,7 +359,8 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
                                                             const float* __restrict__ lse2,
                                                             const float* __restrict__ ot,
                                                             float* __restrict__ lse2c, float* __restrict__ dd,
-                                                            uint4* __restrict__ ext) {
+                                                            uint4* __restrict__ ext, int32_t* __restrict__ dst,
+                                                            int32_t* __restrict__ nbt) {
   constexpr int L = D >= 64 ? 8 : 4;  // lanes per row
   constexpr int U = D / (8 * L);      // 8-column units per lane
   constexpr int RPI = 32 / L;         // rows per load step
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
     tile_box(g, tile, tb);
     int lr[3];
     const bool valid = slot_local(g, tb.e, within >> 7, within & 127, lr);
-    int64_t row = 0;  // token row, or -1 - slot for a multiply-covered row
+    int64_t row = 0;  // token row
     bool single = true;
     float lc = 0.f;
     if (valid) {
@@ -446,7 +447,13 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
     // finite, the extension MMA multiplies it by the other statistic's zero weights
     lse2c[slot] = valid ? -lc : -INFINITY;
     dd[slot] = valid ? -part : 0.f;
-    if (ext) ext[slot] = valid ? stat_row(-lc / g.scale_log2, -part) : stat_row(-1e30f, 0.f);
+    if (ext) {  // tensor-core form
+      ext[slot] = valid ? stat_row(-lc / g.scale_log2, -part) : stat_row(-1e30f, 0.f);
+      dst[slot] = !valid ? -1 : single ? (int32_t)(row - (int64_t)bh * g.N) : -2;
+      if (bh == 0 && within == 0)
+        nbt[tile] = fdiv(tb.e[0] + g.bt - 1, g.fb[0]) * fdiv(tb.e[1] + g.by - 1, g.fb[1]) *
+                    fdiv(tb.e[2] + g.bx - 1, g.fb[2]);
+    }
   }
 }
 
@@ -542,25 +549,25 @@ cudaError_t launch_merge_fwd(const Geom& g, const float* ot, void* out, int out_
 
 template <typename OutT, typename InT>
 static void run_bwd_prep(const Geom& g, const void* out, const void* dout, const float* lse2, const float* ot,
-                         float* lse2c, float* dd, uint4* ext, cudaStream_t st) {
+                         float* lse2c, float* dd, uint4* ext, int32_t* dst, int32_t* nbt, cudaStream_t st) {
   const unsigned grid = grid_for((int64_t)g.B * g.nh * g.ntiles * g.per_tile);
   const OutT* o = static_cast<const OutT*>(out);
   const InT* d = static_cast<const InT*>(dout);
-  if (g.d == 128) bwd_prep_kernel<OutT, InT, 128><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext);
-  else if (g.d == 64) bwd_prep_kernel<OutT, InT, 64><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext);
+  if (g.d == 128) bwd_prep_kernel<OutT, InT, 128><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext, dst, nbt);
+  else if (g.d == 64) bwd_prep_kernel<OutT, InT, 64><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext, dst, nbt);
   else if constexpr (sizeof(InT) == 4)  // d = 32: FP32 inputs only
-    bwd_prep_kernel<OutT, InT, 32><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext);
+    bwd_prep_kernel<OutT, InT, 32><<<grid, kThreads, 0, st>>>(g, o, d, lse2, ot, lse2c, dd, ext, dst, nbt);
 }
 
 cudaError_t launch_bwd_prep(const Geom& g, const void* out, int out_dtype, const void* dout, int in_dtype,
-                            const float* lse2, const float* ot, float* lse2c, float* dd, void* ext_,
-                            cudaStream_t st) {
+                            const float* lse2, const float* ot, float* lse2c, float* dd, void* ext_, int32_t* dst,
+                            int32_t* nbt, cudaStream_t st) {
   uint4* ext = static_cast<uint4*>(ext_);
   using bf = __nv_bfloat16;
-  if (out_dtype == GATTN_BF16 && in_dtype == GATTN_BF16) run_bwd_prep<bf, bf>(g, out, dout, lse2, ot, lse2c, dd, ext, st);
-  else if (out_dtype == GATTN_BF16) run_bwd_prep<bf, float>(g, out, dout, lse2, ot, lse2c, dd, ext, st);
-  else if (in_dtype == GATTN_BF16) run_bwd_prep<float, bf>(g, out, dout, lse2, ot, lse2c, dd, ext, st);
-  else run_bwd_prep<float, float>(g, out, dout, lse2, ot, lse2c, dd, ext, st);
+  if (out_dtype == GATTN_BF16 && in_dtype == GATTN_BF16) run_bwd_prep<bf, bf>(g, out, dout, lse2, ot, lse2c, dd, ext, dst, nbt, st);
+  else if (out_dtype == GATTN_BF16) run_bwd_prep<bf, float>(g, out, dout, lse2, ot, lse2c, dd, ext, dst, nbt, st);
+  else if (in_dtype == GATTN_BF16) run_bwd_prep<float, bf>(g, out, dout, lse2, ot, lse2c, dd, ext, dst, nbt, st);
+  else run_bwd_prep<float, float>(g, out, dout, lse2, ot, lse2c, dd, ext, dst, nbt, st);
   return cudaGetLastError();
 }
 

@@ -290,13 +290,11 @@ __global__ void __launch_bounds__(kThreadsB, 1)
     const uint64_t s2 = f2pack(g.scale_log2, g.scale_log2);
     uint32_t G = 0, W = 0;
     bool ok = true;
-    for (int w = blockIdx.x; w < a.items && ok; w += gridDim.x) {
-      int bh, tile, kb;
-      decode_item(g, w, bh, tile, kb);
-      TileBlocks tbk;
-      tile_blocks(g, tile, tbk);
-      if (kb >= tbk.NB) continue;
-      for (int i = 0; i < tbk.NB && ok; ++i, ++G) {
+    int w = blockIdx.x;
+    int nb = next_boxes(a, w);
+    while (nb > 0) {
+      const int place = a.dst[(int64_t)w * 128 + row];  // slots of an item: w * 128 ...
+      for (int i = 0; i < nb && ok; ++i, ++G) {
         if (!(ok = WAIT(s_full, G & 1))) break;
         tc_fence_after();
         uint32_t sv[32], dv[32], pk[16];
@@ -320,16 +318,11 @@ __global__ void __launch_bounds__(kThreadsB, 1)
         if (lane == 0) mbar_arrive(p_full + 1);
       }
       if (!ok) break;
-      // ---- where this thread's key row goes, while the last gradient products run
-      int ko[3], kl[3];
-      block_origin(g, tbk, kb, ko);
-      block_row(g, ko, row, kl);
-      const bool kvalid = inside(tbk, kl);
-      const int p[3] = {tbk.tb.lo[0] + kl[0], tbk.tb.lo[1] + kl[1], tbk.tb.lo[2] + kl[2]};
-      const bool single = kvalid && only_cover(g, tbk.tb, p);
-      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const int64_t off = ((int64_t)bh * g.N + tok) * kD + c4 * 32;
-      const int64_t slots = (tile_slot0(g, bh, tile) + kb * 128 + quad * 32) * kD + c4 * 32;
+      const bool kvalid = place != -1, single = place >= 0;
+      const int64_t off = (single ? ((int64_t)item_bh(g, w) * g.N + place) * kD : 0) + c4 * 32;
+      const int64_t slots = ((int64_t)w * 128 + quad * 32) * kD + c4 * 32;
+      w += gridDim.x;
+      nb = next_boxes(a, w);
       // ---- epilogue: columns [32 c4, 32 c4 + 32) of dK, then of dV
       if (!(ok = WAIT(acc_full, W & 1))) break;
       tc_fence_after();
@@ -622,13 +615,11 @@ __global__ void __launch_bounds__(kThreadsB, 1)
     };
     uint32_t G = 0, W = 0;
     bool ok = true, staged = false;  // staged: this item's Q, dOut were copied during the previous item
-    for (int w = blockIdx.x; w < a.items && ok; w += gridDim.x) {
-      int bh, tile, qb;
-      decode_item(g, w, bh, tile, qb);
-      TileBlocks tbk;
-      tile_blocks(g, tile, tbk);
-      if (qb >= tbk.NB) continue;
-      const int64_t qslot = tile_slot0(g, bh, tile) + qb * 128 + row;
+    int w = blockIdx.x;
+    int nb = next_boxes(a, w);
+    while (nb > 0) {
+      const int64_t qslot = (int64_t)w * 128 + row;
+      const int place = a.dst[qslot];
       const float nL = a.lse2c[qslot];  // -lse' (-inf for padding rows)
       const float nD = a.dd[qslot];     // -D
       if (!staged && !(ok = copy_qdo(W & 1))) break;
@@ -636,15 +627,9 @@ __global__ void __launch_bounds__(kThreadsB, 1)
       // the next item's Q, dOut are copied once this item's last score
       // products are complete, so its first S and dP run during this item's
       // epilogue
-      bool has_next = false;
-      for (int wn = w + gridDim.x; wn < a.items && !has_next; wn += gridDim.x) {
-        int bh2, tile2, qb2;
-        decode_item(g, wn, bh2, tile2, qb2);
-        TileBlocks t2;
-        tile_blocks(g, tile2, t2);
-        has_next = qb2 < t2.NB;
-      }
-      for (int j = 0; j < tbk.NB && ok; ++j, ++G) {
+      int wn = w + gridDim.x;
+      const int nbn = next_boxes(a, wn);
+      for (int j = 0; j < nb && ok; ++j, ++G) {
         if (!(ok = WAIT(s_full, G & 1))) break;
         tc_fence_after();
         uint32_t sv[32], dv[32], pk[16];
@@ -668,20 +653,17 @@ __global__ void __launch_bounds__(kThreadsB, 1)
         if (lane == 0) mbar_arrive(p_full);
         // s_full[1] of the last box covers every score product of the item:
         // Q, dOut in TMEM are no longer read
-        if (j == tbk.NB - 1 && has_next) {
+        if (j == nb - 1 && nbn > 0) {
           if (!(ok = copy_qdo((W + 1) & 1))) break;
           staged = true;
         }
       }
       if (!ok) break;
-      // where this item's rows go, while the last dQ product runs
-      int qo[3], ql[3];
-      block_origin(g, tbk, qb, qo);
-      block_row(g, qo, row, ql);
-      const bool qvalid = inside(tbk, ql);
-      const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
-      const bool single = qvalid && only_cover(g, tbk.tb, p);
-      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
+      const bool qvalid = place != -1, single = place >= 0;
+      const int64_t off = (single ? ((int64_t)item_bh(g, w) * g.N + place) * kD : 0) + c4 * 32;
+      const int64_t slots = ((int64_t)w * 128 + quad * 32) * kD + c4 * 32;
+      w = wn;
+      nb = nbn;
       if (!(ok = WAIT(acc_full, W & 1))) break;
       tc_fence_after();
       const int c0 = c4 * 32;
@@ -691,8 +673,7 @@ __global__ void __launch_bounds__(kThreadsB, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);  // released before the stores
-      row_slots<OutT>(rq, g.scale, qvalid, single, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
-                      a.dq_s + (qslot - lane) * kD + c0, lane);
+      row_slots<OutT>(rq, g.scale, qvalid, single, static_cast<OutT*>(a.dq) + off, a.dq_s + slots, lane);
       ++W;
     }
   }
@@ -706,13 +687,15 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 
 template <typename OutT>
 cudaError_t run_bwd128(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
-                       const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext, void* dq,
-                       void* dk, void* dv, float* dq_s, float* dk_s, float* dv_s, cudaStream_t st) {
+                       const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext, const int32_t* dst,
+                       const int32_t* nbt, void* dq, void* dk, void* dv, float* dq_s, float* dk_s, float* dv_s, cudaStream_t st) {
   if (!ext || reinterpret_cast<uintptr_t>(ext) % 16) return cudaErrorInvalidValue;
   BwdArgs a;
   a.g = g;
   a.lse2c = lse2c;
   a.dd = dd;
+  a.dst = dst;
+  a.nbt = nbt;
   a.ext = static_cast<const uint4*>(ext);
   a.dq = dq;
   a.dk = dk;
@@ -751,14 +734,14 @@ cudaError_t run_bwd128(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat1
 
 cudaError_t launch_sm103_bwd(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                              const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext,
-                             void* dq, void* dk, void* dv, int out_dtype, float* dq_s, float* dk_s, float* dv_s,
-                             uint32_t, cudaStream_t st) {
+                             const int32_t* dst, const int32_t* nbt, void* dq, void* dk, void* dv, int out_dtype,
+                             float* dq_s, float* dk_s, float* dv_s, uint32_t, cudaStream_t st) {
   if (g.d == 64)
-    return launch_sm103_bwd64(g, q, k, v, dout, lse2c, dd, ext, dq, dk, dv, out_dtype, dq_s, dk_s, dv_s, st);
+    return launch_sm103_bwd64(g, q, k, v, dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, out_dtype, dq_s, dk_s, dv_s, st);
   if (g.d != kD) return cudaErrorNotSupported;
   if (out_dtype == GATTN_BF16)
-    return run_bwd128<__nv_bfloat16>(g, q, k, v, dout, lse2c, dd, ext, dq, dk, dv, dq_s, dk_s, dv_s, st);
-  return run_bwd128<float>(g, q, k, v, dout, lse2c, dd, ext, dq, dk, dv, dq_s, dk_s, dv_s, st);
+    return run_bwd128<__nv_bfloat16>(g, q, k, v, dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, dq_s, dk_s, dv_s, st);
+  return run_bwd128<float>(g, q, k, v, dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, dq_s, dk_s, dv_s, st);
 }
 
 }  // namespace gattn

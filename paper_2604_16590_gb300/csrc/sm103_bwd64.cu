@@ -343,22 +343,12 @@ __global__ void __launch_bounds__(kThreads64, 1)
         if (has_dk) mbar_arrive(kv_empty + ((W - 1) & 1));
       }
     };
-    // The first item at or after w: its boxes, 0 if there is none.  Called for
-    // the next item before the wait for the current item's last gradient
-    // products, which hides it.
+    // The next item is looked up before the wait for the current item's last
+    // gradient products, which hides it.
     int w = blockIdx.x;
-    auto advance = [&]() -> int {
-      for (; w < a.items; w += gridDim.x) {
-        int bh, tile, kb;
-        TileBlocks tbk;
-        decode_item(g, w, bh, tile, kb);
-        tile_blocks(g, tile, tbk);
-        if (kb < tbk.NB) return tbk.NB;
-      }
-      return 0;
-    };
-    int nb = advance();
+    int nb = next_boxes(a, w);
     while (nb > 0) {
+      const int place = a.dst[(int64_t)w * 128 + row];  // slots of an item: w * 128 ...
       for (int i = 0; i < nb && ok; ++i, ++G) {
         if (!(ok = WAIT(s_full, G & 1))) break;
         tc_fence_after();
@@ -389,23 +379,13 @@ __global__ void __launch_bounds__(kThreads64, 1)
         if (i == 0) release_staged();
       }
       if (!ok) break;
-      // ---- where this thread's key row goes (decoded again: keeping the tile's
-      // geometry over the boxes would spill), and the next item
-      int bh, tile, kb, ko[3], kl[3];
-      TileBlocks tbk;
-      decode_item(g, w, bh, tile, kb);
-      tile_blocks(g, tile, tbk);
-      block_origin(g, tbk, kb, ko);
-      block_row(g, ko, row, kl);
-      const bool kvalid = inside(tbk, kl);
-      const int p[3] = {tbk.tb.lo[0] + kl[0], tbk.tb.lo[1] + kl[1], tbk.tb.lo[2] + kl[2]};
-      const bool single = kvalid && only_cover(g, tbk.tb, p);
-      const int64_t tok = single ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
+      const bool kvalid = place != -1, single = place >= 0;
       const int c0 = (c4 & 1) * 32;
-      OutT* dst = static_cast<OutT*>(has_dk ? a.dk : a.dv) + ((int64_t)bh * g.N + tok) * kD + c0;
-      const int srow = (int)(tile_slot0(g, bh, tile) + kb * 128 + quad * 32);
+      OutT* dst = static_cast<OutT*>(has_dk ? a.dk : a.dv) + c0;
+      if (single) dst += ((int64_t)item_bh(g, w) * g.N + place) * kD;
+      const int srow = w * 128 + quad * 32;
       w += gridDim.x;
-      nb = advance();
+      nb = next_boxes(a, w);
       // ---- epilogue: 32 columns of the row of dK or of dV
       if (!(ok = WAIT(acc_full, W & 1))) break;
       tc_fence_after();
@@ -702,29 +682,20 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
     const float sl2 = g.scale_log2;
     uint32_t G = 0, W = 0;
-    int w = (int)blockIdx.x - (int)gridDim.x, nb = 0;
-    int64_t qslot = 0;
+    int w = (int)blockIdx.x - (int)gridDim.x, nb = 0, place = -1;
     float nL = 0.f, nD = 0.f;
-    // The next item: its boxes, slot and statistics, and its Q and dOut from
+    // The next item: its boxes, places and statistics, and its Q and dOut from
     // shared memory into TMEM (the A operands of S and dP; elements
     // [16 c4, 16 c4 + 16) of the row).  Called once the current item's last
     // scores were read, so its S and dP products are complete; the next item's
     // start while its last dQ product runs and its output is written (dQ kernel
     // 3.13 -> 2.40 ms on 24 x 24 tiles, 72.9 -> 68.8 on the paper regime's).
     auto next_item = [&]() -> bool {
-      int bh, tile, qb;
-      do {
-        w += (int)gridDim.x;
-        if (w >= a.items) {
-          nb = 0;
-          return true;
-        }
-        TileBlocks tbk;
-        decode_item(g, w, bh, tile, qb);
-        tile_blocks(g, tile, tbk);
-        nb = tbk.NB;
-      } while (qb >= nb);
-      qslot = tile_slot0(g, bh, tile) + qb * 128 + row;
+      w += (int)gridDim.x;
+      nb = next_boxes(a, w);
+      if (nb == 0) return true;
+      const int64_t qslot = (int64_t)w * 128 + row;
+      place = a.dst[qslot];
       nL = a.lse2c[qslot];  // -lse' (-inf for padding rows)
       nD = a.dd[qslot];     // -D
       if (!WAIT(qd_full, W & 1)) return false;
@@ -774,23 +745,15 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
         if (lane == 0) mbar_arrive(p_full + b);
       }
       if (!ok) break;
-      // where this item's rows go
-      int bh, tile, qb, qo[3], ql[3];
-      TileBlocks tbk;
-      decode_item(g, w, bh, tile, qb);
-      tile_blocks(g, tile, tbk);
-      block_origin(g, tbk, qb, qo);
-      block_row(g, qo, row, ql);
-      const bool qvalid = inside(tbk, ql);
-      const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
-      const int64_t tok = qvalid ? ((int64_t)p[0] * g.G[1] + p[1]) * g.G[2] + p[2] : 0;
-      const bool single = qvalid && only_cover(g, tbk.tb, p);
-      const int srow = (int)(qslot - lane);
+      const bool qvalid = place != -1, single = place >= 0;
+      const int c0 = c4 * 16;
+      OutT* dst = static_cast<OutT*>(a.dq) + c0;
+      if (single) dst += ((int64_t)item_bh(g, w) * g.N + place) * kD;
+      const int srow = w * 128 + quad * 32;
       const uint32_t item = W - 1;
       if (!(ok = next_item())) break;
       if (!(ok = WAIT(acc_full, item & 1))) break;
       tc_fence_after();
-      const int c0 = c4 * 16;
       uint32_t rq[16];
       tmem_ld16(tl + C::kColDQ + c0, rq);
       tmem_wait_ld(rq);
@@ -801,8 +764,8 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
         bulk_wait_read();        // the previous item's store has read this warp's staging block
       }
       __syncwarp();
-      row_out<16, OutT>(rq, g.scale, qvalid, single, true, static_cast<OutT*>(a.dq) + ((int64_t)bh * g.N + tok) * kD + c0,
-                        &tdq, smem_u32(smem + C::kOut) + (warp - kMath0) * 2048, lane, c0, srow);
+      row_out<16, OutT>(rq, g.scale, qvalid, single, true, dst, &tdq, smem_u32(smem + C::kOut) + (warp - kMath0) * 2048,
+                        lane, c0, srow);
     }
     if (lane == 0) bulk_wait_all();
   }
@@ -816,13 +779,15 @@ __global__ void __launch_bounds__(kThreadsQ64, 1)
 
 template <typename OutT>
 cudaError_t run_bwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
-                      const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext, void* dq,
-                      void* dk, void* dv, float* dq_s, float* dk_s, float* dv_s, cudaStream_t st) {
+                      const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext, const int32_t* dst,
+                      const int32_t* nbt, void* dq, void* dk, void* dv, float* dq_s, float* dk_s, float* dv_s, cudaStream_t st) {
   if (!ext || reinterpret_cast<uintptr_t>(ext) % 16) return cudaErrorInvalidValue;
   BwdArgs a;
   a.g = g;
   a.lse2c = lse2c;
   a.dd = dd;
+  a.dst = dst;
+  a.nbt = nbt;
   a.ext = static_cast<const uint4*>(ext);
   a.dq = dq;
   a.dk = dk;
@@ -864,12 +829,12 @@ cudaError_t run_bwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16
 
 cudaError_t launch_sm103_bwd64(const Geom& g, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                                const __nv_bfloat16* dout, const float* lse2c, const float* dd, const void* ext,
-                               void* dq, void* dk, void* dv, int out_dtype, float* dq_s, float* dk_s, float* dv_s,
+                               const int32_t* dst, const int32_t* nbt, void* dq, void* dk, void* dv, int out_dtype, float* dq_s, float* dk_s, float* dv_s,
                                cudaStream_t st) {
   if (g.d != kD) return cudaErrorNotSupported;
   if (out_dtype == GATTN_BF16)
-    return run_bwd64<__nv_bfloat16>(g, q, k, v, dout, lse2c, dd, ext, dq, dk, dv, dq_s, dk_s, dv_s, st);
-  return run_bwd64<float>(g, q, k, v, dout, lse2c, dd, ext, dq, dk, dv, dq_s, dk_s, dv_s, st);
+    return run_bwd64<__nv_bfloat16>(g, q, k, v, dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, dq_s, dk_s, dv_s, st);
+  return run_bwd64<float>(g, q, k, v, dout, lse2c, dd, ext, dst, nbt, dq, dk, dv, dq_s, dk_s, dv_s, st);
 }
 
 }  // namespace gattn
