@@ -89,11 +89,6 @@ struct Geom {
   FastDiv fslots;              // by per_tile
 };
 
-__host__ __device__ __forceinline__ int floordiv(int a, int b) {
-  int q = a / b;
-  return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
-}
-
 struct TileBox {
   int k[3];
   int lo[3];
@@ -117,15 +112,6 @@ __host__ __device__ __forceinline__ void tile_box(const Geom& g, int tile, TileB
     tb.e[a] = hi - lo;
     tb.L *= tb.e[a];
   }
-}
-
-// grid token index of row r of the extended tile
-__host__ __device__ __forceinline__ int64_t tile_token(const Geom& g, const TileBox& tb, int r) {
-  int lx = r % tb.e[2];
-  int rr = r / tb.e[2];
-  int ly = rr % tb.e[1];
-  int lt = rr / tb.e[1];
-  return ((int64_t)(tb.lo[0] + lt) * g.G[1] + (tb.lo[1] + ly)) * g.G[2] + (tb.lo[2] + lx);
 }
 
 __host__ __device__ __forceinline__ void token_pos(const Geom& g, int64_t i, int p[3]) {
@@ -166,26 +152,6 @@ __host__ __device__ __forceinline__ bool only_cover(const Geom& g, const TileBox
     one = one && (k == 0 || p[a] - g.h[a] >= k * g.c[a]) && (k == g.n[a] - 1 || p[a] + g.h[a] < (k + 1) * g.c[a]);
   }
   return one;
-}
-
-// true if exactly one tile covers grid position p
-__host__ __device__ __forceinline__ bool single_cover(const Geom& g, const int p[3]) {
-  bool one = true;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    int k0, k1;
-    cover_dim(g, a, p[a], k0, k1);
-    one = one && (k0 == k1);
-  }
-  return one;
-}
-
-// tile-local coordinates of row r (row-major over the clipped extents)
-__host__ __device__ __forceinline__ void tile_local(const TileBox& tb, int r, int l[3]) {
-  l[2] = r % tb.e[2];
-  const int rr = r / tb.e[2];
-  l[1] = rr % tb.e[1];
-  l[0] = rr / tb.e[1];
 }
 
 // offset (t, y, x) of row rho (0 <= rho < 128) inside a box; the quotients

@@ -179,23 +179,6 @@ struct RowState {
   float lc;  // Kahan compensation of l (the sum runs over every key block of the tile)
 };
 
-template <int N>
-__device__ __forceinline__ float tree_max(float (&v)[N]) {
-#pragma unroll
-  for (int w = N / 2; w >= 1; w /= 2)
-#pragma unroll
-    for (int i = 0; i < w; ++i) v[i] = fmaxf(v[i], v[i + w]);
-  return v[0];
-}
-template <int N>
-__device__ __forceinline__ float tree_sum(float (&v)[N]) {
-#pragma unroll
-  for (int w = N / 2; w >= 1; w /= 2)
-#pragma unroll
-    for (int i = 0; i < w; ++i) v[i] += v[i + w];
-  return v[0];
-}
-
 // named barrier of the two warps that share a TMEM lane quadrant
 __device__ __forceinline__ void pair_sync(int quad) {
   asm volatile("bar.sync %0, 64;" ::"r"(quad + 1) : "memory");
