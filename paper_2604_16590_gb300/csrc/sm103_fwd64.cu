@@ -19,13 +19,18 @@
 //
 // Warp roles (384 threads = three warpgroups, one CTA per SM, persistent over
 // work items (batch*head, tile, box pair)):
-//   warp 0        TMA producer (Q_A, Q_B once per item; K_j, V_j through a ring)
+//   warp 0        TMA producer (lane 0: Q_A, Q_B once per item; K_j, V_j through
+//                 a ring) and key-mask writer (all lanes: for a key block with
+//                 padding rows or rows outside the tile, the bias row of its
+//                 stage, see below)
 //   warp 1        TMEM allocator + issuer of the S products
-//   warp 2        issuer of the P V products (a thread's mbarrier waits stall
-//                 until its own issued MMAs drain, so the two product streams
-//                 come from two threads)
-//   warp 3        key-mask writer: for a key block with padding rows or rows
-//                 outside the tile, the bias row of its stage (see below)
+//   warps 2, 3    issuers of the P V products, one per box.  A thread's mbarrier
+//                 waits stall until its own issued MMAs have drained, which the
+//                 other threads' MMAs in the pipe prolong: with one issuer for
+//                 both boxes, P_A(j) lay finished for up to half a block while
+//                 that thread still waited out P V_B(j-1) (16 heads of 1024
+//                 tiles of 24 x 24: 2.03 -> 1.88 ms; tiles of 36864 tokens, where
+//                 the softmax threads' own chain sets the pace, 58.4 ms either way)
 //   warps 4..7    softmax + epilogue of box A, warps 8..11 of box B: one warp
 //                 per TMEM lane quadrant, one thread per query row owning all
 //                 128 key columns (no cross-warp reduction)
@@ -83,8 +88,8 @@ struct Cfg {
   static constexpr int kBias = kOnes + 4096;
   static constexpr int kBar = kBias + kStages * 4096;
   // q_full[2], q_empty[2], k_full[S], k_empty[S], v_full[S], v_empty[S],
-  // per box: s_full, s_empty, p_full, p_empty, o_full, o_empty; drain[2], never
-  static constexpr int kNumBars = 4 + 4 * kStages + 2 * 6 + 3;
+  // per box: s_full, s_empty, p_full, p_empty, o_full, o_empty; drain[3], never
+  static constexpr int kNumBars = 4 + 4 * kStages + 2 * 6 + 4;
   static constexpr int kMisc = kBar + kNumBars * 8;
   static constexpr int kGeom = kMisc + 16;  // ragged mode: one geometry per warp
   static constexpr int kSmem = kGeom + (RAGGED ? (kThreadsF / 32) * (int)sizeof(Geom) : 0) + 1024;
@@ -277,8 +282,8 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   auto p_empty = [&](int x) { return boxbar + 6 * x + 3; };
   auto o_full = [&](int x) { return boxbar + 6 * x + 4; };
   auto o_empty = [&](int x) { return boxbar + 6 * x + 5; };
-  uint64_t* drain = boxbar + 12;  // [2]
-  uint64_t* never = drain + 2;
+  uint64_t* drain = boxbar + 12;  // [3], one per issuing thread
+  uint64_t* never = drain + 3;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::kMisc + 4);
 
@@ -298,10 +303,10 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       mbar_init(q_empty + b, RAGGED ? 1 : 1 + 8);  // the last score product; the softmax warps (staged outputs read)
     }
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(k_full + s, 2);  // the K load (producer) and the stage's bias row (mask writer)
+      mbar_init(k_full + s, 1);
       mbar_init(k_empty + s, 1);
       mbar_init(v_full + s, 1);
-      mbar_init(v_empty + s, 1);
+      mbar_init(v_empty + s, 2);  // the P V product of each box
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(s_full(x), 1);
@@ -311,8 +316,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       mbar_init(o_full(x), 1);
       mbar_init(o_empty(x), 4);
     }
-    mbar_init(drain, 1);
-    mbar_init(drain + 1, 1);
+    for (int i = 0; i < 3; ++i) mbar_init(drain + i, 1);
     mbar_init(never, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -337,15 +341,19 @@ __global__ void __launch_bounds__(kThreadsF, 1)
 
   if (warp < kSoft0) {
     setmaxnreg_dec<kRegsLow>();
-    if (warp == 0 && lane == 0) {
-      // ---------------------------------------------------------- TMA producer
+    if (warp == 0) {
+      // ---------------------------------------------------------- TMA producer (lane 0) and key-mask writer
+      // The whole warp walks the blocks: its lanes write the bias row of a block that has one, lane 0 does the
+      // waits and the loads.  The arrival that announces K_j's load follows the row, so k_full covers both.
+      const uint32_t neg = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(-1e30f));
       uint32_t G = 0, W = 0;
-      uint32_t q_arm = 0, q_par = 0, k_arm = 0, k_par = 0, v_arm = 0, v_par = 0;
+      uint32_t q_arm = 0, q_par = 0, k_arm = 0, k_par = 0, v_arm = 0, v_par = 0;  // lane 0's
       int last_req = -1;
       bool ok = true;
+      auto all_ok = [&]() { return ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0; };
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
-        if (!resolve<RAGGED, true>(a, &tq, &tk, &tv, w, rc, it)) continue;
+        if (!resolve<RAGGED, false>(a, &tq, &tk, &tv, w, rc, it)) continue;
         const Geom& g = *it.g;
         const int bh = it.bh;
         TileBlocks tbk;
@@ -353,48 +361,61 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         const int qa = 2 * it.pair;
         if (qa >= tbk.NB) continue;
         const int nact = qa + 1 < tbk.NB ? 2 : 1;
-        if (RAGGED && it.req != last_req) {
-          tmap_acquire(it.tq);  // this launch's descriptor table may hold a new map here
-          last_req = it.req;
-        }
-        // Q of this item goes to buffer W & 1, so it loads while the previous
-        // item's score products still read the other buffer
-        const uint32_t qb = W & 1, qn = (W >> 1) & 1;
-        if (!(ok = WAIT(q_empty + qb, qn ^ 1))) break;
-        mbar_arrive_expect_tx(q_full + qb, nact * g.R * 128);
-        q_arm |= 1u << qb;
-        q_par = (q_par & ~(1u << qb)) | (qn << qb);
-        for (int x = 0; x < nact; ++x) {
-          int o[3];
-          block_origin(g, tbk, qa + x, o);
-          tma_load_5d(smem + C::kQ + (2 * qb + x) * kBox, it.tq, q_full + qb, 0, tbk.tb.lo[2] + o[2],
-                      tbk.tb.lo[1] + o[1], tbk.tb.lo[0] + o[0], bh);
-        }
-        int jt = 0, jy = 0, jx = 0;
-        for (int j = 0; j < tbk.NB; ++j, ++G) {
-          const uint32_t st = G % kStages, n = G / kStages;
-          const int c1 = tbk.tb.lo[2] + (jx * g.bx), c2 = tbk.tb.lo[1] + (jy * g.by), c3 = tbk.tb.lo[0] + (jt * g.bt);
-          if (++jx == tbk.nb[2]) {
-            jx = 0;
-            if (++jy == tbk.nb[1]) {
-              jy = 0;
-              ++jt;
+        if (lane == 0) {
+          if (RAGGED && it.req != last_req) {
+            tmap_acquire(it.tq);  // this launch's descriptor table may hold a new map here
+            last_req = it.req;
+          }
+          // Q of this item goes to buffer W & 1, so it loads while the previous
+          // item's score products still read the other buffer
+          const uint32_t qb = W & 1, qn = (W >> 1) & 1;
+          if ((ok = WAIT(q_empty + qb, qn ^ 1))) {
+            mbar_arrive_expect_tx(q_full + qb, nact * g.R * 128);
+            q_arm |= 1u << qb;
+            q_par = (q_par & ~(1u << qb)) | (qn << qb);
+            for (int x = 0; x < nact; ++x) {
+              int o[3];
+              block_origin(g, tbk, qa + x, o);
+              tma_load_5d(smem + C::kQ + (2 * qb + x) * kBox, it.tq, q_full + qb, 0, tbk.tb.lo[2] + o[2],
+                          tbk.tb.lo[1] + o[1], tbk.tb.lo[0] + o[0], bh);
             }
           }
-          if (!(ok = WAIT(k_empty + st, (n & 1) ^ 1))) break;
-          mbar_arrive_expect_tx(k_full + st, g.R * 128);
-          k_arm |= 1u << st;
-          k_par = (k_par & ~(1u << st)) | ((n & 1) << st);
-          tma_load_5d(smem + C::kK + st * kBox, it.tk, k_full + st, 0, c1, c2, c3, bh);
-          if (!(ok = WAIT(v_empty + st, (n & 1) ^ 1))) break;
-          mbar_arrive_expect_tx(v_full + st, g.R * 128);
-          v_arm |= 1u << st;
-          v_par = (v_par & ~(1u << st)) | ((n & 1) << st);
-          tma_load_5d(smem + C::kV + st * kBox, it.tv, v_full + st, 0, c1, c2, c3, bh);
         }
+        const bool all_full = tile_all_full(g, tbk);
+        BlockWalk bw;
+        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
+          const uint32_t st = G % kStages, n = G / kStages;
+          const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
+          if (lane == 0 && ok) ok = WAIT(k_empty + st, (n & 1) ^ 1);
+          if (!all_ok()) break;
+          if (!all_full && !bw.full(g, tbk)) {
+            for (int r = lane; r < 128; r += 32) {
+              int kl[3];
+              block_row(g, ko, r, kl);
+              *reinterpret_cast<uint4*>(smem + C::kBias + st * 4096 + r * 16) =
+                  make_uint4(inside(tbk, kl) ? 0u : neg, 0u, 0u, 0u);
+            }
+            fence_proxy_async_smem();  // the tensor core reads what these lanes wrote
+            __syncwarp();
+          }
+          if (lane == 0) {
+            const int c1 = tbk.tb.lo[2] + ko[2], c2 = tbk.tb.lo[1] + ko[1], c3 = tbk.tb.lo[0] + ko[0];
+            mbar_arrive_expect_tx(k_full + st, g.R * 128);
+            k_arm |= 1u << st;
+            k_par = (k_par & ~(1u << st)) | ((n & 1) << st);
+            tma_load_5d(smem + C::kK + st * kBox, it.tk, k_full + st, 0, c1, c2, c3, bh);
+            if ((ok = WAIT(v_empty + st, (n & 1) ^ 1))) {
+              mbar_arrive_expect_tx(v_full + st, g.R * 128);
+              v_arm |= 1u << st;
+              v_par = (v_par & ~(1u << st)) | ((n & 1) << st);
+              tma_load_5d(smem + C::kV + st * kBox, it.tv, v_full + st, 0, c1, c2, c3, bh);
+            }
+          }
+        }
+        if (!all_ok()) break;
         ++W;
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         // let every load this thread issued land before the CTA exits
         for (int b = 0; b < 2; ++b)
           if (q_arm & (1u << b)) mbar_wait<set_status_f64>(q_full + b, (q_par >> b) & 1, abort_flag, false);
@@ -429,7 +450,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         BlockWalk bw;
         for (int j = 0; j < tbk.NB && ok; ++j, ++G, bw.next(tbk)) {
           const uint32_t st = G % kStages;
-          // a masked block's bias row was filled by the mask writer
+          // a masked block's bias row was written by the producer warp
           const bool masked = !all_full && !bw.full(g, tbk);
           if (!(ok = WAIT(k_full + st, (G / kStages) & 1))) break;
           const uint64_t dk = dmove(dK0, st * kBox), db = dmove(dBias0, st * 4096);
@@ -457,11 +478,13 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       }
       umma_commit(drain);
       mbar_wait<set_status_f64>(drain, 0, abort_flag, false);
-    } else if (warp == 2 && lane == 0) {
-      // ---------------------------------------------------------- issuer of O_x += P_x V
+    } else if (warp >= 2 && lane == 0) {
+      // ---------------------------------------------------------- issuers of O_x += P_x V, one thread per box
+      const int x = warp - 2;
       constexpr uint32_t idO = idesc_bf16(128, kD, 1);
       const uint64_t dV0 = sw128_desc(smem_u32(smem + C::kV), 16384, 1024);  // MN-major (K = keys)
-      uint32_t G = 0, GX0 = 0, GX1 = 0, WX0 = 0, WX1 = 0;
+      const uint32_t tO = tmem + col_o(x), tP = tmem + col_p(x);
+      uint32_t G = 0, GX = 0, WX = 0;
       bool ok = true;
       for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         Item it;
@@ -470,70 +493,30 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         tile_blocks(*it.g, it.tile, tbk);
         const int qa = 2 * it.pair;
         if (qa >= tbk.NB) continue;
-        const int nact = qa + 1 < tbk.NB ? 2 : 1;
-        for (int j = 0; j < tbk.NB && ok; ++j, ++G) {
+        const bool act = qa + x < tbk.NB;
+        for (int j = 0; j < tbk.NB; ++j, ++G) {
           const uint32_t st = G % kStages;
           if (!(ok = WAIT(v_full + st, (G / kStages) & 1))) break;
+          if (!act) {  // an item of one box: the other issuer's product is V_j's only reader
+            mbar_arrive(v_empty + st);
+            continue;
+          }
           const uint64_t dv = dmove(dV0, st * kBox);
+          if (!(ok = WAIT(p_full(x), GX & 1))) break;
+          if (j == 0 && !(ok = WAIT(o_empty(x), (WX & 1) ^ 1))) break;
+          tc_fence_after();
 #pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            if (x >= nact) break;
-            uint32_t& gx = x == 0 ? GX0 : GX1;
-            const uint32_t wx = x == 0 ? WX0 : WX1;
-            if (!(ok = WAIT(p_full(x), gx & 1))) break;
-            if (j == 0 && !(ok = WAIT(o_empty(x), (wx & 1) ^ 1))) break;
-            tc_fence_after();
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-              umma_bf16_ts(tmem + col_o(x), tmem + col_p(x) + ks * 8, dmove(dv, ks * 2048), idO,
-                           (j > 0 || ks > 0) ? 1u : 0u);
-            umma_commit(p_empty(x));
-            if (j == tbk.NB - 1) umma_commit(o_full(x));
-            ++gx;
-          }
-          if (!ok) break;
+          for (int ks = 0; ks < 8; ++ks)
+            umma_bf16_ts(tO, tP + ks * 8, dmove(dv, ks * 2048), idO, (j > 0 || ks > 0) ? 1u : 0u);
+          umma_commit(p_empty(x));
+          if (j == tbk.NB - 1) umma_commit(o_full(x));
           umma_commit(v_empty + st);
+          ++GX;
         }
-        ++WX0;
-        if (nact > 1) ++WX1;
+        if (act) ++WX;
       }
-      umma_commit(drain + 1);
-      mbar_wait<set_status_f64>(drain + 1, 0, abort_flag, false);
-    } else if (warp == 3) {
-      // ---------------------------------------------------------- key-mask writer
-      // One arrival on k_full per stage use (the stage's second arrival), in
-      // the producer's order.  It first waits until the stage is free again,
-      // which also guarantees that the previous phase of k_full completed.
-      const uint32_t neg = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(-1e30f));
-      uint32_t G = 0;
-      bool ok = true;
-      for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
-        Item it;
-        if (!resolve<RAGGED, false>(a, &tq, &tk, &tv, w, rc, it)) continue;
-        const Geom& g = *it.g;
-        TileBlocks tbk;
-        tile_blocks(g, it.tile, tbk);
-        if (2 * it.pair >= tbk.NB) continue;
-        BlockWalk bw;
-        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
-          const uint32_t st = G % kStages, n = G / kStages;
-          const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
-          if (lane == 0) ok = WAIT(k_empty + st, (n & 1) ^ 1);
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-          if (!ok) break;
-          if (!block_full(g, tbk, ko)) {
-            for (int r = lane; r < 128; r += 32) {
-              int kl[3];
-              block_row(g, ko, r, kl);
-              *reinterpret_cast<uint4*>(smem + C::kBias + st * 4096 + r * 16) =
-                  make_uint4(inside(tbk, kl) ? 0u : neg, 0u, 0u, 0u);
-            }
-            fence_proxy_async_smem();  // the tensor core reads what these lanes wrote
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(k_full + st);
-        }
-      }
+      umma_commit(drain + 1 + x);
+      mbar_wait<set_status_f64>(drain + 1 + x, 0, abort_flag, false);
     }
   } else {
     setmaxnreg_inc<kRegsHigh>();
@@ -592,8 +575,9 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         qvalid = inside(tbk, ql);
       }
       float m = -INFINITY, l = 0.f, lc = 0.f;  // lc: Kahan compensation of the row sum l
+      bool s_ready = false;
       for (int j = 0; j < nb; ++j, ++GX) {
-        if (!(ok = WAIT(s_full(x), GX & 1))) break;
+        if (!s_ready && !(ok = WAIT(s_full(x), GX & 1))) break;
         tc_fence_after();
         // the row's 128 scores into registers, then S_x is released
         uint32_t s0[32], s1[32], s2r[32], s3[32];
@@ -663,6 +647,9 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         tmem_st16(tP + 16, pk1);
         tmem_st16(tP + 32, pk2);
         tmem_st16(tP + 48, pk3);
+        // the next scores are usually there by now: ask while P is being stored (tiles
+        // of 36864 tokens 59.7 -> 58.4 ms; ragged mode is 1 % slower with it)
+        s_ready = !RAGGED && j + 1 < nb && mbar_try_wait(smem_u32(s_full(x)), (GX + 1) & 1);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
