@@ -426,6 +426,7 @@ CompressPlan compress_plan(int B, int nh, int S, int M) {
       full = f;
       best = chunk;
     }
+    if (want == cap) break;  // the shortest ranges: more waves change nothing
   }
   p.splits = (int)(((long long)S + best - 1) / best);
   p.chunk = (int)best;

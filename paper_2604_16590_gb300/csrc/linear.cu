@@ -583,7 +583,9 @@ struct BQArgs {
 //           of a row's 64 columns each and exchange the row's two sums (den,
 //           phi(q) . U) through shared memory, added in a fixed order.
 // At the end the CTA writes its dS and dz partials.  16 heads of 262144
-// tokens: 705 -> 481 us (one group of eight warps, plain stores of dq, before).
+// tokens: 705 -> 436 us (one group of eight warps, plain stores of dq and
+// 1216 CTAs before); 1.61 GB in that time, 0.54 of the HBM rate: the math
+// groups' row work (phi, its parts, the row sums) sets the pace.
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid_constant__ CUtensorMap tq,
                                                                     const __grid_constant__ CUtensorMap tg,
                                                                     const __grid_constant__ CUtensorMap tdq,
@@ -938,8 +940,9 @@ struct BKArgs {
 // A stage is released by the four quadrants once their stores have read it.
 // Two math warps per group and TMEM lane quadrant, each taking 32 of a row's
 // 64 columns (nothing here sums over a row).  16 heads of 262144 tokens:
-// 713 -> 406 us (one group of eight warps, a thread storing its own 64
-// bytes of a row, before).
+// 713 -> 327 us (one group of eight warps, a thread storing its own 64
+// bytes of a row and 16 tiles per CTA before); 2.15 GB in that time, 0.97 of
+// the HBM rate.
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_constant__ CUtensorMap tk,
                                                                   const __grid_constant__ CUtensorMap tv,
                                                                   const __grid_constant__ CUtensorMap tdk,
@@ -1171,7 +1174,7 @@ static int tiles_per_cta(int ntiles, int BH, int slots) {
       full = f;
       best = per;
     }
-    if (full >= 0.95) break;
+    if (full >= 0.95 || per == 1) break;  // one tile each: more waves change nothing
   }
   return best;
 }
@@ -1188,9 +1191,7 @@ LinearPlan linear_plan(int B, int nh, int64_t N) {
   return p;
 }
 
-LinearLayout linear_layout(int B, int nh, int64_t N) {
-  const LinearPlan p = linear_plan(B, nh, N);
-  const size_t BH = (size_t)B * nh;
+static LinearLayout layout_of(const LinearPlan& p, size_t BH) {
   LinearLayout l;
   l.part_S = 0;
   l.part_z = l.part_S + align_up((size_t)p.chunks * BH * kD * kD * 4);
@@ -1201,13 +1202,17 @@ LinearLayout linear_layout(int B, int nh, int64_t N) {
   return l;
 }
 
+LinearLayout linear_layout(int B, int nh, int64_t N) {
+  return layout_of(linear_plan(B, nh, N), (size_t)B * nh);
+}
+
 size_t linear_ws_bytes(int B, int nh, int64_t N) { return linear_layout(B, nh, N).bytes; }
 
 cudaError_t launch_linear(const void* q, const void* k, const void* v, void* out, void* ws, int B, int nh, int64_t N,
                           cudaStream_t st) {
   const LinearPlan p = linear_plan(B, nh, N);
-  const LinearLayout lay = linear_layout(B, nh, N);
   const int BH = B * nh;
+  const LinearLayout lay = layout_of(p, BH);
   char* w = static_cast<char*>(ws);
   SumArgs sa;
   sa.N = (int)N;
@@ -1262,9 +1267,7 @@ cudaError_t launch_linear(const void* q, const void* k, const void* v, void* out
   return e;
 }
 
-LinearBwdLayout linear_bwd_layout(int B, int nh, int64_t N) {
-  const LinearPlan p = linear_plan(B, nh, N);
-  const size_t BH = (size_t)B * nh;
+static LinearBwdLayout bwd_layout_of(const LinearPlan& p, size_t BH) {
   LinearBwdLayout l;
   l.part_dS = 0;
   l.part_dz = l.part_dS + align_up((size_t)p.b_chunks * BH * kD * kD * 4);
@@ -1277,12 +1280,16 @@ LinearBwdLayout linear_bwd_layout(int B, int nh, int64_t N) {
   return l;
 }
 
+LinearBwdLayout linear_bwd_layout(int B, int nh, int64_t N) {
+  return bwd_layout_of(linear_plan(B, nh, N), (size_t)B * nh);
+}
+
 cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const void* dout, const void* saved,
                               void* dq, void* dk, void* dv, void* ws, int B, int nh, int64_t N, cudaStream_t st) {
   const LinearPlan p = linear_plan(B, nh, N);
-  const LinearLayout fl = linear_layout(B, nh, N);
-  const LinearBwdLayout bl = linear_bwd_layout(B, nh, N);
   const int BH = B * nh;
+  const LinearLayout fl = layout_of(p, BH);
+  const LinearBwdLayout bl = bwd_layout_of(p, BH);
   const char* sv = static_cast<const char*>(saved);
   char* w = static_cast<char*>(ws);
   BQArgs qa;

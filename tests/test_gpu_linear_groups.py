@@ -1,6 +1,6 @@
 """Linear attention backward at the edges of its two-group schedule: one tile,
-odd and even tile counts per CTA, ragged last tiles and the 16-tile CTAs of the
-key pass, against the oracle's analytic gradient (max-rel <= 2e-2, rms-rel <=
+odd and even tile counts per CTA, ragged last tiles and the tile counts around
+16, against the oracle's analytic gradient (max-rel <= 2e-2, rms-rel <=
 3e-3, the bar of the other linear tests); and a NaN in q, which has to reach
 the same elements as in the oracle (feature maps built from minima and maxima
 would lose it)."""
