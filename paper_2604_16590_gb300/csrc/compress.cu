@@ -403,7 +403,11 @@ cudaError_t launch_d(const CArgs& a, int d, cudaStream_t st) {
 // Frame ranges: the fewest (the partials of a range cost a write and a read of
 // 4 d + 8 bytes per location) that fill four or more whole waves of the
 // persistent CTAs to 95 %, else the fullest up to sixteen waves; at least 64
-// frames per range.
+// frames per range.  Where ranges of 64 frames make fewer than four waves, one
+// to three are looked at too, or the ranges would be cut short for a second
+// wave that stays half empty (237 frames of 223 locations, 16 heads, d = 128:
+// 96 -> 78 us; 2027 of 61, 8 heads: 109 -> 95; 40 sizes between 9 and 6104
+// frames: none slower than with the former eight or more ranges).
 // 512 frames of 2048 locations, 8 heads, d = 128: four ranges instead of eight,
 // and the combine in 16-byte loads: combine 48 -> 14 us, call 699 -> 667 us (the
 // stream alone takes 632 at the copy rate).
@@ -414,7 +418,8 @@ CompressPlan compress_plan(int B, int nh, int S, int M) {
   const long long cap = S / 64 > 1 ? S / 64 : 1;
   long long best = S;  // frames per range
   double full = 0.0;
-  for (long long w = 4; w <= 16 && full < 0.95; ++w) {
+  const long long w0 = kPersistentCtas * 4 / base > cap ? 1 : 4;
+  for (long long w = w0; w <= 16 && full < 0.95; ++w) {
     long long want = kPersistentCtas * w / base;
     if (want < 1) want = 1;
     if (want > cap) want = cap;
