@@ -42,10 +42,14 @@ __device__ __forceinline__ void block_origin(const Geom& g, const TileBlocks& t,
   o[2] = jx * g.bx;
 }
 
+// every token of the block lies inside the tile (rows R..127 may be padding)
+__device__ __forceinline__ bool block_inside(const Geom& g, const TileBlocks& t, const int o[3]) {
+  return o[0] + g.bt <= t.tb.e[0] && o[1] + g.by <= t.tb.e[1] && o[2] + g.bx <= t.tb.e[2];
+}
 // all 128 rows of the block hold tokens of the tile (no padding row, none
 // outside the tile)
 __device__ __forceinline__ bool block_full(const Geom& g, const TileBlocks& t, const int o[3]) {
-  return g.R == 128 && o[0] + g.bt <= t.tb.e[0] && o[1] + g.by <= t.tb.e[1] && o[2] + g.bx <= t.tb.e[2];
+  return g.R == 128 && block_inside(g, t, o);
 }
 
 // tile-local coordinates of row rho of a block with origin o; a padding row
@@ -64,12 +68,16 @@ __device__ __forceinline__ bool tile_all_full(const Geom& g, const TileBlocks& t
 }
 
 // Walks the blocks of a tile in index order with counters instead of
-// divisions; full() says whether the current block is full (block_full).
+// divisions; full() and inside() are block_full and block_inside of the current one.
 struct BlockWalk {
   int jt = 0, jy = 0, jx = 0;
   __device__ __forceinline__ bool full(const Geom& g, const TileBlocks& t) const {
     const int o[3] = {jt * g.bt, jy * g.by, jx * g.bx};
     return block_full(g, t, o);
+  }
+  __device__ __forceinline__ bool inside(const Geom& g, const TileBlocks& t) const {
+    const int o[3] = {jt * g.bt, jy * g.by, jx * g.bx};
+    return block_inside(g, t, o);
   }
   __device__ __forceinline__ void next(const TileBlocks& t) {
     if (++jx == t.nb[2]) {
@@ -84,6 +92,11 @@ struct BlockWalk {
 
 __device__ __forceinline__ bool inside(const TileBlocks& t, const int l[3]) {
   return l[0] < t.tb.e[0] && l[1] < t.tb.e[1] && l[2] < t.tb.e[2];
+}
+
+// tile-local coordinates l[3] (at or past the tile's end, never before its start) lie on the grid
+__device__ __forceinline__ bool in_grid(const Geom& g, const TileBlocks& t, const int l[3]) {
+  return t.tb.lo[0] + l[0] < g.G[0] && t.tb.lo[1] + l[1] < g.G[1] && t.tb.lo[2] + l[2] < g.G[2];
 }
 
 // Zero rows R..127 of n consecutive 16 KB operand blocks starting at `base`

@@ -19,17 +19,20 @@
 //
 // Warp roles (384 threads, one CTA per SM, persistent over work items
 // (batch*head, tile, query block)):
-//   warp 0      TMA producer (Q once per item; K_j, V_j through a ring of stages)
+//   warp 0      TMA producer (Q once per item; K_j and V_j through rings of three and two stages)
 //   warp 1      TMEM allocator + issuer of the S = Q K^T products
 //   warps 2..9  softmax + epilogue: one query row per TMEM lane, two warps per
 //               lane quadrant splitting each row's keys and output columns
 //               (two math warps per SM sub-partition hide TMEM/MUFU latency)
 //   warp 10     issuer of the P V products
-//   warp 11     key-mask writer: the bias row of a key block with padding rows or
-//               keys outside the tile, added to its scores by one more K = 16 MMA
-//               step, so the softmax has one branch-free form (a second, masked
+//   warp 11     key-mask writer: for a key block that reaches out of the tile, zeroes
+//               the K rows of tokens outside the tile and writes the block's bias
+//               row (0 or -inf per key), which one more K = 16 MMA step adds to the
+//               scores, so the softmax has one branch-free form (a second, masked
 //               form of the loop, cost the ragged 7 x 45 x 77 crop of 12 heads 2.16 ms
-//               against 1.44 now, and unmasked tiles 1 %)
+//               against 1.44 without it, and unmasked tiles 1 %).  A block inside the
+//               tile whose only masked keys are padding rows takes a bias row written
+//               once per launch
 // Two issuing threads, because a thread's shared-memory accesses (an mbarrier
 // wait included) are held until the tcgen05.mma it issued before them have
 // drained from the tensor pipe: with one issuer every wait between the S and
@@ -52,19 +55,21 @@ template <int D>
 struct FwdCfg {
   static constexpr int kHalves = D / 64;            // 128-byte column chunks of a row
   static constexpr int kBlock = 128 * D * 2;        // bytes of one Q/K/V block
-  static constexpr int kStages = D == 64 ? 4 : 2;   // K/V ring depth
+  static constexpr int kStagesK = 3, kStagesV = 2;  // ring depths
   static constexpr int kQ = 0;
   static constexpr int kK = kQ + kBlock;
-  static constexpr int kV = kK + kStages * kBlock;
+  static constexpr int kV = kK + kStagesK * kBlock;
   // Key-mask extension operands (as in the d = 64 forward): A = 1 in K-column 0
-  // of 128 rows, and per stage the key block's bias row (0, or -1e30 for a
-  // padding key or a key outside the tile), each followed by 2 KB of zeros.
-  static constexpr int kOnes = kV + kStages * kBlock;
+  // of 128 rows, and per stage the key block's bias row (0, or -inf for a
+  // padding key or a key outside the tile), then one for blocks that have only
+  // padding keys; each followed by 2 KB of zeros.
+  static constexpr int kOnes = kV + kStagesV * kBlock;
   static constexpr int kBias = kOnes + 4096;
-  static constexpr int kBar = kBias + kStages * 4096;
-  // q_full, q_empty, qt_full, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], s_empty[2],
+  static constexpr int kPadBias = kBias + kStagesK * 4096;
+  static constexpr int kBar = kPadBias + 4096;
+  // q_full, q_empty, qt_full, k_full[S], k_load[S], k_empty[S], v_full[S], v_empty[S], s_full[2], s_empty[2],
   // p_full, pv_done[2], o_empty, drain[2], never (test hook: nothing arrives on it)
-  static constexpr int kNumBars = 3 + 4 * kStages + 4 + 7;
+  static constexpr int kNumBars = 3 + 3 * kStagesK + 2 * kStagesV + 4 + 7;
   static constexpr int kMisc = kBar + kNumBars * 8;
   static constexpr int kRed = kMisc + 16;           // float [3 slots][2 half][128 rows]
   static constexpr int kSmem = kRed + 3072 + 1024;  // + slack for 1024-byte alignment
@@ -167,6 +172,7 @@ constexpr int kMathWarps = 8;
 constexpr int kThreads = 64 + 32 * kMathWarps + 64;
 constexpr int kIssuerPV = 2 + kMathWarps;  // warp index of the P V issuer
 constexpr int kMaskWriter = kIssuerPV + 1;
+constexpr uint32_t kNegInf = 0xFF80u;  // BF16 -inf
 
 // Online-softmax state of one query row, as held by one of its two threads.
 // P = exp2(s S log2e - m) is formed against a reference max m that only moves
@@ -262,7 +268,7 @@ __device__ __forceinline__ bool softmax_block(RowState& rs, uint32_t tS, uint32_
   tmem_ld32(tS + 32, r1);
   tmem_wait_ld(r0);
   tmem_wait_ld(r1);
-  // masked keys carry -1e30 from the extension step: no mask here
+  // masked keys carry -inf from the extension step: no mask here
   chunk_max(r0, mx);
   chunk_max(r1, mx);
   const float mine = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
@@ -321,10 +327,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* q_empty = bars + 1;
   uint64_t* qt_full = bars + 2;
   uint64_t* k_full = bars + 3;
-  uint64_t* k_empty = k_full + C::kStages;
-  uint64_t* v_full = k_empty + C::kStages;
-  uint64_t* v_empty = v_full + C::kStages;
-  uint64_t* s_full = v_empty + C::kStages;
+  uint64_t* k_load = k_full + C::kStagesK;  // the K loads of blocks that reach out of their tile
+  uint64_t* k_empty = k_load + C::kStagesK;
+  uint64_t* v_full = k_empty + C::kStagesK;
+  uint64_t* v_empty = v_full + C::kStagesV;
+  uint64_t* s_full = v_empty + C::kStagesV;
   uint64_t* s_empty = s_full + 2;
   uint64_t* p_full = s_empty + 2;
   uint64_t* pv_done = p_full + 1;  // [2], one per P buffer
@@ -335,20 +342,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::kMisc + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  zero_pad_rows(smem, (1 + 2 * C::kStages) * C::kHalves, a.pad_R);  // Q and the K and V rings
-  for (int r = threadIdx.x; r < (1 + C::kStages) * 256; r += kThreads) {
+  zero_pad_rows(smem, (1 + C::kStagesK + C::kStagesV) * C::kHalves, a.pad_R);  // Q and the K and V rings
+  for (int r = threadIdx.x; r < (2 + C::kStagesK) * 256; r += kThreads) {
     const int blk = r >> 8, rr = r & 255;
-    const uint4 v = (blk == 0 && rr < 128) ? make_uint4(0x00003F80u, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
-    if (blk == 0 || rr >= 128) *reinterpret_cast<uint4*>(smem + C::kOnes + blk * 4096 + rr * 16) = v;
+    uint32_t v = 0;
+    if (blk == 0 && rr < 128) v = 0x3F80u;                                // BF16 1
+    if (blk == 1 + C::kStagesK && rr < 128 && rr >= a.pad_R) v = kNegInf;
+    *reinterpret_cast<uint4*>(smem + C::kOnes + blk * 4096 + rr * 16) = make_uint4(v, 0u, 0u, 0u);
   }
   fence_proxy_async_smem();
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     mbar_init(q_empty, kMathWarps);
     mbar_init(qt_full, kMathWarps);
-    for (int s = 0; s < C::kStages; ++s) {
-      mbar_init(k_full + s, 2);  // the K load (producer) and the stage's bias row (mask writer)
+    for (int s = 0; s < C::kStagesK; ++s) {
+      mbar_init(k_full + s, 1);  // the K load, or the mask writer
+      mbar_init(k_load + s, 1);
       mbar_init(k_empty + s, 1);
+    }
+    for (int s = 0; s < C::kStagesV; ++s) {
       mbar_init(v_full + s, 1);
       mbar_init(v_empty + s, 1);
     }
@@ -383,61 +395,109 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
+    // K runs one block ahead of V, over the items' ends too (after an item of one
+    // block its V goes first: the next item's Q waits for this item to begin).  A V
+    // stage comes free only with the P V product of two blocks before, too late
+    // for a K block loaded after it: with K behind V and two K stages the forward
+    // took 56.1 ms on two tiles of 136 x 32 x 64 tokens (52.9 now), and the mask
+    // writer's turn between a masked block's load and its product would have cost
+    // the ragged 7 x 45 x 77 crop of 12 heads 9 % (1.55 -> 1.69 ms; 1.44 now).
     if (lane == 0) {
-      uint32_t G = 0, W = 0;
-      // arming record for the abort drain: bit s of k_arm/v_arm = stage s armed at
-      // least once, bit s of k_par/v_par = parity of its latest arming
-      uint32_t k_arm = 0, v_arm = 0, k_par = 0, v_par = 0, q_arm = 0, q_par = 0;
+      uint32_t GK = 0, GV = 0, W = 0;
+      // arming record for the abort drain: bit s of k_arm/v_arm (l_arm: k_load) =
+      // stage s armed at least once, bit s of k_par/v_par (l_par) = parity of its
+      // latest arming
+      uint32_t k_arm = 0, v_arm = 0, k_par = 0, v_par = 0, l_arm = 0, l_par = 0, q_arm = 0, q_par = 0;
       int last_req = -1;
-      bool ok = true;
-      for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
-        Item it;
-        if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
-        const Geom& g = *it.g;
-        const int bh = it.bh, tile = it.tile, qb = it.blk;
-        TileBlocks tbk;
-        tile_blocks(g, tile, tbk);
-        if (qb >= tbk.NB) continue;
+      auto next_item = [&](int& w, Item& it, TileBlocks& t) -> bool {
+        for (; w < n_items; w += gridDim.x) {
+          if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
+          tile_blocks(*it.g, it.tile, t);
+          if (it.blk < t.NB) return true;
+        }
+        return false;
+      };
+      auto load_q = [&](const Item& it, const TileBlocks& t) -> bool {
         if (RAGGED && it.req != last_req) {
           tmap_acquire(it.tq);  // this launch's descriptor table may hold a new map here
           last_req = it.req;
         }
         int o[3];
-        block_origin(g, tbk, qb, o);
-        if (!(ok = mbar_wait<set_status_fwd>(q_empty, (W & 1) ^ 1, abort_flag))) break;
-        mbar_arrive_expect_tx(q_full, C::kHalves * g.R * 128);
+        block_origin(*it.g, t, it.blk, o);
+        if (!mbar_wait<set_status_fwd>(q_empty, (W & 1) ^ 1, abort_flag)) return false;
+        mbar_arrive_expect_tx(q_full, C::kHalves * it.g->R * 128);
         q_arm = 1;
         q_par = W & 1;
         for (int h = 0; h < C::kHalves; ++h)
-          tma_load_5d(smem + C::kQ + h * 16384, it.tq, q_full, 64 * h, tbk.tb.lo[2] + o[2], tbk.tb.lo[1] + o[1],
-                      tbk.tb.lo[0] + o[0], bh);
-        BlockWalk bw;
-        for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
-          const uint32_t st = G % C::kStages, n = G / C::kStages;
-          const int c1 = tbk.tb.lo[2] + bw.jx * g.bx, c2 = tbk.tb.lo[1] + bw.jy * g.by,
-                    c3 = tbk.tb.lo[0] + bw.jt * g.bt;
-          if (!(ok = mbar_wait<set_status_fwd>(k_empty + st, (n & 1) ^ 1, abort_flag))) break;
-          mbar_arrive_expect_tx(k_full + st, C::kHalves * g.R * 128);
+          tma_load_5d(smem + C::kQ + h * 16384, it.tq, q_full, 64 * h, t.tb.lo[2] + o[2], t.tb.lo[1] + o[1],
+                      t.tb.lo[0] + o[0], it.bh);
+        ++W;
+        return true;
+      };
+      auto load_k = [&](const Item& it, const TileBlocks& t, const BlockWalk& b) -> bool {
+        const Geom& g = *it.g;
+        const uint32_t st = GK % C::kStagesK, n = GK / C::kStagesK;
+        const bool out = !b.inside(g, t);
+        uint64_t* bar = out ? k_load + st : k_full + st;
+        if (!mbar_wait<set_status_fwd>(k_empty + st, (n & 1) ^ 1, abort_flag)) return false;
+        mbar_arrive_expect_tx(bar, C::kHalves * g.R * 128);
+        if (out) {
+          l_par ^= l_arm & (1u << st);  // the phases of k_load alternate over a stage's such blocks
+          l_arm |= 1u << st;
+          k_arm &= ~(1u << st);  // the stage's earlier load has been used
+        } else {
           k_arm |= 1u << st;
           k_par = (k_par & ~(1u << st)) | ((n & 1) << st);
-          for (int h = 0; h < C::kHalves; ++h)
-            tma_load_5d(smem + C::kK + st * C::kBlock + h * 16384, it.tk, k_full + st, 64 * h, c1, c2, c3, bh);
-          if (!(ok = mbar_wait<set_status_fwd>(v_empty + st, (n & 1) ^ 1, abort_flag))) break;
-          mbar_arrive_expect_tx(v_full + st, C::kHalves * g.R * 128);
-          v_arm |= 1u << st;
-          v_par = (v_par & ~(1u << st)) | ((n & 1) << st);
-          for (int h = 0; h < C::kHalves; ++h)
-            tma_load_5d(smem + C::kV + st * C::kBlock + h * 16384, it.tv, v_full + st, 64 * h, c1, c2, c3, bh);
         }
-        ++W;
+        for (int h = 0; h < C::kHalves; ++h)
+          tma_load_5d(smem + C::kK + st * C::kBlock + h * 16384, it.tk, bar, 64 * h, t.tb.lo[2] + b.jx * g.bx,
+                      t.tb.lo[1] + b.jy * g.by, t.tb.lo[0] + b.jt * g.bt, it.bh);
+        ++GK;
+        return true;
+      };
+      auto load_v = [&](const Item& it, const TileBlocks& t, const BlockWalk& b) -> bool {
+        const Geom& g = *it.g;
+        const uint32_t st = GV % C::kStagesV, n = GV / C::kStagesV;
+        if (!mbar_wait<set_status_fwd>(v_empty + st, (n & 1) ^ 1, abort_flag)) return false;
+        mbar_arrive_expect_tx(v_full + st, C::kHalves * g.R * 128);
+        v_arm |= 1u << st;
+        v_par = (v_par & ~(1u << st)) | ((n & 1) << st);
+        for (int h = 0; h < C::kHalves; ++h)
+          tma_load_5d(smem + C::kV + st * C::kBlock + h * 16384, it.tv, v_full + st, 64 * h, t.tb.lo[2] + b.jx * g.bx,
+                      t.tb.lo[1] + b.jy * g.by, t.tb.lo[0] + b.jt * g.bt, it.bh);
+        ++GV;
+        return true;
+      };
+      int w = blockIdx.x;
+      Item it;
+      TileBlocks t;
+      bool more = next_item(w, it, t);
+      bool ok = !more || (load_q(it, t) && load_k(it, t, BlockWalk()));
+      while (more && ok) {
+        BlockWalk b;
+        for (int j = 0; j + 1 < t.NB && ok; ++j) {
+          BlockWalk bk = b;
+          bk.next(t);
+          ok = load_k(it, t, bk) && load_v(it, t, b);
+          b = bk;
+        }
+        const Item it1 = it;
+        const TileBlocks t1 = t;
+        w += gridDim.x;
+        more = next_item(w, it, t);
+        if (t1.NB == 1) ok = ok && load_v(it1, t1, b);
+        if (more) ok = ok && load_q(it, t) && load_k(it, t, BlockWalk());
+        if (t1.NB > 1) ok = ok && load_v(it1, t1, b);
       }
       if (!ok) {
         // let every load this thread issued land before the CTA exits
         if (q_arm) mbar_wait<set_status_fwd>(q_full, q_par, abort_flag, false);
-        for (int s = 0; s < C::kStages; ++s) {
+        for (int s = 0; s < C::kStagesK; ++s) {
           if (k_arm & (1u << s)) mbar_wait<set_status_fwd>(k_full + s, (k_par >> s) & 1, abort_flag, false);
-          if (v_arm & (1u << s)) mbar_wait<set_status_fwd>(v_full + s, (v_par >> s) & 1, abort_flag, false);
+          if (l_arm & (1u << s)) mbar_wait<set_status_fwd>(k_load + s, (l_par >> s) & 1, abort_flag, false);
         }
+        for (int s = 0; s < C::kStagesV; ++s)
+          if (v_arm & (1u << s)) mbar_wait<set_status_fwd>(v_full + s, (v_par >> s) & 1, abort_flag, false);
       }
     }
   } else if (warp == 1) {
@@ -458,13 +518,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         tile_blocks(*it.g, it.tile, tbk);
         if (it.blk >= tbk.NB) continue;
         if (!(ok = mbar_wait<set_status_fwd>(qt_full, W & 1, abort_flag))) break;  // Q in TMEM
-        const bool all_full = tile_all_full(*it.g, tbk);
         BlockWalk bw;
         for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
-          const uint32_t st = G % C::kStages, sb = G & 1;
-          // a masked block's bias row was filled by the mask writer
-          const bool masked = !all_full && !bw.full(*it.g, tbk);
-          if (!(ok = mbar_wait<set_status_fwd>(k_full + st, (G / C::kStages) & 1, abort_flag))) break;
+          const uint32_t st = G % C::kStagesK, sb = G & 1;
+          // a block that reaches out of the tile comes with its bias row from the mask writer
+          const bool in = bw.inside(*it.g, tbk), masked = !in || it.g->R < 128;
+          if (!(ok = mbar_wait<set_status_fwd>(k_full + st, (G / C::kStagesK) & 1, abort_flag))) break;
           if (!(ok = mbar_wait<set_status_fwd>(s_empty + sb, ((G >> 1) & 1) ^ 1, abort_flag))) break;
           tc_fence_after();
           const uint64_t dk = dmove(dK0, st * C::kBlock);
@@ -472,7 +531,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int ks = 0; ks < D / 16; ++ks)
             umma_bf16_ts(tmem + sb * 128, tmem + C::kColQ + ks * 8, dmove(dk, (ks >> 2) * 16384 + (ks & 3) * 32),
                          idS, ks > 0);
-          if (masked) umma_bf16(tmem + sb * 128, dOnes, dmove(dBias0, st * 4096), idS, 1u);  // + bias of each key column
+          if (masked)  // + bias of each key column
+            umma_bf16(tmem + sb * 128, dOnes, dmove(dBias0, (in ? C::kStagesK : st) * 4096), idS, 1u);
           umma_commit(s_full + sb);
           umma_commit(k_empty + st);
         }
@@ -496,8 +556,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         tile_blocks(*it.g, it.tile, tbk);
         if (it.blk >= tbk.NB) continue;
         for (int j = 0; j < tbk.NB; ++j, ++G) {
-          const uint32_t st = G % C::kStages, pb = G % C::kPBufs;
-          if (!(ok = mbar_wait<set_status_fwd>(v_full + st, (G / C::kStages) & 1, abort_flag))) break;
+          const uint32_t st = G % C::kStagesV, pb = G % C::kPBufs;
+          if (!(ok = mbar_wait<set_status_fwd>(v_full + st, (G / C::kStagesV) & 1, abort_flag))) break;
           if (!(ok = mbar_wait<set_status_fwd>(p_full, G & 1, abort_flag))) break;
           if (j == 0 && !(ok = mbar_wait<set_status_fwd>(o_empty, (W & 1) ^ 1, abort_flag))) break;
           tc_fence_after();
@@ -517,10 +577,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMaskWriter) {
     // ------------------------------------------------------------ key-mask writer
-    // One arrival on k_full per stage use (the stage's second arrival), in the
-    // producer's order; it first waits until the stage is free again.
-    const uint32_t neg = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(-1e30f));
-    uint32_t G = 0;
+    // Takes a block that reaches out of its tile once its K load has landed, and
+    // gives k_full its one arrival when the block is prepared.
+    // K rows of tokens outside the tile are rows of other tiles: they are zeroed, so
+    // that whatever they hold (a NaN or an infinity would outlive any finite bias)
+    // the masked scores are 0 - inf and their probabilities exactly 0, at any scale.
+    // Rows outside the grid and rows R.. are zeros already.
+    uint32_t G = 0, l_par = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
       Item it;
@@ -531,20 +594,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (it.blk >= tbk.NB) continue;
       BlockWalk bw;
       for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
-        const uint32_t st = G % C::kStages, n = G / C::kStages;
+        const uint32_t st = G % C::kStagesK;
         const int ko[3] = {bw.jt * g.bt, bw.jy * g.by, bw.jx * g.bx};
-        if (lane == 0) ok = mbar_wait<set_status_fwd>(k_empty + st, (n & 1) ^ 1, abort_flag);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
-        if (!block_full(g, tbk, ko)) {
-          for (int r = lane; r < 128; r += 32) {
-            int kl[3];
-            block_row(g, ko, r, kl);
-            *reinterpret_cast<uint4*>(smem + C::kBias + st * 4096 + r * 16) =
-                make_uint4(inside(tbk, kl) ? 0u : neg, 0u, 0u, 0u);
-          }
-          fence_proxy_async_smem();  // the tensor core reads what these lanes wrote
+        if (block_inside(g, tbk, ko)) continue;
+        uint32_t in = 0, zero = 0;  // bit i: row lane + 32 i is a key of the tile; has to be zeroed
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = lane + 32 * i;
+          int kl[3];
+          block_row(g, ko, r, kl);
+          if (inside(tbk, kl)) in |= 1u << i;
+          else if (r < g.R && in_grid(g, tbk, kl)) zero |= 1u << i;
         }
+        ok = mbar_wait<set_status_fwd>(k_load + st, (l_par >> st) & 1, abort_flag);
+        l_par ^= 1u << st;
+        if (!(ok = __all_sync(0xffffffffu, ok) != 0)) break;
+        uint8_t* kst = smem + C::kK + st * C::kBlock;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = lane + 32 * i;
+          *reinterpret_cast<uint4*>(smem + C::kBias + st * 4096 + r * 16) =
+              make_uint4(in >> i & 1 ? 0u : kNegInf, 0u, 0u, 0u);
+          if (zero >> i & 1) {
+#pragma unroll
+            for (int u = 0; u < 8 * C::kHalves; ++u)  // whole rows: the swizzle stays within a row
+              *reinterpret_cast<uint4*>(kst + (u >> 3) * 16384 + r * 128 + ((u + r) & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+        fence_proxy_async_smem();  // the tensor core reads what these lanes wrote
         __syncwarp();
         if (lane == 0) mbar_arrive(k_full + st);
       }
