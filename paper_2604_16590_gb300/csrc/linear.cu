@@ -51,6 +51,7 @@ constexpr int kQStages = 2;
 
 __device__ void set_status_l(uint32_t c) { set_status(c); }
 #define LWAIT(bar, par) mbar_wait<set_status_l>((bar), (par), abort_flag)
+#define WARP_LWAIT(bar, par) warp_ok(LWAIT(bar, par))
 
 __device__ __forceinline__ float phi_f(float x) { return x > 0.f ? x + 1.f : ex2(x * 1.4426950408889634f); }
 
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
     // epilogue: S partial from TMEM (M = 64: rows 16q .. 16q+15 in lanes 0..15
     // of lane quadrant q; this warp's 32 of the 64 columns), z partial reduced
     // over the 128 rows in fixed order
-    const bool got = ok && LWAIT(done, 0);
+    const bool got = ok && WARP_LWAIT(done, 0);
     tc_fence_after();
     uint32_t s0[32];
     const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + 32 * h;
@@ -733,9 +734,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     for (int G = grp, n = 0; G < count; G += 2, ++n) {
       const int st = G % kBQStages;
       const bool valid = (int64_t)(t0 + G) * kTile + r < a.N;
-      if (!(ok = LWAIT(full + st, (G / kBQStages) & 1))) break;
+      // (a failed wait is carried to the pair's next vote: what is computed until
+      // then stays in shared memory)
+      ok = WARP_LWAIT(full + st, (G / kBQStages) & 1);
       // the group's low tiles are free once its previous tile's dS product is done
-      if (n > 0 && !(ok = LWAIT(lofree + grp, (n - 1) & 1))) break;
+      if (n > 0) ok = ok && WARP_LWAIT(lofree + grp, (n - 1) & 1);
       // phi(q) in FP32, this half's part of den, and phi's parts (hi over q, lo in the low tile)
       const uint32_t aq = smem_u32(stq(st)), ap = smem_u32(lop(grp));
       uint64_t dp2 = 0;
@@ -759,11 +762,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
       float d0, d1;
       f2unpack(dp2, d0, d1);
       xden[h * 128 + r] = d0 + d1;
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+      if (!(ok = pair_vote(pair_bar, ok))) break;
       const float den = xden[r] + xden[128 + r];
       const float inv = valid ? 1.f / den : 0.f;
       // this half of the U row (the U product is done: the g tile may be overwritten below)
-      if (!(ok = LWAIT(ufull + grp, n & 1))) break;
+      ok = WARP_LWAIT(ufull + grp, n & 1);
       tc_fence_after();
       // phi(q) again from its parts, eight columns of a chunk at a time
       auto phi_parts = [&](int c, uint64_t (&f)[4]) {
@@ -791,7 +794,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
       f2unpack(gp2, d0, d1);
       xgo[h * 128 + r] = d0 + d1;
       if (lane == 0) bulk_wait_read();  // the previous dq store has read this warp's staging block
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+      if (!(ok = pair_vote(pair_bar, ok))) break;
       const float go = (xgo[r] + xgo[128 + r]) * inv;
       // dq = (U - z go) / den * phi'(q); dz -= phi(q) go / den
       const uint64_t ngo2 = f2pack(-go, -go), inv2 = f2pack(inv, inv), ngi2 = f2pack(-(go * inv), -(go * inv));
@@ -849,7 +852,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     // epilogue: dS partial (M = 64: rows 16q .. 16q+15 in lanes 0..15 of lane
     // quadrant q; group 0's warps, 32 of the 64 columns each) and dz reduced
     // over both groups' 128 rows in fixed order
-    const bool got = ok && LWAIT(done, 0);
+    const bool got = ok && WARP_LWAIT(done, 0);
     tc_fence_after();
     const size_t part = (size_t)chunk * a.BH + bh;
     if (grp == 0) {
@@ -1072,13 +1075,14 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
     const uint32_t al = smem_u32(lop(grp));
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + 128 * grp + 32 * h;
     const bool storer = h == 0 && lane == 0;  // stores its quadrant's rows
+    bool ok = true;
     for (int G = grp, n = 0; G < count; G += 2, ++n) {
       const int st = G % kBKStages;
       if (n > 0 && storer) {  // the previous tile's stores have read their stage
         bulk_wait_read();
         mbar_arrive(empty + (G - 2) % kBKStages);
       }
-      if (!LWAIT(full + st, (G / kBKStages) & 1)) break;
+      ok = WARP_LWAIT(full + st, (G / kBKStages) & 1);  // a failed wait is carried to the pair's vote
       const uint32_t ak = smem_u32(stk(st)), av = smem_u32(stv(st));
       uint64_t f[16];
 #pragma unroll
@@ -1097,8 +1101,8 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(kready + grp);
-      if (!LWAIT(pfull + grp, n & 1)) break;
+      if (ok && lane == 0) mbar_arrive(kready + grp);
+      ok = ok && WARP_LWAIT(pfull + grp, n & 1);
       tc_fence_after();
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
@@ -1110,7 +1114,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
         if (hh == 1) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(pfree + grp);
+          if (ok && lane == 0) mbar_arrive(pfree + grp);
         }
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -1133,7 +1137,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_c
         }
       }
       fence_proxy_async_smem();  // the copy unit reads what these threads wrote
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+      if (!(ok = pair_vote(pair_bar, ok))) break;
       if (storer) {
         tma_store_5d(&tdk, ak + quad * 4096, 0, (t0 + G) * kTile + quad * 32, 0, 0, bh);
         tma_store_5d(&tdv, av + quad * 4096, 0, (t0 + G) * kTile + quad * 32, 0, 0, bh);

@@ -94,6 +94,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The outcome of a bounded wait, the same for every lane of the warp (false if
+// it ran out in any of them).
+__device__ __forceinline__ bool warp_ok(bool x) { return __all_sync(0xffffffffu, x) != 0; }
+// Named barrier `bar` of two warps (all 64 threads), true if both came with ok.
+// Two warps that meet inside a loop with bounded waits meet only here, also when
+// a wait has run out (with ok = false): they leave on the common outcome, so
+// that neither is left at a barrier to which the other never comes.
+__device__ __forceinline__ bool pair_vote(int bar, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %2, 0;\n\t"
+      "bar.red.and.pred p, %1, 64, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"(bar), "r"(ok ? 1u : 0u)
+      : "memory");
+  return r != 0;
+}
+
 // ------------------------------------------------------------------ TMA
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
