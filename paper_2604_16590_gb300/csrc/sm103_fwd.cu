@@ -248,7 +248,8 @@ __device__ __forceinline__ void rescale_o(uint32_t tO, float f) {
 // One 128-key block of the online softmax for this thread's half of a query
 // row: partial row max (exchanged with the partner thread), lazy rescale of
 // the reference max (and of O in TMEM, after the previous P V completed),
-// exp2 of the 64 scores into BF16 P in TMEM, row-sum update.
+// exp2 of the 64 scores into BF16 P in TMEM, row-sum update.  Returns false if
+// one of its waits, which all follow the exchange, ran out.
 template <int D>
 __device__ __forceinline__ bool softmax_block(RowState& rs, uint32_t tS, uint32_t tO, uint32_t tP, int row, int ch,
                                               int quad, float* red, int parity, float sl2,
@@ -634,9 +635,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t tO = tl + C::kColO + ch * (D / 2);
     float* red = reinterpret_cast<float*>(smem + C::kRed);
-    uint32_t G = 0, W = 0;
+    uint32_t G = 0, W = 0, Gend = 0;  // Gend: blocks up to the end of the item
     bool ok = true;
-    for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+    // The two warps of a quadrant meet at a barrier per block and one in the epilogue,
+    // at which they exchange whether their waits succeeded.  One whose wait runs out
+    // goes through its item's remaining barriers (its partner may be at any of them)
+    // and both leave at the item's last.  (An outcome exchanged with every block: 52.9
+    // -> 55.5 ms on two tiles of 136 x 32 x 64 tokens.)
+    for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
       Item it;
       if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
       const Geom& g = *it.g;
@@ -650,6 +656,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool qvalid = inside(tbk, ql);
 
       // the query block: shared memory (TMA) -> registers -> TMEM (A operand of S = Q K^T)
+      Gend = G + tbk.NB;
       if (!(ok = mbar_wait<set_status_fwd>(q_full, W & 1, abort_flag))) break;
       {
         const uint32_t sQ = smem_u32(smem + C::kQ);
@@ -687,7 +694,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t p_free_par = ((G / C::kPBufs) & 1) ^ 1;
         ok = softmax_block<D>(rs, tS, tO, tP, row, ch, quad, red, sb, g.scale_log2, j == 0, pv_last, pv_last_par,
                               pv_done + pb, p_free_par, abort_flag);
-        if (!ok) break;
+        if (!ok) {
+          ++G;  // past this block's barrier
+          break;
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
@@ -696,14 +706,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       if (!ok) break;
-      // ---- epilogue: wait for the last P V, full row sum from the two halves, O / l
-      if (!(ok = mbar_wait<set_status_fwd>(pv_done + (G - 1) % C::kPBufs, ((G - 1) / C::kPBufs) & 1, abort_flag)))
-        break;
-      tc_fence_after();
-      const float l = rs.l + pair_exchange(red, 2, ch, row, quad, rs.l);  // slot 2: epilogue only
-      const float inv = 1.f / l;
+      // ---- epilogue: where the row goes, wait for the last P V, full row sum from the two halves, O / l
       const int64_t slot = tile_slot0(g, bh, tile) + qb * 128 + row;
-      if (qvalid && ch == 0 && it.lse2) it.lse2[slot] = rs.m + __log2f(l);
       const int p[3] = {tbk.tb.lo[0] + ql[0], tbk.tb.lo[1] + ql[1], tbk.tb.lo[2] + ql[2]};
       const bool single = qvalid && only_cover(g, tbk.tb, p);
       const bool slots = __any_sync(0xffffffffu, qvalid && !single);
@@ -711,6 +715,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int c0 = ch * (D / 2);
       OutT* dst_out = static_cast<OutT*>(it.out) + ((int64_t)bh * g.N + tok) * D + c0;
       float* dst_scr = it.ot + (slot - lane) * D + c0;
+      if (!(ok = mbar_wait<set_status_fwd>(pv_done + (G - 1) % C::kPBufs, ((G - 1) / C::kPBufs) & 1, abort_flag)))
+        break;
+      tc_fence_after();
+      red[(4 + ch) * 128 + row] = rs.l;  // slot 2: epilogue only
+      if (!pair_vote(quad + 1, true)) break;  // the partner's wait ran out
+      const float l = rs.l + red[(4 + (ch ^ 1)) * 128 + row];
+      const float inv = 1.f / l;
+      if (qvalid && ch == 0 && it.lse2) it.lse2[slot] = rs.m + __log2f(l);
       uint32_t r[32];
 #pragma unroll
       for (int c = 0; c < D / 64; ++c) {
@@ -733,6 +745,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(o_empty);
       ++W;
+    }
+    if (!ok) {
+      for (; G < Gend; ++G) pair_sync(quad);
+      pair_vote(quad + 1, false);
     }
   }
   tc_fence_before();

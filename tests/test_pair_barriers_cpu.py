@@ -43,3 +43,20 @@ def test_no_pair_waits_for_a_warp_that_left(name):
     assert len(loops) == 2 and sum(b.count("pair_vote(") for b in loops) == text.count("pair_vote(") == 3
     for body in loops:
         _check_loop(body)
+
+
+def test_d128_forward_walks_its_barriers():
+    """The d = 128 forward's math warps: a warp that leaves an item early goes
+    through the barriers that its partner may still be at, then both vote."""
+    text = _source("sm103_fwd.cu")
+    start = text.index("for (int w = blockIdx.x; w < n_items; w += gridDim.x)")
+    items = _block(text, start)
+    after = re.sub(r"\s+", " ", text[start + items.__len__() :])
+    # barriers of an item: one per block (in softmax_block, before any of its waits), one vote
+    assert items.count("pair_vote(") == 1 and "pair_sync" not in items and "pair_exchange" not in items
+    block = _block(text, text.index("bool softmax_block("))
+    assert block.count("pair_exchange(") == 1 and "mbar_wait" not in block[: block.index("pair_exchange(")]
+    # G counts the block barriers passed; Gend is known before the first wait
+    assert items.index("Gend = G + tbk.NB;") < items.index("mbar_wait")
+    assert re.search(r"if \(!ok\) \{\s*\+\+G;\s*break;", items[items.index("softmax_block") :])
+    assert "if (!ok) { for (; G < Gend; ++G) pair_sync(quad); pair_vote(quad + 1, false); }" in after
