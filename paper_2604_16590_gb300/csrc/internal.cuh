@@ -127,6 +127,7 @@ struct LinearPlan {
   int chunk_tiles, chunks;      // summary
   int q_tiles;                  // query pass, tiles per CTA
   int b_chunk_tiles, b_chunks;  // both backward passes
+  int sum_tiles;                // tiles summed by the tensor core before a compensated sum takes them (both split-N passes)
 };
 LinearPlan linear_plan(int B, int nh, int64_t N);
 // Forward workspace: per-chunk FP32 partials of S and z, then the combined

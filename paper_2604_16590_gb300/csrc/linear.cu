@@ -114,13 +114,81 @@ __device__ __forceinline__ float column_sum(float* m, int t) {
   return s;
 }
 
+// ---- sums over a CTA's tiles.  The tensor core's FP32 accumulator is neither
+// compensated nor rounded to nearest, so its error grows with the number of
+// products it takes.  It is folded into a compensated sum after every `sum_tiles`
+// tiles (LinearPlan), two accumulators in turn so that the products go on
+// meanwhile; sum and compensation live in tensor memory, where the M = 64
+// accumulator lies: rows 16 q .. 16 q + 15 in lanes 0..15 of lane quadrant q.
+// Each of the eight warps that fold takes the 32 columns at its address.
+// (16 heads of 262144 tokens in 108 tiles a CTA: S and dS lay 3.0e-5 and 4.6e-5
+// from FP64 in relative RMS with one accumulator for all of them, 7.5e-6 and
+// 1.2e-5 with a CTA and a partial for every 27, 4.4e-6 and 7.2e-6 with sums of 14;
+// 64 heads: 4.1e-5 and 1.3e-4, 3.0e-5 and 4.7e-5, 4.7e-6 and 8.1e-6.  The folds
+// cost the forward nothing and the backward 2 %: 770 -> 789 us at 16 heads; a CTA
+// for every 27 tiles took 422 us forward and 825 backward, against 398 and 789.)
+__device__ __forceinline__ void kahan8(uint32_t (&s)[8], uint32_t (&c)[8], const uint32_t (&x)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float sum = __uint_as_float(s[i]);
+    const float y = __uint_as_float(x[i]) - __uint_as_float(c[i]);
+    const float t = sum + y;
+    c[i] = __float_as_uint((t - sum) - y);
+    s[i] = __float_as_uint(t);
+  }
+}
+// accumulator `acc` (its products are complete) into the sum; the first one sets it
+__device__ __forceinline__ void fold_sum(uint32_t acc, uint32_t sum, uint32_t comp, bool first) {
+#pragma unroll 1  // (registers)
+  for (int h = 0; h < 32; h += 8) {
+    uint32_t x[8], s[8], c[8];
+    tmem_ld8(acc + h, x);
+    if (first) {
+      tmem_wait_ld(x);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        s[i] = x[i];
+        c[i] = 0;
+      }
+    } else {
+      tmem_ld8(sum + h, s);
+      tmem_ld8(comp + h, c);
+      tmem_wait_ld(x);
+      tmem_wait_ld(s);
+      tmem_wait_ld(c);
+      kahan8(s, c, x);
+    }
+    tmem_st8(sum + h, s);
+    tmem_st8(comp + h, c);
+  }
+  tmem_wait_st();
+}
+// the last accumulator and, if there were others, the sum of those: this lane's 32 values
+__device__ __forceinline__ void last_sum(uint32_t acc, uint32_t sum, uint32_t comp, bool only, uint32_t (&r)[32]) {
+#pragma unroll
+  for (int h = 0; h < 32; h += 8) {
+    uint32_t x[8], s[8], c[8];
+    tmem_ld8(acc + h, x);
+    tmem_wait_ld(x);
+    if (!only) {
+      tmem_ld8(sum + h, s);
+      tmem_ld8(comp + h, c);
+      tmem_wait_ld(s);
+      tmem_wait_ld(c);
+      kahan8(s, c, x);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r[h + i] = only ? x[i] : s[i];
+  }
+}
+
 struct SumArgs {
-  int N, BH, ntiles, chunk_tiles;
+  int N, BH, ntiles, chunk_tiles, sum_tiles;
   float* ws_S;  // [chunks, BH, 64, 64]
   float* ws_z;  // [chunks, BH, 64]
 };
 
-__global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_constant__ CUtensorMap tk,
+__global__ void __launch_bounds__(kThreadsL, 2) la_summary_kernel(const __grid_constant__ CUtensorMap tk,
                                                                const __grid_constant__ CUtensorMap tv,
                                                                const SumArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -128,7 +196,9 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStagesS * kSumStage);
   uint64_t* kready = full + kStagesS;
   uint64_t* empty = kready + kStagesS;
-  uint64_t* done = empty + kStagesS;
+  uint64_t* sfull = empty + kStagesS;  // [2]: an accumulator's last product is complete
+  uint64_t* sfree = sfull + 2;         // [2]: it has been folded
+  uint64_t* done = sfree + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -140,6 +210,10 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
       mbar_init(kready + i, 8);
       mbar_init(empty + i, 1);
     }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(sfull + i, 1);
+      mbar_init(sfree + i, 8);
+    }
     mbar_init(done, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -147,7 +221,7 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
     prefetch_tmap(&tv);
   }
   if (warp == 1) {
-    tmem_alloc(tslot, 64);
+    tmem_alloc(tslot, 256);  // S accumulators at columns 0 and 64, their sum at 128, its compensation at 192
     tmem_relinquish();
   }
   tc_fence_before();
@@ -179,19 +253,27 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
       // B = V tile MN-major (N = d contiguous); a K = 16 step is 16 token rows.
       constexpr uint32_t idS = idesc_bf16(64, 64, 1) | (1u << 15);  // A MN-major
       bool ok = true;
+      int m = 0, ch = 0;  // tile within its sum, sum
       for (int t = t0, G = 0; t < t1; ++t, ++G) {
-        const int st = G % kStagesS, n = G / kStagesS;
+        const int st = G % kStagesS, n = G / kStagesS, b = ch & 1;
         if (!(ok = LWAIT(kready + st, n & 1))) break;
+        if (m == 0 && ch >= 2 && !(ok = LWAIT(sfree + b, ((ch >> 1) - 1) & 1))) break;
         tc_fence_after();
+        const uint32_t tS = tmem + 64 * b;
         const uint32_t base = smem_u32(smem + st * kSumStage);
         const uint64_t dA = sw128_desc(base, 16384, 1024), dB = sw128_desc(base + kTileBytes, 16384, 1024);
         const uint64_t dAl = sw128_desc(base + 2 * kTileBytes, 16384, 1024);
 #pragma unroll
         for (int ks = 0; ks < kTile / 16; ++ks)
-          umma_bf16(tmem, dmove(dA, ks * 2048), dmove(dB, ks * 2048), idS, (G > 0 || ks > 0) ? 1u : 0u);
+          umma_bf16(tS, dmove(dA, ks * 2048), dmove(dB, ks * 2048), idS, (m > 0 || ks > 0) ? 1u : 0u);
 #pragma unroll
-        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tmem, dmove(dAl, ks * 2048), dmove(dB, ks * 2048), idS, 1u);
+        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tS, dmove(dAl, ks * 2048), dmove(dB, ks * 2048), idS, 1u);
         umma_commit(empty + st);
+        if (++m == a.sum_tiles) {
+          umma_commit(sfull + b);
+          m = 0;
+          ++ch;
+        }
       }
       umma_commit(done);
       if (!ok) *abort_flag = 1;
@@ -206,10 +288,12 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
     float zacc[kD / 2];
 #pragma unroll
     for (int i = 0; i < kD / 2; ++i) zacc[i] = 0.f;
+    const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + 32 * h;
     bool ok = true;
+    int m = 0, ch = 0;  // tiles of the current sum, sums folded
     for (int t = t0, G = 0; t < t1; ++t, ++G) {
       const int st = G % kStagesS, n = G / kStagesS;
-      if (!(ok = LWAIT(full + st, n & 1))) break;
+      if (!(ok = WARP_LWAIT(full + st, n & 1))) break;
       uint8_t* kt = smem + st * kSumStage;
       const bool valid = t * kTile + r < a.N;
 #pragma unroll
@@ -227,6 +311,18 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
       fence_proxy_async_smem();  // the tensor core reads what these threads wrote
       __syncwarp();
       if (lane == 0) mbar_arrive(kready + st);
+      // the sum that ended with the previous tile, while this tile's products run
+      if (m == a.sum_tiles) {
+        if (!(ok = WARP_LWAIT(sfull + (ch & 1), (ch >> 1) & 1))) break;
+        tc_fence_after();
+        fold_sum(tq + 64 * (ch & 1), tq + 128, tq + 192, ch == 0);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sfree + (ch & 1));
+        ++ch;
+        m = 0;
+      }
+      ++m;
     }
     // epilogue: S partial from TMEM (M = 64: rows 16q .. 16q+15 in lanes 0..15
     // of lane quadrant q; this warp's 32 of the 64 columns), z partial reduced
@@ -234,9 +330,7 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
     const bool got = ok && WARP_LWAIT(done, 0);
     tc_fence_after();
     uint32_t s0[32];
-    const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + 32 * h;
-    tmem_ld32(tq, s0);
-    tmem_wait_ld(s0);
+    last_sum(tq + 64 * (ch & 1), tq + 128, tq + 192, ch == 0, s0);
     const size_t part = (size_t)chunk * a.BH + bh;
     if (got && lane < 16) {
       float* dst = a.ws_S + (part * kD + quad * 16 + lane) * kD + 32 * h;
@@ -258,7 +352,7 @@ __global__ void __launch_bounds__(kThreadsL) la_summary_kernel(const __grid_cons
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, 64);
+    tmem_dealloc(tmem, 256);
   }
 }
 
@@ -562,7 +656,7 @@ __device__ __forceinline__ void load_mats(int tid, int nthr, int n, const __nv_b
 }
 
 struct BQArgs {
-  int N, BH, ntiles, chunk_tiles;
+  int N, BH, ntiles, chunk_tiles, sum_tiles;
   const __nv_bfloat16* sth;  // forward summary S^T, high and low parts [BH, 64 (v), 64 (k)]
   const __nv_bfloat16* stl;
   const float* zt;           // [BH, 64]
@@ -607,7 +701,9 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
   uint64_t* ufree = ufull + 2;          // [group]
   uint64_t* dsready = ufree + 2;        // [group]
   uint64_t* lofree = dsready + 2;       // [group]
-  uint64_t* sready = lofree + 2;
+  uint64_t* sfull = lofree + 2;         // [2]: a dS accumulator's last product is complete
+  uint64_t* sfree = sfull + 2;          // [2]: it has been folded
+  uint64_t* sready = sfree + 2;
   uint64_t* done = sready + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
@@ -625,6 +721,8 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
       mbar_init(ufree + i, 8);
       mbar_init(dsready + i, 8);
       mbar_init(lofree + i, 1);
+      mbar_init(sfull + i, 1);
+      mbar_init(sfree + i, 8);
     }
     mbar_init(sready, 16);
     mbar_init(done, 1);
@@ -635,7 +733,9 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     prefetch_tmap(&tdq);
   }
   if (warp == 1) {
-    tmem_alloc(tslot, 256);  // the groups' U buffers at columns 0 and 64, dS (M = 64) at 128
+    // the groups' U buffers at columns 0 and 64, dS accumulators (M = 64) at 128 and 192, their sum at 256, its
+    // compensation at 320
+    tmem_alloc(tslot, 512);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -682,22 +782,30 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
         return true;
       };
       for (int G = 0; G < 2 && G < count && ok; ++G) ok = issue_u(G);
+      int m = 0, ch = 0;  // tile within its sum, sum
       for (int G = 0; G < count && ok; ++G) {
-        const int st = G % kBQStages, b = G & 1;
+        const int st = G % kBQStages, b = G & 1, sb = ch & 1;
         // dS += phi(Q)^T (G / den) once the math warps wrote both operands' parts
         if (!(ok = LWAIT(dsready + b, (G >> 1) & 1))) break;
+        if (m == 0 && ch >= 2 && !(ok = LWAIT(sfree + sb, ((ch >> 1) - 1) & 1))) break;
         tc_fence_after();
+        const uint32_t tD = tmem + 128 + 64 * sb;
         const uint64_t pH = sw128_desc(smem_u32(stq(st)), 16384, 1024), pL = sw128_desc(smem_u32(lop(b)), 16384, 1024);
         const uint64_t gH = sw128_desc(smem_u32(stg(st)), 16384, 1024), gL = sw128_desc(smem_u32(glo(b)), 16384, 1024);
 #pragma unroll
         for (int ks = 0; ks < kTile / 16; ++ks)
-          umma_bf16(tmem + 128, dmove(pH, ks * 2048), dmove(gH, ks * 2048), idDS, (G > 0 || ks > 0) ? 1u : 0u);
+          umma_bf16(tD, dmove(pH, ks * 2048), dmove(gH, ks * 2048), idDS, (m > 0 || ks > 0) ? 1u : 0u);
 #pragma unroll
-        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tmem + 128, dmove(pH, ks * 2048), dmove(gL, ks * 2048), idDS, 1u);
+        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tD, dmove(pH, ks * 2048), dmove(gL, ks * 2048), idDS, 1u);
 #pragma unroll
-        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tmem + 128, dmove(pL, ks * 2048), dmove(gH, ks * 2048), idDS, 1u);
+        for (int ks = 0; ks < kTile / 16; ++ks) umma_bf16(tD, dmove(pL, ks * 2048), dmove(gH, ks * 2048), idDS, 1u);
         umma_commit(empty + st);
         umma_commit(lofree + b);
+        if (++m == a.sum_tiles) {
+          umma_commit(sfull + sb);
+          m = 0;
+          ++ch;
+        }
         if (G + 2 < count) ok = issue_u(G + 2);
       }
       umma_commit(done);
@@ -730,13 +838,26 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     uint64_t dz[kD / 4];
 #pragma unroll
     for (int i = 0; i < kD / 4; ++i) dz[i] = 0;
+    // group 0 folds the sums of dS, `ch` of them so far
+    const uint32_t ts = tl + 128;
+    int ch = 0;
+    auto fold = [&]() -> bool {
+      if (!WARP_LWAIT(sfull + (ch & 1), (ch >> 1) & 1)) return false;
+      tc_fence_after();
+      fold_sum(ts + 64 * (ch & 1), ts + 128, ts + 192, ch == 0);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sfree + (ch & 1));
+      ++ch;
+      return true;
+    };
     bool ok = true;
     for (int G = grp, n = 0; G < count; G += 2, ++n) {
       const int st = G % kBQStages;
       const bool valid = (int64_t)(t0 + G) * kTile + r < a.N;
       // (a failed wait is carried to the pair's next vote: what is computed until
       // then stays in shared memory)
-      ok = WARP_LWAIT(full + st, (G / kBQStages) & 1);
+      ok = ok && WARP_LWAIT(full + st, (G / kBQStages) & 1);
       // the group's low tiles are free once its previous tile's dS product is done
       if (n > 0) ok = ok && WARP_LWAIT(lofree + grp, (n - 1) & 1);
       // phi(q) in FP32, this half's part of den, and phi's parts (hi over q, lo in the low tile)
@@ -848,7 +969,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
         tma_store_5d(&tdq, out, 32 * h, (t0 + G) * kTile + quad * 32, 0, 0, bh);
         bulk_commit();
       }
+      if (grp == 0)  // sums that ended before this tile
+        while (ok && (ch + 1) * a.sum_tiles <= G) ok = fold();
     }
+    if (grp == 0)
+      while (ok && (ch + 1) * a.sum_tiles < count) ok = fold();
     // epilogue: dS partial (M = 64: rows 16q .. 16q+15 in lanes 0..15 of lane
     // quadrant q; group 0's warps, 32 of the 64 columns each) and dz reduced
     // over both groups' 128 rows in fixed order
@@ -857,9 +982,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
     const size_t part = (size_t)chunk * a.BH + bh;
     if (grp == 0) {
       uint32_t s0[32];
-      const uint32_t tq4 = tmem + ((uint32_t)(quad * 32) << 16) + 128 + 32 * h;
-      tmem_ld32(tq4, s0);
-      tmem_wait_ld(s0);
+      last_sum(ts + 64 * (ch & 1), ts + 128, ts + 192, ch == 0, s0);
       if (got && lane < 16) {
         float* dst = a.part_dS + (part * kD + quad * 16 + lane) * kD + 32 * h;
 #pragma unroll
@@ -886,7 +1009,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, 256);
+    tmem_dealloc(tmem, 512);
   }
 }
 
@@ -1192,6 +1315,9 @@ LinearPlan linear_plan(int B, int nh, int64_t N) {
   p.q_tiles = tiles_per_cta(p.ntiles, BH, 456);      // three
   p.b_chunk_tiles = tiles_per_cta(p.ntiles, BH, 152);  // one, as the key pass
   p.b_chunks = (p.ntiles + p.b_chunk_tiles - 1) / p.b_chunk_tiles;
+  // half of what a CTA would sum with 1216 CTAs, 16 at most
+  p.sum_tiles = (int)(((int64_t)p.ntiles * BH + 2431) / 2432);
+  if (p.sum_tiles > 16) p.sum_tiles = 16;
   return p;
 }
 
@@ -1223,6 +1349,7 @@ cudaError_t launch_linear(const void* q, const void* k, const void* v, void* out
   sa.BH = BH;
   sa.ntiles = p.ntiles;
   sa.chunk_tiles = p.chunk_tiles;
+  sa.sum_tiles = p.sum_tiles;
   sa.ws_S = reinterpret_cast<float*>(w + lay.part_S);
   sa.ws_z = reinterpret_cast<float*>(w + lay.part_z);
   CombArgs ca;
@@ -1301,6 +1428,7 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   qa.BH = BH;
   qa.ntiles = p.ntiles;
   qa.chunk_tiles = p.b_chunk_tiles;
+  qa.sum_tiles = p.sum_tiles;
   qa.sth = reinterpret_cast<const __nv_bfloat16*>(sv + fl.sth);
   qa.stl = reinterpret_cast<const __nv_bfloat16*>(sv + fl.stl);
   qa.zt = reinterpret_cast<const float*>(sv + fl.z);
