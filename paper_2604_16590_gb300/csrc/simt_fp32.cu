@@ -485,6 +485,14 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_dkdv_kernel(const Geom g, 
 #pragma unroll
       for (int i = 0; i < 8; ++i) s[i][j] = exp2f(fmaf(s[i][j], g.scale_log2, nL));
     }
+    if (i0 + kBN > tb.L) {
+      // rows past the tile are zeros, which an infinite key turns into NaN: P = 0 whatever the key is
+#pragma unroll
+      for (int j = 0; j < S::KT; ++j)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (i0 + lg + S::LG * j >= tb.L) s[i][j] = 0.f;
+    }
     axpys<S>(s, sm.go, sm.p[warp], rg, lg, adv);
     dots<S>(sm.v + r0 * S::LD, sm.go, lg, dp);
     __syncthreads();  // dOut has been read
