@@ -300,7 +300,7 @@ size_t gattn_saved_bytes(const gattn_desc* desc) {
 
 size_t gattn_bwd_workspace_bytes(const gattn_desc* desc) {
   Geom g;
-  return make_geom(desc, &g) ? bwd_layout(g).bytes : 0;
+  return make_geom(desc, &g) ? bwd_layout(g, desc->in_dtype).bytes : 0;
 }
 
 gattn_status gattn_fwd(const gattn_desc* desc, const void* q, const void* k, const void* v, void* out,
@@ -342,7 +342,7 @@ gattn_status gattn_bwd(const gattn_desc* desc, const void* q, const void* k, con
   for (const void* p : ptrs)
     if (!p || !aligned16(p)) return GATTN_ERR_INVALID_ARG;
   const SavedLayout sl = saved_layout(g);
-  const BwdLayout bl = bwd_layout(g);
+  const BwdLayout bl = bwd_layout(g, desc->in_dtype);
   if (saved_bytes < sl.bytes || ws_bytes < bl.bytes) return GATTN_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const float* lse2 = reinterpret_cast<const float*>(static_cast<const char*>(saved) + sl.lse_off);
@@ -350,7 +350,7 @@ gattn_status gattn_bwd(const gattn_desc* desc, const void* q, const void* k, con
   char* w = static_cast<char*>(ws);
   float* lse2c = reinterpret_cast<float*>(w + bl.lse_off);
   float* dd = reinterpret_cast<float*>(w + bl.dd_off);
-  // the statistics rows are read only by the tensor-core dK/dV kernels
+  // these three are read only by the tensor-core kernels
   void* ext = desc->in_dtype == GATTN_BF16 ? static_cast<void*>(w + bl.ext_off) : nullptr;
   int32_t* dst = ext ? reinterpret_cast<int32_t*>(w + bl.dst_off) : nullptr;
   int32_t* nbt = ext ? reinterpret_cast<int32_t*>(w + bl.nbt_off) : nullptr;
@@ -427,7 +427,7 @@ static DpsLayout dps_layout(const gattn_desc* desc, const Geom& g) {
   const size_t nd = (size_t)g.B * g.nh * g.N * g.d;
   l.saved = 0;
   l.bws = align_up(saved_layout(g).bytes);
-  l.D = l.bws + align_up(bwd_layout(g).bytes);
+  l.D = l.bws + align_up(bwd_layout(g, desc->in_dtype).bytes);
   l.dq = l.D + align_up(nd * 4);
   l.dk = l.dq + align_up(nd * 4);
   l.dv = l.dk + align_up(nd * 4);
@@ -464,7 +464,7 @@ gattn_status gattn_dps_step(const gattn_desc* desc, const gattn_dps_params* p, f
   float* dv = reinterpret_cast<float*>(w + l.dv);
   void* r = w + l.r;
   const void* a = bf16 ? static_cast<const void*>(zb) : static_cast<const void*>(z);
-  const size_t sb = saved_layout(g).bytes, bb = bwd_layout(g).bytes;
+  const size_t sb = saved_layout(g).bytes, bb = bwd_layout(g, desc->in_dtype).bytes;
   gattn_status s = gattn_fwd(desc, a, a, a, D, w + l.saved, sb, stream);
   if (s != GATTN_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -35,25 +35,27 @@ inline SavedLayout saved_layout(const Geom& g) {
 //   dd    : float[S]      -D, D = dOut . O_t per slot, negated
 //   dq_s, dk_s, dv_s : float[S * d]  per-tile gradients of multiply-covered rows
 //   dst   : int32[S]      where a slot's output row goes: the token of a row covered by one tile, -2 for a
-//                          multiply-covered row (its slot), -1 for a slot outside the tile (tensor-core form only)
+//                          multiply-covered row (its slot), -1 for a slot outside the tile
 //   nbt   : int32[ntiles] boxes of each tile
 //   ext   : 16 B[S]       BF16 row (x0, x1, x2, y0, y1, y2, 0, 0) per slot: x0 + x1 + x2 = -lse' / (scale
 //                          log2 e) and y0 + y1 + y2 = -D, each split into three BF16 terms; the BF16
 //                          dK/dV kernels add both to S^T and dP^T with one extra K = 16 MMA step each
+// dst, nbt and ext serve the tensor-core form only and have no bytes for FP32 inputs.
 struct BwdLayout {
   size_t S, lse_off, dd_off, dst_off, nbt_off, ext_off, dq_off, dk_off, dv_off, bytes;
 };
-inline BwdLayout bwd_layout(const Geom& g) {
+inline BwdLayout bwd_layout(const Geom& g, int in_dtype) {
   BwdLayout b;
   b.S = (size_t)g.B * g.nh * g.ntiles * g.per_tile;
   size_t vec = align_up(b.S * sizeof(float));
   size_t mat = align_up(b.S * g.d * sizeof(float));
   b.lse_off = 0;
   b.dd_off = vec;
+  const bool tc = in_dtype == GATTN_BF16;
   b.dst_off = 2 * vec;
-  b.nbt_off = 3 * vec;
-  b.ext_off = b.nbt_off + align_up((size_t)g.ntiles * sizeof(int32_t));
-  b.dq_off = b.ext_off + align_up(b.S * 16);
+  b.nbt_off = b.dst_off + (tc ? vec : 0);
+  b.ext_off = b.nbt_off + (tc ? align_up((size_t)g.ntiles * sizeof(int32_t)) : 0);
+  b.dq_off = b.ext_off + (tc ? align_up(b.S * 16) : 0);
   b.dk_off = b.dq_off + mat;
   b.dv_off = b.dk_off + mat;
   b.bytes = b.dv_off + mat;
