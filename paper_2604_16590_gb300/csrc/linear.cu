@@ -646,7 +646,7 @@ __device__ __forceinline__ void split_pair(uint64_t f, uint32_t& hi, uint32_t& l
 }
 
 // 64 x 64 BF16 matrices (rows of 128 bytes) from global memory into 128-byte-
-// swizzled shared memory, n of them; every math thread (tid 0..127) takes part
+// swizzled shared memory, n of them; every math thread (tid 0..nthr - 1) takes part
 __device__ __forceinline__ void load_mats(int tid, int nthr, int n, const __nv_bfloat16* const* src,
                                           uint8_t* const* dst) {
   for (int i = tid; i < n * 64 * 8; i += nthr) {
@@ -660,7 +660,6 @@ struct BQArgs {
   const __nv_bfloat16* sth;  // forward summary S^T, high and low parts [BH, 64 (v), 64 (k)]
   const __nv_bfloat16* stl;
   const float* zt;           // [BH, 64]
-  __nv_bfloat16* dq;
   float* part_dS;            // [chunks, BH, 64 (k), 64 (v)]
   float* part_dz;            // [chunks, BH, 64]
 };
@@ -1047,11 +1046,9 @@ __global__ void __launch_bounds__(256) la_bwd_combine_kernel(const BCombArgs a) 
 }
 
 struct BKArgs {
-  int N, BH, ntiles, tiles_per_cta;
+  int ntiles, tiles_per_cta;
   const __nv_bfloat16 *dsh, *dsl, *dsth, *dstl;
   const float* dz;
-  __nv_bfloat16* dk;
-  __nv_bfloat16* dv;
 };
 
 // Key pass, grid (ceil(ntiles / tiles_per_cta), BH): per 128-token key tile
@@ -1432,7 +1429,6 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   qa.sth = reinterpret_cast<const __nv_bfloat16*>(sv + fl.sth);
   qa.stl = reinterpret_cast<const __nv_bfloat16*>(sv + fl.stl);
   qa.zt = reinterpret_cast<const float*>(sv + fl.z);
-  qa.dq = static_cast<__nv_bfloat16*>(dq);
   qa.part_dS = reinterpret_cast<float*>(w + bl.part_dS);
   qa.part_dz = reinterpret_cast<float*>(w + bl.part_dz);
   BCombArgs ca;
@@ -1446,8 +1442,6 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   ca.dstl = reinterpret_cast<__nv_bfloat16*>(w + bl.dstl);
   ca.dz = reinterpret_cast<float*>(w + bl.dz);
   BKArgs ka;
-  ka.N = (int)N;
-  ka.BH = BH;
   ka.ntiles = p.ntiles;
   ka.tiles_per_cta = p.b_chunk_tiles;
   ka.dsh = ca.dsh;
@@ -1455,8 +1449,6 @@ cudaError_t launch_linear_bwd(const void* q, const void* k, const void* v, const
   ka.dsth = ca.dsth;
   ka.dstl = ca.dstl;
   ka.dz = ca.dz;
-  ka.dk = static_cast<__nv_bfloat16*>(dk);
-  ka.dv = static_cast<__nv_bfloat16*>(dv);
 
   CUtensorMap mq, mg, mk, mv, mdq, mdk, mdv;
   if (!make_tmap_5d(&mq, q, kD, (int)N, 1, 1, BH, kTile, 1, 1) || !make_tmap_5d(&mg, dout, kD, (int)N, 1, 1, BH, kTile, 1, 1) ||

@@ -349,8 +349,8 @@ struct Oct<__nv_bfloat16> {
 // whole boxes without masking queries.  A warp takes 32 consecutive slots:
 // geometry and merge weights are computed a slot per lane, then eight lanes
 // read each row (its dOut and O_t as contiguous runs, D / 64 units of 8
-// columns a lane; 4 columns at D = 32), four rows at a time and four such
-// loads in flight.  (A thread reading its own rows, 16 bytes at a time: 0.69 ms
+// columns a lane) and four rows a step; at D = 32 four lanes and eight rows.
+// Four units of a lane are in flight.  (A thread reading its own rows, 16 bytes at a time: 0.69 ms
 // against 0.67 on 16 heads of 1024 tiles of 24 x 24, 82 us against 64 on the
 // long temporal context at d = 128.)
 template <typename OutT, typename InT, int D>
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
 #pragma unroll 1
     for (int it0 = 0; it0 < L; it0 += BATCH) {
       Oct<InT> a[BATCH][U];
-      Oct<OutT> o1[BATCH][U];
+      Oct<OutT> o1[BATCH][U];  // BF16 outputs only: FP32 rows and slots share the registers of o2
       Oct<float> o2[BATCH][U];
 #pragma unroll
       for (int b = 0; b < BATCH; ++b) {
@@ -418,8 +418,10 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
         for (int u = 0; u < U; ++u) {
           const int c = 8 * (sub + L * u);
           a[b][u].load(dout + r * D + c);
-          if (singles >> src & 1) o1[b][u].load(out + r * D + c);
-          else o2[b][u].load(ot + (slot - lane + src) * D + c);
+          const float* slot_row = ot + (slot - lane + src) * D + c;
+          if constexpr (sizeof(OutT) == 4) o2[b][u].load(singles >> src & 1 ? out + r * D + c : slot_row);
+          else if (singles >> src & 1) o1[b][u].load(out + r * D + c);
+          else o2[b][u].load(slot_row);
         }
       }
 #pragma unroll
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(kThreads) bwd_prep_kernel(Geom g, const OutT* 
           for (int u = 0; u < U; ++u) {
             float x[8], y[8];
             a[b][u].get(x);
-            if (singles >> src & 1) o1[b][u].get(y);
+            if (sizeof(OutT) == 2 && singles >> src & 1) o1[b][u].get(y);
             else o2[b][u].get(y);
 #pragma unroll
             for (int e = 0; e < 8; ++e) s = fmaf(x[e], y[e], s);

@@ -118,7 +118,7 @@ struct Item {
   const CUtensorMap* tk;
   const CUtensorMap* tv;
   void* out;
-  float* lse2;  // may be null (no backward)
+  float* lse2;  // null in ragged mode, which stores none
   float* ot;    // ragged mode (else the slots' tensor map serves)
   int bh, tile, pair;
   int req;  // request index (ragged mode), else -1
