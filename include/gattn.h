@@ -34,6 +34,13 @@
  * caller passes the saved-state and workspace buffers, sized by the query
  * functions below.  Every call is asynchronous on the given CUDA stream.
  *
+ * Non-finite inputs.  A NaN or an infinity reaches the tiles that contain its
+ * token.  The BF16 form reads tiles in boxes of up to 128 tokens that may reach
+ * past a tile's end, and a non-finite value there can also reach the outputs and
+ * gradients of that tile; only the d = 128 forward keeps those of K out.  Keys
+ * past a tile's end are masked for scales of about 1e-28 and more, in the
+ * d = 128 forward for every scale.
+ *
  * Errors.  Argument and shape errors are returned synchronously, before any
  * launch.  A failed launch returns GATTN_ERR_CUDA.  Device-side conditions
  * (a bounded wait that ran out, a debug bounds check) set a per-library

@@ -6,7 +6,7 @@
 //
 // Work decomposition: one CTA per (row block, tile, batch*head); a warp owns
 // 8 RG rows of the extended tile, keys (or queries, for dK/dV) stream through
-// shared memory 64 at a time.  Both kinds of products are register-tiled, 8
+// shared memory 64 at a time (32 for short tiles, see with_shape).  Both kinds of products are register-tiled, 8
 // rows per thread, and issue packed FP32 pairs (fma.rn.f32x2), so that the FMA
 // pipe is the limit and not the issue slots or the shared-memory reads:
 //   scores   8 rows x KT keys a thread, contraction over d in pairs of
@@ -19,7 +19,7 @@
 //            loads per 16 pair instructions (with P doubled in shared memory
 //            instead, 5: the loads, not the FMAs, then set the pace)
 // Rows never leave their warp: P goes through a warp-private buffer, so CTA
-// barriers only order the streamed blocks.  Every 64-row block is reduced
+// barriers only order the streamed blocks.  Every streamed block is reduced
 // locally before it is folded into the running sums (two-level summation,
 // which keeps the FP32 error of L-long sums near eps * (sqrt(64) + sqrt(L/64))).
 // Bound: the FP32 pipe (128 lanes a clock and SM), 53-57 % active with two
@@ -40,24 +40,24 @@ using sm103::fadd2;
 using sm103::ffma2;
 using sm103::fmul2;
 
-constexpr int kBN = 64;  // streamed rows per block
-
-// Shape of the kernels at head size D with W warps per CTA and RG row groups
-// of 8 rows per warp.
-template <int D_, int W_, int RG_>
+// Shape of the kernels at head size D with W warps per CTA, RG row groups of 8
+// rows per warp and BN streamed rows per block.
+template <int D_, int W_, int RG_, int BN_ = 64>
 struct Shape {
-  static constexpr int D = D_, W = W_, RG = RG_;
+  static constexpr int D = D_, W = W_, RG = RG_, BN = BN_;
   static constexpr int LG = 32 / RG;            // lanes of a row group
-  static constexpr int KT = kBN / LG;           // score columns per thread: keys lg + LG * jj
+  static constexpr int KT = BN / LG;            // score columns per thread: keys lg + LG * jj
   static constexpr int CT = D / LG;             // output columns per thread: CT * lg ...
   static constexpr int WR = 8 * RG;             // rows per warp
   static constexpr int BM = W * WR;             // rows per CTA
   static constexpr int T = 32 * W;
   static constexpr int LD = D + 4;              // padded row of a staged matrix (floats): conflict-free column walks
-  static constexpr int HJ = RG == 1 && D == 64 ? 1 : 2;  // score columns per thread exchanged at a time
+  static constexpr int HJ = KT == 1 || (RG == 1 && D == 64) ? 1 : 2;  // score columns per thread exchanged at a time
   static constexpr int HK = HJ * LG;            // keys of P exchanged at a time
-  static constexpr int NH = kBN / HK;
-  static constexpr int CTAS = D == 128 ? 1 : 2;  // resident CTAs per SM (shared memory)
+  static constexpr int NH = BN / HK;
+  // resident CTAs per SM (registers, shared memory)
+  static constexpr int CTAS = D == 128 ? (BN == 64 ? 1 : W == 2 ? 3 : 2) : D == 64 ? (BN == 64 ? 2 : 4) : BN == 32 ? 16 / W : W == 4 ? 3 : 2;
+  static constexpr bool SKIP = BN < 64;         // warps without a row of the tile only stage
   static constexpr int PB = WR + 4;             // floats per key of the P buffer, padded
   static constexpr int PW = HK * PB;            // floats of a warp's P buffer
 };
@@ -234,8 +234,8 @@ __device__ __forceinline__ float group_sum(float v) {
 template <class S>
 struct FwdSmem {
   float q[S::BM * S::LD];
-  float k[2][kBN * S::LD];
-  float v[2][kBN * S::LD];
+  float k[2][S::BN * S::LD];
+  float v[2][S::BN * S::LD];
   float p[S::W][S::PW];
 };
 
@@ -255,9 +255,10 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_fwd_kernel(const Geom g, c
   const int rg = lane / S::LG, lg = lane % S::LG;
   const int64_t base = (int64_t)bh * g.N * S::D;
   stage<S, S::BM>(g, tb, row0, Q + base, sm.q);
-  stage<S, kBN>(g, tb, 0, K + base, sm.k[0]);
-  stage<S, kBN>(g, tb, 0, V + base, sm.v[0]);
+  stage<S, S::BN>(g, tb, 0, K + base, sm.k[0]);
+  stage<S, S::BN>(g, tb, 0, V + base, sm.v[0]);
   cp_commit();
+  const bool busy = row0 + warp * S::WR < tb.L;  // the warp has a row of the tile
   const int r0 = warp * S::WR + rg * 8;  // first of this thread's 8 rows within the CTA
   float* pb = sm.p[warp];
 
@@ -269,14 +270,15 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_fwd_kernel(const Geom g, c
     m[i] = -INFINITY;
     l[i] = 0.f;
   }
-  for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
+  for (int j0 = 0, b = 0; j0 < tb.L; j0 += S::BN, b ^= 1) {
     cp_wait<0>();
     __syncthreads();  // block j0 is staged, block j0 - 64 has been read by every warp
-    if (j0 + kBN < tb.L) {
-      stage<S, kBN>(g, tb, j0 + kBN, K + base, sm.k[b ^ 1]);
-      stage<S, kBN>(g, tb, j0 + kBN, V + base, sm.v[b ^ 1]);
+    if (j0 + S::BN < tb.L) {
+      stage<S, S::BN>(g, tb, j0 + S::BN, K + base, sm.k[b ^ 1]);
+      stage<S, S::BN>(g, tb, j0 + S::BN, V + base, sm.v[b ^ 1]);
       cp_commit();
     }
+    if (S::SKIP && !busy) continue;
     float s[8][S::KT];
     dots<S>(sm.q + r0 * S::LD, sm.k[b], lg, s);
 #pragma unroll
@@ -333,8 +335,8 @@ template <class S>
 struct DqSmem {
   float q[S::BM * S::LD];
   float go[S::BM * S::LD];
-  float k[2][kBN * S::LD];
-  float v[kBN * S::LD];
+  float k[2][S::BN * S::LD];
+  float v[S::BN * S::LD];
   float p[S::W][S::PW];
 };
 
@@ -356,9 +358,10 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_dq_kernel(const Geom g, co
   const int64_t base = (int64_t)bh * g.N * S::D;
   stage<S, S::BM>(g, tb, row0, Q + base, sm.q);
   stage<S, S::BM>(g, tb, row0, dO + base, sm.go);
-  stage<S, kBN>(g, tb, 0, K + base, sm.k[0]);
-  stage<S, kBN>(g, tb, 0, V + base, sm.v);
+  stage<S, S::BN>(g, tb, 0, K + base, sm.k[0]);
+  stage<S, S::BN>(g, tb, 0, V + base, sm.v);
   cp_commit();
+  const bool busy = row0 + warp * S::WR < tb.L;  // the warp has a row of the tile
   const int r0 = warp * S::WR + rg * 8;
   float nL[8], nD[8];  // -lse' and -D (negated in the workspace)
 #pragma unroll
@@ -376,25 +379,28 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_dq_kernel(const Geom g, co
   }
   Acc<S> acc;
   zero_acc<S>(acc);
-  for (int j0 = 0, b = 0; j0 < tb.L; j0 += kBN, b ^= 1) {
-    const bool more = j0 + kBN < tb.L;
+  for (int j0 = 0, b = 0; j0 < tb.L; j0 += S::BN, b ^= 1) {
+    const bool more = j0 + S::BN < tb.L;
     cp_wait<0>();
     __syncthreads();  // block j0 is staged, the other K buffer has been read
-    if (more) stage<S, kBN>(g, tb, j0 + kBN, K + base, sm.k[b ^ 1]);
+    if (more) stage<S, S::BN>(g, tb, j0 + S::BN, K + base, sm.k[b ^ 1]);
     float s[8][S::KT], dp[8][S::KT];
-    dots<S>(sm.q + r0 * S::LD, sm.k[b], lg, s);
+    if (!S::SKIP || busy) {
+      dots<S>(sm.q + r0 * S::LD, sm.k[b], lg, s);
 #pragma unroll
-    for (int j = 0; j < S::KT; ++j) {
-      const bool in = j0 + lg + S::LG * j < tb.L;
+      for (int j = 0; j < S::KT; ++j) {
+        const bool in = j0 + lg + S::LG * j < tb.L;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) s[i][j] = in ? exp2f(fmaf(s[i][j], g.scale_log2, nL[i])) : 0.f;
+        for (int i = 0; i < 8; ++i) s[i][j] = in ? exp2f(fmaf(s[i][j], g.scale_log2, nL[i])) : 0.f;
+      }
+      dots<S>(sm.go + r0 * S::LD, sm.v, lg, dp);
     }
-    dots<S>(sm.go + r0 * S::LD, sm.v, lg, dp);
     __syncthreads();  // V has been read
     if (more) {
-      stage<S, kBN>(g, tb, j0 + kBN, V + base, sm.v);
+      stage<S, S::BN>(g, tb, j0 + S::BN, V + base, sm.v);
       cp_commit();
     }
+    if (S::SKIP && !busy) continue;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
@@ -421,10 +427,10 @@ template <class S>
 struct DkvSmem {
   float k[S::BM * S::LD];
   float v[S::BM * S::LD];
-  float q[2][kBN * S::LD];
-  float go[kBN * S::LD];
+  float q[2][S::BN * S::LD];
+  float go[S::BN * S::LD];
   float p[S::W][S::PW];
-  float nL[2][kBN], nD[2][kBN];
+  float nL[2][S::BN], nD[2][S::BN];
 };
 
 template <class S, typename OutT>
@@ -446,7 +452,7 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_dkdv_kernel(const Geom g, 
   const int64_t base = (int64_t)bh * g.N * S::D;
   // -lse' and -D of the block's queries; rows past the tile get P = 0
   auto stats = [&](int i0, int b) {
-    for (int t = threadIdx.x; t < kBN; t += S::T) {
+    for (int t = threadIdx.x; t < S::BN; t += S::T) {
       float a = -INFINITY, d = 0.f;
       if (i0 + t < tb.L) {
         int lr[3];
@@ -461,45 +467,49 @@ __global__ void __launch_bounds__(S::T, S::CTAS) simt_dkdv_kernel(const Geom g, 
   };
   stage<S, S::BM>(g, tb, row0, K + base, sm.k);
   stage<S, S::BM>(g, tb, row0, V + base, sm.v);
-  stage<S, kBN>(g, tb, 0, Q + base, sm.q[0]);
-  stage<S, kBN>(g, tb, 0, dO + base, sm.go);
+  stage<S, S::BN>(g, tb, 0, Q + base, sm.q[0]);
+  stage<S, S::BN>(g, tb, 0, dO + base, sm.go);
   cp_commit();
   stats(0, 0);
+  const bool busy = row0 + warp * S::WR < tb.L;  // the warp has a row of the tile
   const int r0 = warp * S::WR + rg * 8;
   Acc<S> adk, adv;
   zero_acc<S>(adk);
   zero_acc<S>(adv);
-  for (int i0 = 0, b = 0; i0 < tb.L; i0 += kBN, b ^= 1) {
-    const bool more = i0 + kBN < tb.L;
+  for (int i0 = 0, b = 0; i0 < tb.L; i0 += S::BN, b ^= 1) {
+    const bool more = i0 + S::BN < tb.L;
     cp_wait<0>();
     __syncthreads();  // block i0 is staged, the other Q buffer has been read
     if (more) {
-      stage<S, kBN>(g, tb, i0 + kBN, Q + base, sm.q[b ^ 1]);
-      stats(i0 + kBN, b ^ 1);
+      stage<S, S::BN>(g, tb, i0 + S::BN, Q + base, sm.q[b ^ 1]);
+      stats(i0 + S::BN, b ^ 1);
     }
     float s[8][S::KT], dp[8][S::KT];
-    dots<S>(sm.k + r0 * S::LD, sm.q[b], lg, s);
+    if (!S::SKIP || busy) {
+      dots<S>(sm.k + r0 * S::LD, sm.q[b], lg, s);
 #pragma unroll
-    for (int j = 0; j < S::KT; ++j) {
-      const float nL = sm.nL[b][lg + S::LG * j];
+      for (int j = 0; j < S::KT; ++j) {
+        const float nL = sm.nL[b][lg + S::LG * j];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) s[i][j] = exp2f(fmaf(s[i][j], g.scale_log2, nL));
+        for (int i = 0; i < 8; ++i) s[i][j] = exp2f(fmaf(s[i][j], g.scale_log2, nL));
+      }
+      if (i0 + S::BN > tb.L) {
+        // rows past the tile are zeros, which an infinite key turns into NaN: P = 0 whatever the key is
+#pragma unroll
+        for (int j = 0; j < S::KT; ++j)
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (i0 + lg + S::LG * j >= tb.L) s[i][j] = 0.f;
+      }
+      axpys<S>(s, sm.go, sm.p[warp], rg, lg, adv);
+      dots<S>(sm.v + r0 * S::LD, sm.go, lg, dp);
     }
-    if (i0 + kBN > tb.L) {
-      // rows past the tile are zeros, which an infinite key turns into NaN: P = 0 whatever the key is
-#pragma unroll
-      for (int j = 0; j < S::KT; ++j)
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (i0 + lg + S::LG * j >= tb.L) s[i][j] = 0.f;
-    }
-    axpys<S>(s, sm.go, sm.p[warp], rg, lg, adv);
-    dots<S>(sm.v + r0 * S::LD, sm.go, lg, dp);
     __syncthreads();  // dOut has been read
     if (more) {
-      stage<S, kBN>(g, tb, i0 + kBN, dO + base, sm.go);
+      stage<S, S::BN>(g, tb, i0 + S::BN, dO + base, sm.go);
       cp_commit();
     }
+    if (S::SKIP && !busy) continue;
 #pragma unroll
     for (int j = 0; j < S::KT; ++j) {
       const float nD = sm.nD[b][lg + S::LG * j];
@@ -563,17 +573,36 @@ cudaError_t bwd_run(const Geom& g, const float* q, const float* k, const float* 
   return cudaGetLastError();
 }
 
-// Runs f with the shape for this problem.  64-row CTAs of warps with 16 rows
-// (8 x 4 score tiles a thread: fewest shared-memory reads per FMA), or, where
-// those would leave SMs without a CTA, 32-row CTAs of warps with 8 rows (8 x 2
-// tiles, twice the warps: a training step on one head of a 64 x 64 frame 285
-// us, 16-row warps 311; the 8-row form costs large problems 15 %).
+// Runs f with the shape for this problem.
+//   Tiles of more than 32 rows: 64-row CTAs of warps with 16 rows (8 x 4 score
+// tiles a thread: fewest shared-memory reads per FMA), or, where those would
+// leave SMs without a CTA, 32-row CTAs of warps with 8 rows (8 x 2 tiles, twice
+// the warps: a training step on one head of a 64 x 64 frame 285 us, 16-row warps
+// 311; the 8-row form costs large problems 15 %).
+//   Tiles of up to 32 rows: blocks of 32 rows and 32-row CTAs (16 rows at d = 128
+// up to 16), twice as many of them per SM, whose warps without a row only stage.
+// Blocks of 64 make such a tile pay for 64 x 64 scores: training steps of 4096
+// tiles of 16 rows took 465, 660 and 1404 us at d = 32, 64 and 128, now 168, 252
+// and 435; at 36 rows the larger blocks are ahead (d = 64 729 against 782).
+//   d = 32: a product is too short to hide its loads with eight warps per SM, so
+// blocks of 32 and four CTAs up to 448 rows (1024 tiles of 64 rows 154 -> 127 us,
+// of 144 669 -> 536, 400-row tiles 802 -> 742), beyond them blocks of 64 and three.
 template <int D, typename F>
 cudaError_t with_shape(const Geom& g, F f) {
   const int64_t blocks = (int64_t)((g.Lmax + 63) / 64) * g.ntiles * g.B * g.nh;
-  if constexpr (D == 128) return blocks > num_sms() ? f(Shape<D, 8, 1>()) : f(Shape<D, 4, 1>());
-  else if constexpr (D == 64) return blocks > num_sms() ? f(Shape<D, 4, 2>()) : f(Shape<D, 4, 1>());
-  else return blocks > num_sms() ? f(Shape<D, 4, 2>()) : f(Shape<D, 2, 2>());
+  const bool many = blocks > num_sms();
+  if constexpr (D == 128) {
+    if (g.Lmax <= 16) return f(Shape<D, 2, 1, 32>());
+    if (g.Lmax <= 32) return f(Shape<D, 4, 1, 32>());
+    return many ? f(Shape<D, 8, 1>()) : f(Shape<D, 4, 1>());
+  } else if constexpr (D == 64) {
+    if (g.Lmax <= 32) return f(Shape<D, 4, 1, 32>());
+    return many ? f(Shape<D, 4, 2>()) : f(Shape<D, 4, 1>());
+  } else {
+    if (g.Lmax <= 32) return f(Shape<D, 2, 2, 32>());
+    if (!many) return f(Shape<D, 2, 2>());
+    return g.Lmax <= 448 ? f(Shape<D, 4, 2, 32>()) : f(Shape<D, 4, 2>());
+  }
 }
 
 template <typename F>

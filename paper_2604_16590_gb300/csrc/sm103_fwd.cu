@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // for a K block loaded after it: with K behind V and two K stages the forward
     // took 56.1 ms on two tiles of 136 x 32 x 64 tokens (52.9 now), and the mask
     // writer's turn between a masked block's load and its product would have cost
-    // the ragged 7 x 45 x 77 crop of 12 heads 9 % (1.55 -> 1.69 ms; 1.44 now).
+    // the ragged 7 x 45 x 77 crop of 12 heads 9 % (1.55 -> 1.69 ms; 1.46 now).
     if (lane == 0) {
       uint32_t GK = 0, GV = 0, W = 0;
       // arming record for the abort drain: bit s of k_arm/v_arm (l_arm: k_load) =
