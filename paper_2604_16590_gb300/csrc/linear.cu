@@ -677,8 +677,8 @@ struct BQArgs {
 //           of a row's 64 columns each and exchange the row's two sums (den,
 //           phi(q) . U) through shared memory, added in a fixed order.
 // At the end the CTA writes its dS and dz partials.  16 heads of 262144
-// tokens: 705 -> 436 us (one group of eight warps, plain stores of dq and
-// 1216 CTAs before); 1.61 GB in that time, 0.54 of the HBM rate: the math
+// tokens: 705 -> 453 us (one group of eight warps, plain stores of dq and
+// 1216 CTAs before; 436 without the folds); 1.61 GB, 0.53 of the HBM rate: the math
 // groups' row work (phi, its parts, the row sums) sets the pace.
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_query_kernel(const __grid_constant__ CUtensorMap tq,
                                                                     const __grid_constant__ CUtensorMap tg,
@@ -1063,8 +1063,8 @@ struct BKArgs {
 // A stage is released by the four quadrants once their stores have read it.
 // Two math warps per group and TMEM lane quadrant, each taking 32 of a row's
 // 64 columns (nothing here sums over a row).  16 heads of 262144 tokens:
-// 713 -> 327 us (one group of eight warps, a thread storing its own 64
-// bytes of a row and 16 tiles per CTA before); 2.15 GB in that time, 0.97 of
+// 713 -> 324 us (one group of eight warps, a thread storing its own 64
+// bytes of a row and 16 tiles per CTA before); 2.15 GB in that time, 0.98 of
 // the HBM rate.
 __global__ void __launch_bounds__(kThreadsB, 1) la_bwd_key_kernel(const __grid_constant__ CUtensorMap tk,
                                                                   const __grid_constant__ CUtensorMap tv,
@@ -1285,7 +1285,8 @@ constexpr int kQSmem = 16384 + (kQStages + 1) * kTileBytes + 1024 + 512;
 // fill of its ring, and the split-N passes for a partial that the combine reads
 // (forward and backward, one head of 1.5 M tokens: 1087 -> 484 us with the
 // sixteen-load combine, half of it from the combines; 16 heads of 262144:
-// 1360 -> 1164; before, 1216 CTAs or 16 tiles each whatever the problem).
+// 1360 -> 1164, 1183 with the folded sums; before, 1216 CTAs or 16 tiles each
+// whatever the problem).
 static int tiles_per_cta(int ntiles, int BH, int slots) {
   int best = 1;
   double full = 0.0;
@@ -1312,9 +1313,10 @@ LinearPlan linear_plan(int B, int nh, int64_t N) {
   p.q_tiles = tiles_per_cta(p.ntiles, BH, 456);      // three
   p.b_chunk_tiles = tiles_per_cta(p.ntiles, BH, 152);  // one, as the key pass
   p.b_chunks = (p.ntiles + p.b_chunk_tiles - 1) / p.b_chunk_tiles;
-  // half of what a CTA would sum with 1216 CTAs, 16 at most
-  p.sum_tiles = (int)(((int64_t)p.ntiles * BH + 2431) / 2432);
-  if (p.sum_tiles > 16) p.sum_tiles = 16;
+  // half of a CTA's share if there were 1216 CTAs (a share of two whole: a fold per
+  // tile cost 4 x 60000 tokens 2 %), 16 at most
+  const int share = (int)(((int64_t)p.ntiles * BH + 1215) / 1216);
+  p.sum_tiles = share <= 2 ? share : share < 32 ? (share + 1) / 2 : 16;
   return p;
 }
 
