@@ -62,9 +62,13 @@ __device__ __forceinline__ void block_row(const Geom& g, const int o[3], int rho
   l[2] = o[2] + b[2];
 }
 
+// no block of the tile reaches out of it
+__device__ __forceinline__ bool tile_inside(const Geom& g, const TileBlocks& t) {
+  return t.nb[0] * g.bt == t.tb.e[0] && t.nb[1] * g.by == t.tb.e[1] && t.nb[2] * g.bx == t.tb.e[2];
+}
 // every block of the tile holds 128 rows of the tile (no padding anywhere)
 __device__ __forceinline__ bool tile_all_full(const Geom& g, const TileBlocks& t) {
-  return g.R == 128 && t.nb[0] * g.bt == t.tb.e[0] && t.nb[1] * g.by == t.tb.e[1] && t.nb[2] * g.bx == t.tb.e[2];
+  return g.R == 128 && tile_inside(g, t);
 }
 
 // Walks the blocks of a tile in index order with counters instead of

@@ -173,6 +173,7 @@ constexpr int kThreads = 64 + 32 * kMathWarps + 64;
 constexpr int kIssuerPV = 2 + kMathWarps;  // warp index of the P V issuer
 constexpr int kMaskWriter = kIssuerPV + 1;
 constexpr uint32_t kNegInf = 0xFF80u;  // BF16 -inf
+constexpr int kLeanBlocks = 512;       // see the TMA producer
 
 // Online-softmax state of one query row, as held by one of its two threads.
 // P = exp2(s S log2e - m) is formed against a reference max m that only moves
@@ -397,12 +398,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     // K runs one block ahead of V, over the items' ends too (after an item of one
-    // block its V goes first: the next item's Q waits for this item to begin).  A V
-    // stage comes free only with the P V product of two blocks before, too late
-    // for a K block loaded after it: with K behind V and two K stages the forward
-    // took 56.1 ms on two tiles of 136 x 32 x 64 tokens (52.9 now), and the mask
-    // writer's turn between a masked block's load and its product would have cost
-    // the ragged 7 x 45 x 77 crop of 12 heads 9 % (1.55 -> 1.69 ms; 1.46 now).
+    // block its V goes first: the next item's Q waits for this item to begin): a V
+    // stage comes free only with the P V product of two blocks before, too late for a
+    // K block loaded after it to take the mask writer's turn unseen (the ragged 7 x 45
+    // x 77 crop of 12 heads 1.55 ms before that writer zeroed K rows, 1.69 with K
+    // behind V, 1.47 now).
+    //   Tiles of more than kLeanBlocks blocks with nothing to mask load K and V in
+    // turn, in a loop of their own (this thread is on the path from product to product
+    // then: 58.1 ms instead of 56.4 on two tiles of 2176 blocks with the loop below).
+    // K ahead of V is faster on them for a moment (52.9 ms), but such a run then meets
+    // the power limit: four heads of two tiles of 2048 blocks, over three seconds, take
+    // 220 ms at 1.44 GHz instead of 202 at 2.0.  Shorter tiles stay below it: 512
+    // blocks 23.9 ms against 25.5, 1024 98.4 against 101, 36 4.27 against 4.54.
     if (lane == 0) {
       uint32_t GK = 0, GV = 0, W = 0;
       // arming record for the abort drain: bit s of k_arm/v_arm (l_arm: k_load) =
@@ -418,6 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         return false;
       };
+      auto lean = [&](const Item& it, const TileBlocks& t) { return t.NB > kLeanBlocks && tile_inside(*it.g, t); };
       auto load_q = [&](const Item& it, const TileBlocks& t) -> bool {
         if (RAGGED && it.req != last_req) {
           tmap_acquire(it.tq);  // this launch's descriptor table may hold a new map here
@@ -470,25 +478,54 @@ __global__ void __launch_bounds__(kThreads, 1)
         return true;
       };
       int w = blockIdx.x;
-      Item it;
-      TileBlocks t;
-      bool more = next_item(w, it, t);
-      bool ok = !more || (load_q(it, t) && load_k(it, t, BlockWalk()));
+      Item it, it1;
+      TileBlocks t, t1;
+      // loaded: the item's Q and first K block are on their way
+      bool more = next_item(w, it, t), loaded = false, ok = true;
       while (more && ok) {
-        BlockWalk b;
-        for (int j = 0; j + 1 < t.NB && ok; ++j) {
-          BlockWalk bk = b;
-          bk.next(t);
-          ok = load_k(it, t, bk) && load_v(it, t, b);
-          b = bk;
+        if (lean(it, t)) {
+          const Geom& g = *it.g;
+          const int bh = it.bh;
+          if (!(ok = load_q(it, t))) break;
+          BlockWalk b;
+          for (int j = 0; j < t.NB; ++j, ++GK, ++GV, b.next(t)) {
+            const uint32_t sk = GK % C::kStagesK, nk = GK / C::kStagesK, sv = GV % C::kStagesV, nv = GV / C::kStagesV;
+            const int c1 = t.tb.lo[2] + b.jx * g.bx, c2 = t.tb.lo[1] + b.jy * g.by, c3 = t.tb.lo[0] + b.jt * g.bt;
+            if (!(ok = mbar_wait<set_status_fwd>(k_empty + sk, (nk & 1) ^ 1, abort_flag))) break;
+            mbar_arrive_expect_tx(k_full + sk, C::kHalves * g.R * 128);
+            k_arm |= 1u << sk;
+            k_par = (k_par & ~(1u << sk)) | ((nk & 1) << sk);
+            for (int h = 0; h < C::kHalves; ++h)
+              tma_load_5d(smem + C::kK + sk * C::kBlock + h * 16384, it.tk, k_full + sk, 64 * h, c1, c2, c3, bh);
+            if (!(ok = mbar_wait<set_status_fwd>(v_empty + sv, (nv & 1) ^ 1, abort_flag))) break;
+            mbar_arrive_expect_tx(v_full + sv, C::kHalves * g.R * 128);
+            v_arm |= 1u << sv;
+            v_par = (v_par & ~(1u << sv)) | ((nv & 1) << sv);
+            for (int h = 0; h < C::kHalves; ++h)
+              tma_load_5d(smem + C::kV + sv * C::kBlock + h * 16384, it.tv, v_full + sv, 64 * h, c1, c2, c3, bh);
+          }
+          w += gridDim.x;
+          more = next_item(w, it, t);
+          continue;
         }
-        const Item it1 = it;
-        const TileBlocks t1 = t;
+        BlockWalk b, bk;
+        if (!loaded) ok = load_q(it, t);
+        int nk = 0;  // K blocks loaded
+        if (loaded) {
+          nk = 1;
+          bk.next(t);
+        }
+        loaded = false;
         w += gridDim.x;
-        more = next_item(w, it, t);
-        if (t1.NB == 1) ok = ok && load_v(it1, t1, b);
-        if (more) ok = ok && load_q(it, t) && load_k(it, t, BlockWalk());
-        if (t1.NB > 1) ok = ok && load_v(it1, t1, b);
+        more = next_item(w, it1, t1);
+        for (int j = 0; j < t.NB && ok; ++j, b.next(t)) {
+          for (; nk < j + 2 && nk < t.NB && ok; ++nk, bk.next(t)) ok = load_k(it, t, bk);
+          if (j > 0 && j + 1 == t.NB && ok && more && !lean(it1, t1))
+            loaded = ok = load_q(it1, t1) && load_k(it1, t1, BlockWalk());
+          ok = ok && load_v(it, t, b);
+        }
+        it = it1;
+        t = t1;
       }
       if (!ok) {
         // let every load this thread issued land before the CTA exits
@@ -519,11 +556,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         tile_blocks(*it.g, it.tile, tbk);
         if (it.blk >= tbk.NB) continue;
         if (!(ok = mbar_wait<set_status_fwd>(qt_full, W & 1, abort_flag))) break;  // Q in TMEM
+        const bool all_in = tile_inside(*it.g, tbk), pad = it.g->R < 128;
         BlockWalk bw;
         for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
           const uint32_t st = G % C::kStagesK, sb = G & 1;
           // a block that reaches out of the tile comes with its bias row from the mask writer
-          const bool in = bw.inside(*it.g, tbk), masked = !in || it.g->R < 128;
+          bool in = true, masked = pad;
+          if (!all_in) {
+            in = bw.inside(*it.g, tbk);
+            masked = masked || !in;
+          }
           if (!(ok = mbar_wait<set_status_fwd>(k_full + st, (G / C::kStagesK) & 1, abort_flag))) break;
           if (!(ok = mbar_wait<set_status_fwd>(s_empty + sb, ((G >> 1) & 1) ^ 1, abort_flag))) break;
           tc_fence_after();
@@ -593,6 +635,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       TileBlocks tbk;
       tile_blocks(g, it.tile, tbk);
       if (it.blk >= tbk.NB) continue;
+      if (tile_inside(g, tbk)) {
+        G += tbk.NB;
+        continue;
+      }
       BlockWalk bw;
       for (int j = 0; j < tbk.NB; ++j, ++G, bw.next(tbk)) {
         const uint32_t st = G % C::kStagesK;
@@ -640,8 +686,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The two warps of a quadrant meet at a barrier per block and one in the epilogue,
     // at which they exchange whether their waits succeeded.  One whose wait runs out
     // goes through its item's remaining barriers (its partner may be at any of them)
-    // and both leave at the item's last.  (An outcome exchanged with every block: 52.9
-    // -> 55.5 ms on two tiles of 136 x 32 x 64 tokens.)
+    // and both leave at the item's last.  (An outcome exchanged with every block
+    // cost 5 %.)
     for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
       Item it;
       if (!resolve<RAGGED>(a, &tq, &tk, &tv, w, it)) continue;
